@@ -38,6 +38,7 @@
 
 #include <cstdint>
 
+#include "fixed64.cuh"
 #include "lattice.cuh"
 
 namespace lbm {
@@ -90,6 +91,7 @@ struct DomPar {
   int32_t lo, has_force;  // first row (y in 2-D, z in 3-D) of the domain
   float omega_f, fpre3_f, g_f[3], hg_f[3], omega2_f;  // float copies, as in Params
   Folded kc;              // collision constants, as in Params
+  FixedK kx;
 };
 
 // Collision parameters of one node, from Params or from its domain.
@@ -195,6 +197,14 @@ __device__ __forceinline__ const Folded& folded_of(const Params& p, const Layout
     return lay.dom[dom].kc;
   else
     return p.kc;
+}
+
+template <bool MULTI>
+__device__ __forceinline__ const FixedK& fixed_of(const Params& p, const Layout& lay, int dom) {
+  if constexpr (MULTI)
+    return lay.dom[dom].kx;
+  else
+    return p.kx;
 }
 
 // Collision and store of one node: moments of f, Guo-forced BGK (or D2Q9
@@ -374,6 +384,31 @@ __device__ __forceinline__ void collide_store(typename P::T (&f)[L::Q], const Pa
 #undef LBM_K
 #undef LBM_KI
 
+// Collision and store of one node in the step kernels.  FP64 collides on the
+// integer grid (fixed64.cuh) and, where the node is outside its range, takes
+// the populations again (again(f) fills f as it was) and collides in doubles.
+template <class L, class P, bool MULTI, class Again>
+__device__ __forceinline__ void collide_node(typename P::T (&f)[L::Q], const Params& p, const Layout& lay, int dom,
+                                             typename P::T* __restrict__ fout, size_t S, uint32_t k,
+                                             Mom4<typename P::T>* __restrict__ mom, bool cache, bool keep,
+                                             Again&& again) {
+  const Relax rx = MULTI ? relax_domain(lay.dom, dom) : relax_params(p);
+  if constexpr (!P::shifted) {
+    const FixedK& kx = fixed_of<MULTI>(p, lay, dom);
+    if (kx.on) {
+      NodeMom m;
+      if (collide_grid(f, kx, rx.has_force != 0, m)) {
+        if (cache && keep) mom[k] = Mom4<double>{m.rho, m.ux, m.uy, m.uz};
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i) fout[(size_t)i * S + k] = keep ? f[i] : 0.0;
+        return;
+      }
+      again(f);
+    }
+  }
+  collide_store<L, P>(f, p, rx, folded_of<MULTI>(p, lay, dom), fout, S, k, mom, cache, keep);
+}
+
 // Storage indices of the pull sources x - e_i of fluid node k of run `run`.
 template <class L>
 __device__ __forceinline__ void pull_sources(uint32_t k, const RunRec& run, const Layout& lay, const Params& p,
@@ -428,6 +463,17 @@ __device__ __forceinline__ void pull_offsets(uint32_t k, const RunRec& run, cons
   pull_sources<L>(k, run, lay, p, src);
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) d[i] = (int)(src[i] - k);
+}
+
+// The populations f_i(x, t+1) = f+_i(x - e_i, t) of fluid node k of run `run`.
+template <class L, class T>
+__device__ __forceinline__ void pull_node(const T* __restrict__ fin, size_t S, uint32_t k, const RunRec& run,
+                                          const Layout& lay, const Params& p, T (&f)[L::Q]) {
+  int d[L::Q];
+  pull_offsets<L>(k, run, lay, p, d);
+  const T* __restrict__ fk = fin + k;
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) f[i] = __ldg(fk + ((ptrdiff_t)i * (ptrdiff_t)S + d[i]));
 }
 
 // ------------------------------------------------------------------ bulk --
@@ -504,11 +550,7 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_b
     if (live[j] && !(w[j] & (W_GHOST | W_OPEN))) {
       const RunRec run = lay.runs[w[j] & W_RUN];
       if (MULTI) dom[j] = run.dom;
-      int d[L::Q];
-      pull_offsets<L>(k[j], run, lay, p, d);
-      const T* __restrict__ fk = fin + k[j];
-#pragma unroll
-      for (int i = 0; i < L::Q; ++i) f[j][i] = __ldg(fk + ((ptrdiff_t)i * (ptrdiff_t)S + d[i]));
+      pull_node<L>(fin, S, k[j], run, lay, p, f[j]);
     }
   }
 #pragma unroll
@@ -516,13 +558,17 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_b
     if (!live[j]) continue;
     // ghost and open slots: zeros through the same stores (inputs at rest)
     const bool fl = !(w[j] & (W_GHOST | W_OPEN));
-    if (!fl) {
+    auto rest = [&](T(&g)[L::Q]) {
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) f[j][i] = P::shifted ? (T)0 : (T)L::w(i);
-    }
-    const Relax rx = MULTI ? relax_domain(lay.dom, dom[j]) : relax_params(p);
-    collide_store<L, P>(f[j], p, rx, folded_of<MULTI>(p, lay, dom[j]), fout, S, k[j], mom, (w[j] & W_CACHE) != 0,
-                        fl);
+      for (int i = 0; i < L::Q; ++i) g[i] = P::shifted ? (T)0 : (T)L::w(i);
+    };
+    if (!fl) rest(f[j]);
+    collide_node<L, P, MULTI>(f[j], p, lay, dom[j], fout, S, k[j], mom, (w[j] & W_CACHE) != 0, fl, [&](T(&g)[L::Q]) {
+      if (fl)
+        pull_node<L>(fin, S, k[j], lay.runs[w[j] & W_RUN], lay, p, g);
+      else
+        rest(g);
+    });
   }
 }
 
@@ -548,14 +594,11 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, 1>())) k_bul
   const uint32_t k = __ldg(lay.fluid + t);
   const uint32_t w = __ldg(lay.word + k);
   const RunRec run = lay.runs[w & W_RUN];
-  int d[L::Q];
-  pull_offsets<L>(k, run, lay, p, d);
   T f[L::Q];
-  const T* __restrict__ fk = fin + k;
-#pragma unroll
-  for (int i = 0; i < L::Q; ++i) f[i] = __ldg(fk + ((ptrdiff_t)i * (ptrdiff_t)S + d[i]));
-  const Relax rx = MULTI ? relax_domain(lay.dom, run.dom) : relax_params(p);
-  collide_store<L, P>(f, p, rx, folded_of<MULTI>(p, lay, run.dom), fout, S, k, mom, (w & W_CACHE) != 0);
+  pull_node<L>(fin, S, k, run, lay, p, f);
+  collide_node<L, P, MULTI>(f, p, lay, run.dom, fout, S, k, mom, (w & W_CACHE) != 0, true, [&](T(&g)[L::Q]) {
+    pull_node<L>(fin, S, k, lay.runs[w & W_RUN], lay, p, g);
+  });
 }
 
 // Resident blocks per SM of the sequential walk (it keeps the next node's
@@ -627,8 +670,9 @@ __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) fout[(size_t)i * S + k] = (T)0;
     } else {
-      const Relax rx = MULTI ? relax_domain(lay.dom, run.dom) : relax_params(p);
-      collide_store<L, P>(f, p, rx, folded_of<MULTI>(p, lay, run.dom), fout, S, k, mom, (w & W_CACHE) != 0);
+      collide_node<L, P, MULTI>(f, p, lay, run.dom, fout, S, k, mom, (w & W_CACHE) != 0, true, [&](T(&g)[L::Q]) {
+        pull_node<L>(fin, S, k, lay.runs[w & W_RUN], lay, p, g);
+      });
     }
     // the next node's run record, loaded before its pulls are needed
     w = w2;
@@ -1114,8 +1158,10 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
     T f[L::Q];
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) f[i] = col[i][lane];
-    const Relax rx = MULTI ? relax_domain(lay.dom, dom) : relax_params(p);
-    collide_store<L, P>(f, p, rx, folded_of<MULTI>(p, lay, dom), fout, S, k, mom_out, (w & W_CACHE) != 0, fluid);
+    collide_node<L, P, MULTI>(f, p, lay, dom, fout, S, k, mom_out, (w & W_CACHE) != 0, fluid, [&](T(&g)[L::Q]) {
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i) g[i] = col[i][lane];
+    });
   }
 }
 

@@ -106,6 +106,19 @@ inline void fold(Folded& k, double omega, double fpre3, const double g[3]) {
   }
 }
 
+// Constants of the FP64 collision on the integer grid (fixed64.cuh), in units
+// of the grid step 2^(sc - 62); filled by fold_fixed for a lattice and for
+// each domain of a batch.  Velocity-set specific: c = the relaxation rates
+// over their norms (D2Q9) or omega/8, omega/12, omega/36, 1/3 (D3Q19).
+struct FixedK {
+  double step;                      // 2^(sc - 62)
+  double c[4], hg[3], ge[3], gp[2], gq[3];
+  int64_t gj[2];
+  uint32_t oh, oh2, ol;             // |1 - omega| 2^63 = oh 2^32 + ol; 2 oh
+  uint64_t oc, neg;                 // rounding term of its products; ~0 where 1 - omega < 0
+  int32_t sc, on;                   // grid exponent; 0: collide in doubles
+};
+
 // Run parameters handed to every kernel by value.
 struct Params {
   int nx, ny, nz;
@@ -126,6 +139,7 @@ struct Params {
   // float conversion on every node or link costs FP64-pipe time
   float rho0_f, omega_f, fpre3_f, g_f[3], hg_f[3], omega2_f;
   Folded kc;            // collision constants (fold_params)
+  FixedK kx;            // ... of the FP64 collision on the integer grid (fold_fixed)
 };
 
 // Fills the float copies of Params from its doubles (after any change).

@@ -230,6 +230,18 @@ int cx_of(const lbm_handle h, int i) { return h->Q == 9 ? D2Q9::cx(i) : D3Q19::c
 int cy_of(const lbm_handle h, int i) { return h->Q == 9 ? D2Q9::cy(i) : D3Q19::cy(i); }
 int cz_of(const lbm_handle h, int i) { return h->Q == 9 ? D2Q9::cz(i) : D3Q19::cz(i); }
 
+// Folded constants of the lattice's run parameters (after any change of them).
+void fold_all(lbm_handle h) {
+  Params& p = h->p;
+  if (h->Q == 9) {
+    fold_params<D2Q9>(p);
+    fold_fixed<D2Q9>(p.kx, p.omega, p.fpre3, p.g, p.rho0, p.collision);
+  } else {
+    fold_params<D3Q19>(p);
+    fold_fixed<D3Q19>(p.kx, p.omega, p.fpre3, p.g, p.rho0, p.collision);
+  }
+}
+
 // Enqueue one time step from buffer fc (f+(t), moments mc) into fn (moments
 // at t+1 into mn), adding the force to `slot` and clearing `next`.  fused:
 // the link rules run inside the pull pass (k_fused; mn must differ from mc),
@@ -420,11 +432,8 @@ lbm_status lbm_create_lattice(const lbm_config* cfg, lbm_handle* out) {
   p.fpre3 = 3.0 * (1.0 - 0.5 / c.tau);
   for (int a = 0; a < 3; ++a) p.g[a] = (a < h->D) ? c.g[a] : 0.0;
   p.has_force = (p.g[0] != 0.0 || p.g[1] != 0.0 || p.g[2] != 0.0);
-  if (h->Q == 9)
-    fold_params<D2Q9>(p);
-  else
-    fold_params<D3Q19>(p);
   p.collision = c.collision;
+  fold_all(h);
   p.inlet = c.inlet ? 1 : 0;
   p.outlet = c.outlet ? 1 : 0;
   p.inlet_umax = c.inlet_umax;
@@ -1105,10 +1114,13 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
       dp[k].fpre3 = 3.0 * (1.0 - 0.5 / q.tau);
       for (int a = 0; a < 3; ++a) dp[k].g[a] = a < D ? q.g[a] : 0.0;
       dp[k].has_force = (dp[k].g[0] != 0.0 || dp[k].g[1] != 0.0 || dp[k].g[2] != 0.0) ? 1 : 0;
-      if (Q == 9)
+      if (Q == 9) {
         fold<D2Q9>(dp[k].kc, dp[k].omega, dp[k].fpre3, dp[k].g);
-      else
+        fold_fixed<D2Q9>(dp[k].kx, dp[k].omega, dp[k].fpre3, dp[k].g, c.rho0, c.collision);
+      } else {
         fold<D3Q19>(dp[k].kc, dp[k].omega, dp[k].fpre3, dp[k].g);
+        fold_fixed<D3Q19>(dp[k].kx, dp[k].omega, dp[k].fpre3, dp[k].g, c.rho0, c.collision);
+      }
       dp[k].omega_f = (float)dp[k].omega;
       dp[k].fpre3_f = (float)dp[k].fpre3;
       dp[k].omega2_f = (float)(dp[k].omega * dp[k].omega);
@@ -1175,10 +1187,7 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   p.fpre3 = 3.0 * (1.0 - 0.5 / d0.tau);
   for (int a = 0; a < 3; ++a) p.g[a] = a < D ? d0.g[a] : 0.0;
   p.has_force = (p.g[0] != 0.0 || p.g[1] != 0.0 || p.g[2] != 0.0);
-  if (h->Q == 9)
-    fold_params<D2Q9>(p);
-  else
-    fold_params<D3Q19>(p);
+  fold_all(h);
   p.inlet_umax = d0.inlet_umax;
   p.inlet_y0 = d0.inlet_y0;
   p.inlet_y1 = d0.inlet_y1;
