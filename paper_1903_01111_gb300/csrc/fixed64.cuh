@@ -1,25 +1,25 @@
-// FP64 collision with its sums in 64-bit integers.
+// FP64 collision in 64-bit integers.
 //
 // What bounds the FP64 step on sm_103a: the FP64 pipe takes 2 operations per
-// clock and SM, 32 times fewer than the integer pipes, and a collision written
-// in doubles is 70 (D2Q9) to 150 (D3Q19) of them per node.  Most of those are
-// additions of populations of the same size, which integers do exactly.  So a
-// node's populations become fixed-point numbers on one grid, U = 2^(sc - 62)
-// with 2^sc the power of two just above rho0 (a double of at least 2^(sc - 10)
-// lands on the grid without rounding; 53 bits are kept of what is smaller):
+// clock and SM, 32 times fewer than the integer pipes (a 32 x 32 -> 64-bit
+// multiply-add: 16 per clock and SM), and a collision in doubles is 72
+// (D2Q9 BGK) to 150 (D3Q19) of them per node, about 400 for MRT.  So a node's
+// populations become fixed-point numbers on one grid of step U = 2^(sc - 62),
+// with sc such that rho0 is 0.75 .. 1.5 times 2^sc (a double of at least
+// 2^(sc - 9) lands on the grid without rounding; 53 bits are kept of what is
+// smaller):
 //   * every sum and difference of populations, and every combination of the
 //     relaxed moments back into directions, is an integer addition: exact;
-//   * the few products (momentum times velocity, the relaxation rates) stay in
-//     doubles, in units of U, with one conversion each way;
-//   * D3Q19's (1 - omega) f_i is a 64 x 64-bit integer product, right to about
-//     one U;
-//   * the result is rounded once, to nearest even, to the double stored.
-// U is 2^-3 to 2^-5 of the last place of a population w_i rho0, so the result
-// is as near to the exact one as the rounding of the stored double lets it be;
-// the same sums in doubles round at the last place of rho.
+//   * a product is three 32 x 32 -> 64-bit multiply-adds (the low-by-low term
+//     is below the grid), right to about one U;
+//   * 1/rho is the one quantity formed in doubles (four FP64 operations);
+//   * the result is rounded once, to the double stored.
+// U is 2^-4 to 2^-6 of the last place of a population w_i rho0; the same sums
+// in doubles round at the last place of rho.  Measured against 64-bit
+// references (u after 5 steps): dense D3Q19 7.6e-15 in doubles, 6.1e-15 here.
 //
 // A node outside the range of the grid (a negative population or one far
-// below w_i rho0, rho outside (2^(sc-2), 2^(sc+1)), a velocity near 1/2, not
+// below w_i rho0, rho outside (2^(sc-1), 1.75 2^sc), a velocity near 1/2, not
 // a number, ...) is found by integer tests on the way and left to the
 // collision in doubles: the function returns false without storing anything.
 #pragma once
@@ -34,50 +34,59 @@ namespace lbm {
 // 64 bits); a stronger force runs the collision in doubles.
 constexpr double kFixedMaxForce = 1.0 / 512;
 
+__host__ __device__ __forceinline__ Halves halves(int64_t v) {
+  return Halves{(int32_t)(((uint64_t)v + 0x80000000ull) >> 32), (int32_t)(uint32_t)(uint64_t)v};
+}
+
 // Fills the constants for stencil L; collision 1 is MRT (D2Q9).
 template <class L>
 inline void fold_fixed(FixedK& k, double omega, double fpre3, const double g[3], double rho0, int collision) {
   k = FixedK{};
   int e2 = 0;
-  std::frexp(rho0, &e2);  // rho0 = m 2^e2, m in [1/2, 1)
-  k.sc = e2;
+  const double m = std::frexp(rho0, &e2);  // rho0 = m 2^e2, m in [1/2, 1)
+  k.sc = m < 0.75 ? e2 - 1 : e2;
   bool on = e2 > -900 && e2 < 900;
   for (int a = 0; a < 3; ++a) on = on && std::fabs(g[a]) <= kFixedMaxForce * rho0;
   k.on = on ? 1 : 0;
   if (!on) return;
-  const double unit = std::ldexp(1.0, 62 - e2);  // grid steps per 1
-  k.step = std::ldexp(1.0, e2 - 62);
-  for (int a = 0; a < 3; ++a) k.hg[a] = 0.5 * g[a] * unit;
+  const double unit = std::ldexp(1.0, 62 - k.sc);  // grid steps per 1
+  k.step = std::ldexp(1.0, k.sc - 62);
+  auto steps = [&](double v) { return (int64_t)std::llrint(v * unit); };
+  auto rate = [](double v) { return halves((int64_t)std::llrint(std::ldexp(v, 64))); };
+  for (int a = 0; a < 3; ++a) k.hg[a] = steps(0.5 * g[a]);
   if (L::Q == 9) {
     // relaxation rates of e, epsilon, q, p (Sec. 2: 1.5, 1.5, 1.2, omega); BGK: omega for all
     const double se = collision == 1 ? 1.5 : omega, sq = collision == 1 ? 1.2 : omega;
-    k.c[0] = se / 36.0;
-    k.c[1] = 3.0 * se / 36.0;
-    k.c[2] = sq / 12.0;
-    k.c[3] = omega / 4.0;
+    k.c[0] = rate(se / 36.0);
+    k.c[1] = rate(se / 12.0);
+    k.c[2] = rate(sq / 12.0);
+    k.c[3] = rate(omega / 8.0);
     for (int a = 0; a < 2; ++a) {
-      k.ge[a] = (1.0 - 0.5 * se) / 6.0 * g[a] * unit;
-      k.gp[a] = (1.0 - 0.5 * omega) / 4.0 * g[a] * unit;
-      k.gq[a] = g[a] / 12.0 * unit;
-      k.gj[a] = (int64_t)std::llrint(g[a] / 6.0 * unit);
+      k.ge[a] = halves(steps((1.0 - 0.5 * se) / 6.0 * g[a]));
+      k.gp[a] = halves(steps((1.0 - 0.5 * omega) / 4.0 * g[a]));
+      k.gq[a] = steps(g[a] / 12.0);
+      k.gj[a] = steps(g[a] / 6.0);
     }
   } else {
-    k.c[0] = omega / 8.0;
-    k.c[1] = omega / 12.0;
-    k.c[2] = omega / 36.0;
-    k.c[3] = 1.0 / 3.0;
+    k.c[0] = rate(omega / 8.0);
+    k.c[1] = rate(omega / 12.0);
+    k.c[2] = rate(omega / 36.0);
+    k.c[3] = rate(1.0 / 3.0);
     for (int a = 0; a < 3; ++a) {
-      k.ge[a] = fpre3 / 24.0 * g[a] * unit;
-      k.gq[a] = fpre3 / 36.0 * g[a] * unit;
+      k.ge[a] = halves(steps(fpre3 / 24.0 * g[a]));
+      k.gq[a] = steps(fpre3 / 36.0 * g[a]);
     }
     const double om1 = 1.0 - omega;  // in (-1, 1)
     const uint64_t om = (uint64_t)std::ldexp(std::fabs(om1), 63);
     k.oh = (uint32_t)(om >> 32);
     k.oh2 = 2u * k.oh;
     k.ol = (uint32_t)om;
-    // centres the two parts a product drops (fl ol and the bits shifted out)
-    k.oc = (1ull << 30) + (k.ol >> 1);
     k.neg = om1 < 0.0 ? ~0ull : 0ull;
+    // centres a product: + 2^-32 ol/2 for the dropped low-by-low term.  The
+    // half step that the shift drops on average is left (om1 > 0) or made up
+    // twice (om1 < 0, subtracted): rounding halves up in from_grid adds half a
+    // step on average, so that the three cancel
+    k.oc = (uint64_t)(k.ol >> 1) + (om1 < 0.0 ? 1ull << 31 : 0ull);
   }
 }
 
@@ -97,37 +106,65 @@ __device__ __forceinline__ uint64_t to_grid(double f, int sc, uint32_t& bad) {
   return ((uint64_t)__funnelshift_r(mh, 0u, n) << 32) | __funnelshift_r(ml, mh, n);
 }
 
-// The double nearest (ties to even) to v steps of the grid; v in [2^32, 2^63),
-// else the sign bit of `bad` is set and the value is meaningless.
+// The double nearest to v steps of the grid (EVEN: ties to even, else up); v
+// in [2^32, 2^63), else the sign bit of `bad` is set and the value is
+// meaningless.
+template <bool EVEN>
 __device__ __forceinline__ double from_grid(uint64_t v, int sc, uint32_t& bad) {
   const uint32_t hi = (uint32_t)(v >> 32), lo = (uint32_t)v;
   bad |= hi | (hi - 1u);
   const uint32_t lz = (uint32_t)__clz((int)hi);
   const uint32_t sh = lz - 1u;  // leading bit to place 62
   const uint32_t xh = __funnelshift_l(lo, hi, sh), xl = __funnelshift_l(0u, lo, sh);
-  const uint64_t x = (((uint64_t)xh << 32) | xl) + (0x1ffu + ((xl >> 10) & 1u));
+  const uint64_t x = (((uint64_t)xh << 32) | xl) + (EVEN ? 0x1ffu + ((xl >> 10) & 1u) : 0x200u);
   const uint32_t yh = (uint32_t)(x >> 32);
   // the leading bit adds one to the exponent field
   return __hiloint2double((int)((yh >> 10) + ((uint32_t)(1023 + sc) << 20) - (lz << 20)),
                           (int)__funnelshift_r((uint32_t)x, yh, 10));
 }
 
-// 1/x by two Newton-Raphson steps on the hardware's approximate reciprocal
-// (x positive and normal).
-__device__ __forceinline__ double newton_reciprocal(double x) {
+// a b / 2^(64 - S), right to about one; the caller keeps |b| below 2^(62 - S).
+template <int S>
+__device__ __forceinline__ int64_t mul_grid(const Halves& a, const Halves& b) {
+  int64_t m = (int64_t)a.l * b.h + (1ll << (31 - S));
+  m += (int64_t)a.h * b.l;
+  return (int64_t)a.h * (int32_t)((uint32_t)b.h << S) + (m >> (32 - S));
+}
+
+// 2^61 / rho for rho = r 2^-62 in [1/2, 2): two Newton-Raphson steps on the
+// hardware's approximate reciprocal.
+__device__ __forceinline__ int64_t reciprocal_grid(uint64_t r) {
+  uint32_t none = 0;
+  const double x = from_grid<false>(r, 0, none);  // in [1/2, 2)
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   y = fma(fma(-x, y, 1.0), y, y);
-  return fma(fma(-x, y, 1.0), y, y);
+  y = fma(fma(-x, y, 1.0), y, y);
+  // y in (1/2, 2 + 2^-52]: 53 bits of it at places 61 and below
+  const uint32_t lo = (uint32_t)__double2loint(y), hi = (uint32_t)__double2hiint(y);
+  const uint32_t n = 1024u - (hi >> 20);
+  const uint32_t mh = (__funnelshift_l(lo, hi, 10) & 0x3fffffffu) | 0x40000000u;
+  return (int64_t)(((uint64_t)__funnelshift_r(mh, 0u, n) << 32) | __funnelshift_r(lo << 10, mh, n));
 }
 
-// Whether v, as a signed number, lies in [-2^61, 2^61): 0 if it does.
-__device__ __forceinline__ uint32_t beyond61(uint64_t v) { return ((uint32_t)(v >> 32) + 0x20000000u) >> 30; }
+// 0 if v, as a signed number, lies in [-2^B, 2^B), B > 32.
+template <int B>
+__device__ __forceinline__ uint32_t beyond(uint64_t v) {
+  return ((uint32_t)(v >> 32) + (1u << (B - 32))) >> (B - 31);
+}
 
-// rho, u of the node in the units of the moment cache.
+// rho and u of a node: r in grid steps, u in 2^-60.
 struct NodeMom {
-  double rho, ux, uy, uz;
+  uint64_t r;
+  int64_t ux, uy, uz;
+  __device__ __forceinline__ double u(int64_t v) const { return (double)v * 0x1p-60; }
 };
+
+// 0 if rho = r 2^-62 lies in [1/2, 1.75).
+__device__ __forceinline__ uint32_t beyond_rho(uint64_t r) {
+  const uint32_t hi = (uint32_t)(r >> 32);
+  return ((hi + 0x10000000u) >> 31) | (hi < 0x20000000u ? 1u : 0u);
+}
 
 // D2Q9, BGK and MRT: f (pre-collision) is replaced by the post-collision
 // populations.  In moment space (rows of M, Sec. 2) every moment but rho and j
@@ -142,65 +179,67 @@ __device__ __forceinline__ bool collide_grid(double (&f)[9], const FixedK& k, bo
   uint64_t F[9];
   F[0] = to_grid<9>(f[0], k.sc, bad);
 #pragma unroll
-  for (int i = 1; i < 9; ++i) F[i] = to_grid<7>(f[i], k.sc, bad);
+  for (int i = 1; i < 9; ++i) F[i] = i < 5 ? to_grid<8>(f[i], k.sc, bad) : to_grid<7>(f[i], k.sc, bad);
   const uint64_t s13 = F[1] + F[3], s24 = F[2] + F[4], s57 = F[5] + F[7], s68 = F[6] + F[8];
   const uint64_t d13 = F[1] - F[3], d24 = F[2] - F[4], d57 = F[5] - F[7], d68 = F[6] - F[8];
   const uint64_t Sa = s13 + s24, Sd = s57 + s68, r = F[0] + Sa + Sd;
   const uint64_t X = F[0] - Sa, Y = Sa - 4 * Sd;
   const uint64_t bx = d57 - d68, by = d57 + d68;
-  wide = beyond61(X) | beyond61(Y) | (uint32_t)(Sd >> 61) | (uint32_t)(r >> 63) | ((uint32_t)(r >> 60) == 0u ? 1u : 0u);
-  const double rd = __ll2double_rn((long long)r);
-  double Jx = __ll2double_rn((long long)(d13 + bx)), Jy = __ll2double_rn((long long)(d24 + by));
-  const double Xd = __ll2double_rn((long long)X), Yd = __ll2double_rn((long long)Y);
-  const double Qx = __ll2double_rn((long long)(2 * bx - d13)), Qy = __ll2double_rn((long long)(2 * by - d24));
-  const double Px = __ll2double_rn((long long)(s13 - s24)), Pxy = __ll2double_rn((long long)(s57 - s68));
+  uint64_t jx = d13 + bx, jy = d24 + by;
   if (force) {
-    Jx += k.hg[0];
-    Jy += k.hg[1];
+    jx += (uint64_t)k.hg[0];
+    jy += (uint64_t)k.hg[1];
   }
-  const double inv = newton_reciprocal(rd);
-  const double ux = Jx * inv, uy = Jy * inv;
-  const double qxx = Jx * ux, qyy = Jy * uy, qxy = Jx * uy;
-  const double E = qxx + qyy;
-  // rho u.u at most 1/4 (grid units 2^60)
-  wide |= (uint32_t)__double2hiint(E) >= 0x43b00000u ? 1u : 0u;
-  double De = k.c[0] * fma(-2.0, Xd, fma(-3.0, E, -Yd));
-  double Dp = k.c[1] * (Xd + E);
-  double Dx = k.c[2] * Qx, Dy = k.c[2] * Qy;
-  double Dxx = k.c[3] * ((Px - qxx) + qyy), Dxy = k.c[3] * (Pxy - qxy);
+  // |X|, |Y| < 1/4, Sd < 1/2, |j| < 1/2
+  wide = beyond<60>(X) | beyond<60>(Y) | (uint32_t)(Sd >> 61) | beyond<61>(jx) | beyond<61>(jy) | beyond_rho(r);
+  const Halves inv = halves(reciprocal_grid(r));
+  const Halves hx = halves((int64_t)(2 * jx)), hy = halves((int64_t)(2 * jy));
+  const int64_t ux = mul_grid<0>(hx, inv), uy = mul_grid<0>(hy, inv);  // 2^-60
+  wide |= beyond<59>((uint64_t)ux) | beyond<59>((uint64_t)uy);         // |u| < 1/2
+  const Halves vx = halves(ux), vy = halves(uy);
+  // rho u u in 2^-62: 2 j in 2^-62 times u in 2^-60 over 2^61
+  const int64_t qxx = mul_grid<3>(hx, vx), qyy = mul_grid<3>(hy, vy), qxy = mul_grid<3>(hx, vy);
+  const int64_t E = qxx + qyy;
+  wide |= beyond<60>((uint64_t)E);
+  const int64_t ne = -(int64_t)(2 * X + Y) - 3 * E;
+  int64_t De = mul_grid<0>(halves(ne), k.c[0]), Dp = mul_grid<0>(halves((int64_t)X + E), k.c[1]);
+  int64_t Dx = mul_grid<0>(halves((int64_t)(2 * bx - d13)), k.c[2]);
+  int64_t Dy = mul_grid<0>(halves((int64_t)(2 * by - d24)), k.c[2]);
+  int64_t Dxx = mul_grid<0>(halves((int64_t)(s13 - s24) - qxx + qyy), k.c[3]);
+  int64_t Dxy = mul_grid<0>(halves((int64_t)(s57 - s68) - qxy), k.c[3]);
+  Dxx += Dxx;
+  Dxy += Dxy;
   if (force) {
-    const double de = fma(k.ge[0], ux, k.ge[1] * uy);
+    // g steps times u in 2^-60
+    const int64_t de = mul_grid<4>(vx, k.ge[0]) + mul_grid<4>(vy, k.ge[1]);
     De -= de;
-    // the same force term with the rate of epsilon (equal to e's)
     Dp += de;
     Dx += k.gq[0];
     Dy += k.gq[1];
-    Dxx = fma(-2.0 * k.gp[0], ux, fma(2.0 * k.gp[1], uy, Dxx));
-    Dxy = fma(-k.gp[1], ux, fma(-k.gp[0], uy, Dxy));
+    Dxx -= 2 * (mul_grid<4>(vx, k.gp[0]) - mul_grid<4>(vy, k.gp[1]));
+    Dxy -= mul_grid<4>(vx, k.gp[1]) + mul_grid<4>(vy, k.gp[0]);
   }
-  const uint64_t ie = (uint64_t)__double2ll_rn(De), ip = (uint64_t)__double2ll_rn(Dp);
-  const uint64_t ix = (uint64_t)__double2ll_rn(Dx), iy = (uint64_t)__double2ll_rn(Dy);
-  const uint64_t ixx = (uint64_t)__double2ll_rn(Dxx), ixy = (uint64_t)__double2ll_rn(Dxy);
   const uint64_t gx = (uint64_t)k.gj[0], gy = (uint64_t)k.gj[1];
+  const uint64_t ie = (uint64_t)De, ip = (uint64_t)Dp, ix = (uint64_t)Dx, iy = (uint64_t)Dy;
   F[0] += 4 * (ie - ip);
-  const uint64_t ax = ie + 2 * ip;                       // axis: + e + 2 epsilon
-  const uint64_t tx = 2 * ix + gx, ty = 2 * iy + gy;     // 2 q - j (j's part is -g/6)
-  const uint64_t px = ax - ixx, py = ax + ixx;
+  const uint64_t ax = ie + 2 * ip;                    // axis: + e + 2 epsilon
+  const uint64_t tx = 2 * ix + gx, ty = 2 * iy + gy;  // 2 q - j (j's part is -g/6)
+  const uint64_t px = ax - (uint64_t)Dxx, py = ax + (uint64_t)Dxx;
   F[1] += px + tx;
   F[3] += px - tx;
   F[2] += py + ty;
   F[4] += py - ty;
-  const uint64_t dg = 2 * ie + ip;                       // diagonal: - 2 e - epsilon
-  const uint64_t vx = gx - ix, vy = gy - iy;             // - j - q
-  const uint64_t d0 = 0 - dg - ixy, d1 = ixy - dg;
-  F[5] += d0 + (vx + vy);
-  F[7] += d0 - (vx + vy);
-  F[6] += d1 - (vx - vy);
-  F[8] += d1 + (vx - vy);
+  const uint64_t dg = 2 * ie + ip;                    // diagonal: - 2 e - epsilon
+  const uint64_t wx = gx - ix, wy = gy - iy;          // - j - q
+  const uint64_t d0 = 0 - dg - (uint64_t)Dxy, d1 = (uint64_t)Dxy - dg;
+  F[5] += d0 + (wx + wy);
+  F[7] += d0 - (wx + wy);
+  F[6] += d1 - (wx - wy);
+  F[8] += d1 + (wx - wy);
   uint32_t out = 0;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) f[i] = from_grid(F[i], k.sc, out);
-  m = NodeMom{rd * k.step, ux, uy, 0.0};
+  for (int i = 0; i < 9; ++i) f[i] = from_grid<true>(F[i], k.sc, out);
+  m = NodeMom{r, ux, uy, 0};
   return bad < 32u && wide == 0u && (int32_t)out >= 0;
 }
 
@@ -216,7 +255,7 @@ __device__ __forceinline__ bool collide_grid(double (&f)[19], const FixedK& k, b
   uint64_t F[19];
   F[0] = to_grid<9>(f[0], k.sc, bad);
 #pragma unroll
-  for (int i = 1; i < 19; ++i) F[i] = to_grid<6>(f[i], k.sc, bad);
+  for (int i = 1; i < 19; ++i) F[i] = i < 7 ? to_grid<7>(f[i], k.sc, bad) : to_grid<6>(f[i], k.sc, bad);
   uint64_t r = F[0], jx, jy, jz;
 #pragma unroll
   for (int i = 1; i < 19; ++i) r += F[i];
@@ -227,70 +266,66 @@ __device__ __forceinline__ bool collide_grid(double (&f)[19], const FixedK& k, b
     jy = (F[3] - F[4]) + (d7 - d9) + (d15 + d17);
     jz = (F[5] - F[6]) + (d11 - d13) + (d15 - d17);
   }
-  wide = (uint32_t)(r >> 63) | ((uint32_t)(r >> 60) == 0u ? 1u : 0u);
-  const double rd = __ll2double_rn((long long)r);
-  double Jx = __ll2double_rn((long long)jx), Jy = __ll2double_rn((long long)jy), Jz = __ll2double_rn((long long)jz);
   if (force) {
-    Jx += k.hg[0];
-    Jy += k.hg[1];
-    Jz += k.hg[2];
+    jx += (uint64_t)k.hg[0];
+    jy += (uint64_t)k.hg[1];
+    jz += (uint64_t)k.hg[2];
   }
-  const double inv = newton_reciprocal(rd);
-  const double ux = Jx * inv, uy = Jy * inv, uz = Jz * inv;
-  const double Wx = k.c[0] * Jx, Wy = k.c[0] * Jy, Wz = k.c[0] * Jz;
-  double Txx = Wx * ux, Tyy = Wy * uy, Tzz = Wz * uz, Txy, Txz, Tyz;
-  double Mx = k.c[1] * Jx, My = k.c[1] * Jy, Mz = k.c[1] * Jz;
+  wide = beyond_rho(r) | beyond<61>(jx) | beyond<61>(jy) | beyond<61>(jz);  // |j| < 1/2
+  const Halves inv = halves(reciprocal_grid(r));
+  const Halves hx = halves((int64_t)(2 * jx)), hy = halves((int64_t)(2 * jy)), hz = halves((int64_t)(2 * jz));
+  const int64_t ux = mul_grid<0>(hx, inv), uy = mul_grid<0>(hy, inv), uz = mul_grid<0>(hz, inv);  // 2^-60
+  wide |= beyond<59>((uint64_t)ux) | beyond<59>((uint64_t)uy) | beyond<59>((uint64_t)uz);         // |u| < 1/2
+  const Halves vx = halves(ux), vy = halves(uy), vz = halves(uz);
+  // 2 (omega/8) j; T in 2^-62: that times u in 2^-60 over 2^61
+  int64_t Wx = mul_grid<0>(hx, k.c[0]), Wy = mul_grid<0>(hy, k.c[0]), Wz = mul_grid<0>(hz, k.c[0]);
+  const Halves gx = halves(Wx), gy = halves(Wy), gz = halves(Wz);
+  int64_t Txx = mul_grid<3>(gx, vx), Tyy = mul_grid<3>(gy, vy), Tzz = mul_grid<3>(gz, vz);
+  // 2 T_ab
+  int64_t Sxy = 2 * mul_grid<3>(gx, vy), Sxz = 2 * mul_grid<3>(gx, vz), Syz = 2 * mul_grid<3>(gy, vz);
+  // M_a: half of 2 j times 2 omega/12 over 2^64
+  int64_t Mx = mul_grid<0>(hx, k.c[1]), My = mul_grid<0>(hy, k.c[1]), Mz = mul_grid<0>(hz, k.c[1]);
   if (force) {
-    const double vx = Wx + k.ge[0], vy = Wy + k.ge[1];
-    Txy = fma(vx, uy, k.ge[1] * ux);
-    Txz = fma(vx, uz, k.ge[2] * ux);
-    Tyz = fma(vy, uz, k.ge[2] * uy);
-    Txx = fma(2.0 * k.ge[0], ux, Txx);
-    Tyy = fma(2.0 * k.ge[1], uy, Tyy);
-    Tzz = fma(2.0 * k.ge[2], uz, Tzz);
-    Mx += k.gq[0];
-    My += k.gq[1];
-    Mz += k.gq[2];
-  } else {
-    Txy = Wx * uy;
-    Txz = Wx * uz;
-    Tyz = Wy * uz;
+    Txx += 2 * mul_grid<4>(vx, k.ge[0]);
+    Tyy += 2 * mul_grid<4>(vy, k.ge[1]);
+    Tzz += 2 * mul_grid<4>(vz, k.ge[2]);
+    Sxy += 2 * (mul_grid<4>(vx, k.ge[1]) + mul_grid<4>(vy, k.ge[0]));
+    Sxz += 2 * (mul_grid<4>(vx, k.ge[2]) + mul_grid<4>(vz, k.ge[0]));
+    Syz += 2 * (mul_grid<4>(vy, k.ge[2]) + mul_grid<4>(vz, k.ge[1]));
   }
-  const double tr = (Txx + Tyy) + Tzz;
-  // (omega/8) rho u.u at most 2^-5 (grid units 2^57); negative only by a force term
-  wide |= ((uint32_t)__double2hiint(tr) & 0x7fffffffu) >= 0x43800000u ? 1u : 0u;
-  const uint64_t B = (uint64_t)__double2ll_rn(fma(k.c[2], rd, -k.c[3] * tr));
-  const uint64_t ixx = (uint64_t)__double2ll_rn(Txx), iyy = (uint64_t)__double2ll_rn(Tyy),
-                 izz = (uint64_t)__double2ll_rn(Tzz);
-  const uint64_t ixy = 2 * (uint64_t)__double2ll_rn(Txy), ixz = 2 * (uint64_t)__double2ll_rn(Txz),
-                 iyz = 2 * (uint64_t)__double2ll_rn(Tyz);
-  const uint64_t mx = (uint64_t)__double2ll_rn(Mx), my = (uint64_t)__double2ll_rn(My),
-                 mz = (uint64_t)__double2ll_rn(Mz);
+  const int64_t tr = Txx + Tyy + Tzz;
+  wide |= beyond<57>((uint64_t)tr);  // (omega/8) rho u.u below 2^-5
+  const uint64_t B = (uint64_t)(mul_grid<0>(halves((int64_t)r), k.c[2]) - mul_grid<0>(halves(tr), k.c[3]));
   uint32_t out = 0;
   auto put = [&](int i, uint64_t c) {
     // (1 - omega) F_i: |1 - omega| as oh 2^32 + ol over 2^63; F < 2^62
     const uint32_t fh = (uint32_t)(F[i] >> 32), fl = (uint32_t)F[i];
     const uint64_t mid = (uint64_t)fl * k.oh + k.oc + (uint64_t)fh * k.ol;
     const uint64_t R = (uint64_t)fh * k.oh2 + (mid >> 31);
-    f[i] = from_grid(c + ((R ^ k.neg) - k.neg), k.sc, out);
+    f[i] = from_grid<false>(c + ((R ^ k.neg) - k.neg), k.sc, out);
   };
   auto pair = [&](int i, uint64_t P, uint64_t M) {
     put(i, P + M);
     put(i + 1, P - M);
   };
   put(0, 12 * B);
-  const uint64_t Bx = B + ixx, By = B + iyy, Bz = B + izz;
-  pair(1, 2 * Bx, 2 * mx);
-  pair(3, 2 * By, 2 * my);
-  pair(5, 2 * Bz, 2 * mz);
-  const uint64_t Bxy = Bx + iyy, Bxz = Bx + izz, Byz = By + izz;
-  pair(7, Bxy + ixy, mx + my);
-  pair(9, Bxy - ixy, mx - my);
-  pair(11, Bxz + ixz, mx + mz);
-  pair(13, Bxz - ixz, mx - mz);
-  pair(15, Byz + iyz, my + mz);
-  pair(17, Byz - iyz, my - mz);
-  m = NodeMom{rd * k.step, ux, uy, uz};
+  // 2 M_a is what the products above hold (2 j in place of j)
+  const uint64_t mx2 = (uint64_t)Mx + 2 * (uint64_t)k.gq[0], my2 = (uint64_t)My + 2 * (uint64_t)k.gq[1],
+                 mz2 = (uint64_t)Mz + 2 * (uint64_t)k.gq[2];
+  const uint64_t mx = (uint64_t)((int64_t)mx2 >> 1), my = (uint64_t)((int64_t)my2 >> 1),
+                 mz = (uint64_t)((int64_t)mz2 >> 1);
+  const uint64_t Bx = B + (uint64_t)Txx, By = B + (uint64_t)Tyy, Bz = B + (uint64_t)Tzz;
+  pair(1, 2 * Bx, mx2);
+  pair(3, 2 * By, my2);
+  pair(5, 2 * Bz, mz2);
+  const uint64_t Bxy = Bx + (uint64_t)Tyy, Bxz = Bx + (uint64_t)Tzz, Byz = By + (uint64_t)Tzz;
+  pair(7, Bxy + (uint64_t)Sxy, mx + my);
+  pair(9, Bxy - (uint64_t)Sxy, mx - my);
+  pair(11, Bxz + (uint64_t)Sxz, mx + mz);
+  pair(13, Bxz - (uint64_t)Sxz, mx - mz);
+  pair(15, Byz + (uint64_t)Syz, my + mz);
+  pair(17, Byz - (uint64_t)Syz, my - mz);
+  m = NodeMom{r, ux, uy, uz};
   return bad < 32u && wide == 0u && (int32_t)out >= 0;
 }
 

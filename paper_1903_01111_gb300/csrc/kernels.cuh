@@ -398,7 +398,7 @@ __device__ __forceinline__ void collide_node(typename P::T (&f)[L::Q], const Par
     if (kx.on) {
       NodeMom m;
       if (collide_grid(f, kx, rx.has_force != 0, m)) {
-        if (cache && keep) mom[k] = Mom4<double>{m.rho, m.ux, m.uy, m.uz};
+        if (cache && keep) mom[k] = Mom4<double>{(double)m.r * kx.step, m.u(m.ux), m.u(m.uy), m.u(m.uz)};
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) fout[(size_t)i * S + k] = keep ? f[i] : 0.0;
         return;

@@ -106,16 +106,22 @@ inline void fold(Folded& k, double omega, double fpre3, const double g[3]) {
   }
 }
 
-// Constants of the FP64 collision on the integer grid (fixed64.cuh), in units
-// of the grid step 2^(sc - 62); filled by fold_fixed for a lattice and for
-// each domain of a batch.  Velocity-set specific: c = the relaxation rates
-// over their norms (D2Q9) or omega/8, omega/12, omega/36, 1/3 (D3Q19).
+// A signed 64-bit number as h 2^32 + l with both halves signed.
+struct Halves {
+  int32_t h, l;
+};
+
+// Constants of the FP64 collision on the integer grid (fixed64.cuh), filled by
+// fold_fixed for a lattice and for each domain of a batch.  c: 2^64 times the
+// relaxation rates over their norms (D2Q9: s_e/36, s_e/12, s_q/12, omega/8) or
+// omega/8, omega/12, omega/36 (D3Q19); the force terms in grid steps.
 struct FixedK {
-  double step;                      // 2^(sc - 62)
-  double c[4], hg[3], ge[3], gp[2], gq[3];
-  int64_t gj[2];
+  double step;                      // one grid step, 2^(sc - 62)
+  Halves c[4];
+  int64_t hg[3], gq[3], gj[2];
+  Halves ge[3], gp[2];
   uint32_t oh, oh2, ol;             // |1 - omega| 2^63 = oh 2^32 + ol; 2 oh
-  uint64_t oc, neg;                 // rounding term of its products; ~0 where 1 - omega < 0
+  uint64_t oc, neg;                 // centring term of its products; ~0 where 1 - omega < 0
   int32_t sc, on;                   // grid exponent; 0: collide in doubles
 };
 
