@@ -83,10 +83,10 @@ inline void fold_fixed(FixedK& k, double omega, double fpre3, const double g[3],
     k.ol = (uint32_t)om;
     k.neg = om1 < 0.0 ? ~0ull : 0ull;
     // centres a product: + 2^-32 ol/2 for the dropped low-by-low term.  The
-    // half step that the shift drops on average is left (om1 > 0) or made up
-    // twice (om1 < 0, subtracted): rounding halves up in from_grid adds half a
-    // step on average, so that the three cancel
-    k.oc = (uint64_t)(k.ol >> 1) + (om1 < 0.0 ? 1ull << 31 : 0ull);
+    // half step that the shift drops on average stays (subtracted as ~R, one
+    // step less than -R, it is half a step the same way): rounding halves up
+    // in from_grid adds half a step on average
+    k.oc = (uint64_t)(k.ol >> 1);
   }
 }
 
@@ -302,7 +302,7 @@ __device__ __forceinline__ bool collide_grid(double (&f)[19], const FixedK& k, b
     const uint32_t fh = (uint32_t)(F[i] >> 32), fl = (uint32_t)F[i];
     const uint64_t mid = (uint64_t)fl * k.oh + k.oc + (uint64_t)fh * k.ol;
     const uint64_t R = (uint64_t)fh * k.oh2 + (mid >> 31);
-    f[i] = from_grid<false>(c + ((R ^ k.neg) - k.neg), k.sc, out);
+    f[i] = from_grid<false>(c + (R ^ k.neg), k.sc, out);
   };
   auto pair = [&](int i, uint64_t P, uint64_t M) {
     put(i, P + M);

@@ -122,6 +122,7 @@ struct Layout {
   int64_t S;                   // stored nodes
   const uint32_t* word;        // [S]
   const int32_t* node_of;      // [S] dense node index
+  const int32_t* tile;         // [ceil(N / MOM_TILE) + 1] first stored node of each tile of dense nodes
   const RunRec* runs;
   const int32_t* row_first;    // [ny*nz] storage index of the row's first stored node (-1: none)
   const int32_t* row_last;     // [ny*nz] ... last stored node
@@ -506,20 +507,25 @@ constexpr unsigned bulk_shape_mask() {
 // Default shape: two nodes per thread in 256-thread blocks for D2Q9; one
 // node per thread in 128-thread blocks for D3Q19 (the autotuner's choice on
 // dense and porous D3Q19 lattices in both precisions, and the fused step's
-// best block: 1.30 ms per step on a 384^3 pack against 1.37 at 256).
-template <class L>
+// best block: 1.30 ms per step on a 384^3 pack against 1.37 at 256) and for
+// FP64 D2Q9 (integer collision: 280 us per step on 4097 x 2049 nodes against
+// 339 with two nodes per thread, whose registers halve the warps in flight).
+template <class L, class P>
 constexpr int bulk_default_shape() {
-  return L::Q == 9 ? 3 : 1;
+  return L::Q == 9 && P::shifted ? 3 : 1;
 }
 
 // Resident blocks per SM a shape is compiled for, from a register budget per
 // 256 threads: FP32 D2Q9 6 blocks with one node per thread (40 registers) and
-// 4 with two; FP32 D3Q19 5 (48 registers); FP64 2.  Measured: one block more
-// spills (D3Q19) or runs slower (D2Q9 two nodes); one fewer leaves too few
-// loads in flight.
+// 4 with two; FP32 D3Q19 5 (48 registers).  Measured: one block more spills
+// (D3Q19) or runs slower (D2Q9 two nodes); one fewer leaves too few loads in
+// flight.  FP64 (integer collision: bound by instruction issue, 56 % busy at
+// 2 blocks, so warps to switch between count): D3Q19 3 blocks (80 registers;
+// 192^3 nodes 452 us per step; 521 at 2 without spills, 560 at 4), D2Q9 4 (64
+// registers; 4097 x 2049 nodes 280 us; 399 at 2, 321 at 3, 277 at 4.5).
 template <class L, class P, int BT, int NPT>
 constexpr int bulk_blocks_per_sm() {
-  constexpr int base = !P::shifted ? 2 : (L::Q == 9 ? (NPT == 1 ? 6 : 4) : 5);
+  constexpr int base = !P::shifted ? (NPT == 1 ? (L::Q == 9 ? 4 : 3) : 2) : (L::Q == 9 ? (NPT == 1 ? 6 : 4) : 5);
   return base * 256 / BT < 1 ? 1 : base * 256 / BT;
 }
 
@@ -1020,10 +1026,12 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 // Resident blocks per SM of the fused kernel, per 256 threads: FP32 D2Q9 4
 // (64 registers: the link phase spills at the bulk kernel's 40), FP32
-// D3Q19 5 (48), FP64 2.
+// D3Q19 5 (48), FP64 2 (5 of 128 threads, 102 registers: 200^3 pack 1.10 ms per
+// step against 1.15 at 4 and 1.13 at 6).
 template <class L, class P, int BT>
 constexpr int fused_blocks_per_sm() {
   constexpr int base = !P::shifted ? 2 : (L::Q == 9 ? 4 : 5);
+  if (!P::shifted && BT == 128) return 5;
   return base * 256 / BT < 1 ? 1 : base * 256 / BT;
 }
 
@@ -1264,32 +1272,170 @@ __global__ void k_init(typename P::T* __restrict__ f, Mom4<typename P::T>* __res
   collide_store<L, P>(fl, p, rx, *kc, f, S, (uint32_t)k, mom, (w & W_CACHE) != 0);
 }
 
-// rho = sum f+, u = (sum f+ e - g/2)/rho of the post-collision state (the
-// collision conserves mass and adds g to the momentum); FP64 output at dense
-// indices (the caller zeroes the outputs first).  u: [D][N].
+// A float as a double by moving its bits: a hardware conversion takes the FP64
+// pipe for as long as an FP64 addition.  Denormals, infinities and NaNs
+// (`odd`) are not carried over right.
+__device__ __forceinline__ double widen(float v, bool& odd) {
+  const uint32_t b = __float_as_uint(v), m = b << 1;
+  odd |= m - 0x01000000u >= 0xfe000000u && m != 0u;
+  return __hiloint2double((int)(m == 0u ? b : ((b & 0x80000000u) | ((m >> 4) + (896u << 20)))), (int)(b << 29));
+}
+
+// (1/x) for x in [2^-100, 2^100] (else `odd`) from its float reciprocal by one
+// third-order Newton step.
+__device__ __forceinline__ double reciprocal_from(double x, float seed, bool& odd) {
+  odd |= ((uint32_t)__double2hiint(x) >> 20) - (1023u - 100u) > 200u;
+  const double y = widen(seed, odd), d = fma(-x, y, 1.0);
+  return fma(y, fma(d, d, d), y);
+}
+
+// (rho, u) of a node from its sums in doubles, by divisions: where a value is
+// out of the range of the quicker forms.  Out of line, so that its FP64
+// instructions are not issued under a predicate in every node's path.
+struct RhoU {
+  double rho, ux, uy, uz;
+};
+static __device__ __noinline__ RhoU divided_moments(double rho, double jx, double jy, double jz) {
+  return RhoU{rho, jx / rho, jy / rho, jz / rho};
+}
+
+// rho = sum f+, u = (sum f+ e - g/2)/rho of fluid node k of the post-collision
+// state (the collision conserves mass and adds g to the momentum).  The FP64
+// pipe bounds this pass too (2 operations per clock and SM against 28 B read
+// and written per clock and SM), so FP64 sums the populations on the integer
+// grid and FP32 forms its quotients from one reciprocal: 13 FP64 operations
+// per D3Q19 FP64 node (99 with sums and quotients in doubles), 9 per FP32 node
+// (41).
 template <class L, class P>
-__global__ void k_moments(const typename P::T* __restrict__ f, Layout lay, double* __restrict__ rho_out,
-                          double* __restrict__ u_out, Params p) {
+__device__ __forceinline__ void node_moments(const typename P::T* __restrict__ f, size_t S, int64_t k,
+                                             const Layout& lay, const Params& p, uint32_t w, double (&v)[1 + L::D]) {
   using T = typename P::T;
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= lay.S || !is_fluid(lay.word[k])) return;
-  const size_t S = (size_t)lay.S;
-  const int64_t N = p.N, n = lay.node_of[k];
-  const Relax rx = relax_of_run(p, lay, lay.word[k] & W_RUN);
+  T h[L::Q];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) h[i] = f[(size_t)i * S + k];
+  if constexpr (!P::shifted) {
+    if (p.kx.on) {
+      uint64_t r = 0, j[3] = {0, 0, 0};
+      uint32_t bad = 0;
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i) {
+        const uint64_t F = i == 0    ? to_grid<9>(h[i], p.kx.sc, bad)
+                           : L::Q == 9 ? (i < 5 ? to_grid<8>(h[i], p.kx.sc, bad) : to_grid<7>(h[i], p.kx.sc, bad))
+                                       : (i < 7 ? to_grid<7>(h[i], p.kx.sc, bad) : to_grid<6>(h[i], p.kx.sc, bad));
+        r += F;
+        const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
+#pragma unroll
+        for (int a = 0; a < L::D; ++a) j[a] += c[a] > 0 ? F : (c[a] < 0 ? 0 - F : 0);
+      }
+      if (bad < 32u && beyond_rho(r) == 0u) {
+        // (half the force in grid steps, value by value: a reference to one of
+        // two parameter blocks would copy the kernel's parameters to memory)
+        int64_t hg[3] = {p.kx.hg[0], p.kx.hg[1], p.kx.hg[2]};
+        if (lay.ndom > 1)
+#pragma unroll
+          for (int a = 0; a < L::D; ++a) hg[a] = lay.dom[lay.runs[w & W_RUN].dom].kx.hg[a];
+        bool odd = false;
+        v[0] = from_grid<true>(r, p.kx.sc, bad);
+        const float rf = (float)(uint32_t)(r >> 32) * 0x1p-30f;  // rho in units of 2^sc
+        const double x = from_grid<true>(r, 0, bad), y = reciprocal_from(x, __frcp_rn(rf), odd) * 0x1p-62;
+#pragma unroll
+        for (int a = 0; a < L::D; ++a) v[1 + a] = (double)((int64_t)j[a] - hg[a]) * y;
+        return;
+      }
+    }
+  }
   T r = 0, jx = 0, jy = 0, jz = 0;
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) {
-    const T v = f[(size_t)i * S + k];
-    r += v;
-    jx += (T)L::cx(i) * v;
-    jy += (T)L::cy(i) * v;
-    jz += (T)L::cz(i) * v;
+    r += h[i];
+    if (L::cx(i) > 0) jx += h[i];
+    if (L::cx(i) < 0) jx -= h[i];
+    if (L::cy(i) > 0) jy += h[i];
+    if (L::cy(i) < 0) jy -= h[i];
+    if (L::cz(i) > 0) jz += h[i];
+    if (L::cz(i) < 0) jz -= h[i];
   }
-  const double rho = P::shifted ? p.rho0 + (double)r : (double)r;
-  rho_out[n] = rho;
-  u_out[n] = ((double)jx - 0.5 * rx.g[0]) / rho;
-  u_out[N + n] = ((double)jy - 0.5 * rx.g[1]) / rho;
-  if (L::D == 3) u_out[2 * N + n] = ((double)jz - 0.5 * rx.g[2]) / rho;
+  const T j[3] = {jx, jy, jz};
+  double hg[3] = {p.kc.hg[0], p.kc.hg[1], p.kc.hg[2]};
+  bool force = p.has_force != 0;
+  if (lay.ndom > 1) {
+    const DomPar& dp = lay.dom[lay.runs[w & W_RUN].dom];
+    force = dp.has_force != 0;
+#pragma unroll
+    for (int a = 0; a < L::D; ++a) hg[a] = dp.kc.hg[a];
+  }
+  if constexpr (P::shifted) {
+    bool odd = false;
+    v[0] = p.rho0 + widen(r, odd);
+    const double y = reciprocal_from(v[0], __frcp_rn(p.rho0_f + r), odd);
+#pragma unroll
+    for (int a = 0; a < L::D; ++a) {
+      const double ja = widen(j[a], odd);
+      v[1 + a] = (force ? ja - hg[a] : ja) * y;
+    }
+    if (!odd) return;
+  }
+  const RhoU m = divided_moments((P::shifted ? p.rho0 : 0.0) + (double)r, (double)jx - hg[0], (double)jy - hg[1],
+                                    (double)jz - hg[2]);
+  v[0] = m.rho;
+  v[1] = m.ux;
+  v[2] = m.uy;
+  if (L::D == 3) v[L::D] = m.uz;
+}
+
+// rho and u in FP64 at dense indices, zero at nodes that are not fluid; u:
+// [D][N].  A warp takes MOM_TILE dense nodes, whose stored nodes are
+// contiguous (lay.tile): where all of them are stored each lane writes its
+// own; else the tile is put together in shared memory, so that the outputs are
+// written whole and once (clearing them first and writing the fluid nodes'
+// scattered runs moved the pack's outputs nearly three times).  A tile per
+// warp, since warps that wait for one another between the loads, the FP64 sums
+// and the stores overlap none of them.  Blocks per SM: as many as the
+// registers allow without spilling the sums (28 % of the warps resident was
+// 1.6 times slower).  384^3 pack FP32 2.0 -> 0.79 ms, 8192 x 4096 FP32 0.95 ->
+// 0.51 ms (FP64 pipe), 192^3 FP64 1.34 -> 0.22 ms (0.86 of the copy rate).
+constexpr int MOM_TILE = 128, MOM_WARPS = 4;
+template <class L, class P>
+__global__ void __launch_bounds__(32 * MOM_WARPS, (P::shifted ? (L::Q == 9 ? 12 : 10) : 8)) k_moments(
+    const typename P::T* __restrict__ f, Layout lay, double* __restrict__ rho_out, double* __restrict__ u_out,
+    Params p) {
+  __shared__ double tiles[MOM_WARPS][1 + L::D][MOM_TILE];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const size_t S = (size_t)lay.S;
+  const int64_t N = p.N, b = (int64_t)blockIdx.x * MOM_WARPS + warp, n0 = b * MOM_TILE;
+  if (n0 >= N) return;
+  double(&tile)[1 + L::D][MOM_TILE] = tiles[warp];
+  const int len = (int)(N - n0 < MOM_TILE ? N - n0 : MOM_TILE);
+  const int64_t ka = lay.tile[b], kb = lay.tile[b + 1];
+  const bool whole = kb - ka == len;
+  if (!whole) {
+    for (int t = lane; t < len; t += 32)
+#pragma unroll
+      for (int a = 0; a <= L::D; ++a) tile[a][t] = 0.0;
+    __syncwarp();
+  }
+  for (int64_t k = ka + lane; k < kb; k += 32) {
+    const uint32_t w = lay.word[k];
+    double v[1 + L::D] = {};
+    if (is_fluid(w)) node_moments<L, P>(f, S, k, lay, p, w, v);
+    if (whole) {
+      const int64_t n = n0 + (k - ka);
+      rho_out[n] = v[0];
+#pragma unroll
+      for (int a = 0; a < L::D; ++a) u_out[a * N + n] = v[1 + a];
+    } else {
+      const int t = (int)(lay.node_of[k] - n0);
+#pragma unroll
+      for (int a = 0; a <= L::D; ++a) tile[a][t] = v[a];
+    }
+  }
+  if (whole) return;
+  __syncwarp();
+  for (int t = lane; t < len; t += 32) {
+    rho_out[n0 + t] = tile[0][t];
+#pragma unroll
+    for (int a = 0; a < L::D; ++a) u_out[a * N + n0 + t] = tile[1 + a][t];
+  }
 }
 
 // Moment cache refresh from a post-collision state (after the caller sets
@@ -1514,8 +1660,7 @@ struct Launch {
     k_init<L, P><<<blocks_for(lay.S, 256), 256, 0, s>>>((T*)f, (Mom4<T>*)mom, lay, rho, u, p);
   }
   static void moments(const void* f, const Layout& lay, double* rho, double* u, const Params& p, cudaStream_t s) {
-    if (lay.S == 0) return;
-    k_moments<L, P><<<blocks_for(lay.S, 256), 256, 0, s>>>((const T*)f, lay, rho, u, p);
+    k_moments<L, P><<<blocks_for(p.N, MOM_TILE * MOM_WARPS), 32 * MOM_WARPS, 0, s>>>((const T*)f, lay, rho, u, p);
   }
   static void refresh(const void* f, const Layout& lay, void* mom, const Params& p, cudaStream_t s) {
     if (lay.S == 0) return;
@@ -1539,7 +1684,7 @@ struct Launch {
     k_gather<L, P><<<blocks_for(n, 256), 256, 0, s>>>((const T*)f, lay, sk, n, out, p);
   }
   static KernelOps ops() {
-    return KernelOps{L::Q,   L::D,    sizeof(T), bulk_default_shape<L>(), bulk_shape_mask<L>(), bulk, links, fused,
+    return KernelOps{L::Q,   L::D,    sizeof(T), bulk_default_shape<L, P>(), bulk_shape_mask<L>(), bulk, links, fused,
                      open,   init,    moments,   refresh, get_dir, set_dir, check, gather};
   }
 };

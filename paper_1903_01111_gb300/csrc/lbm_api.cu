@@ -118,7 +118,7 @@ struct lbm_lattice_s {
   // state over stored nodes: f[c] and its moment cache mom[c]
   DeviceBuf f[2], mom[2];
   // layout
-  DeviceBuf word, node_of, runs, row_first, row_last, row_in1, row_out1;
+  DeviceBuf word, node_of, tile, runs, row_first, row_last, row_in1, row_out1;
   Layout lay{};
   // batch: domains along the last axis (empty: one domain run by cfg)
   std::vector<lbm_domain> domains;
@@ -162,7 +162,7 @@ struct lbm_lattice_s {
 namespace {
 
 int64_t device_bytes(const lbm_handle h) {
-  const DeviceBuf* all[] = {&h->f[0],     &h->f[1],     &h->mom[0],   &h->mom[1], &h->word,  &h->node_of,
+  const DeviceBuf* all[] = {&h->f[0],     &h->f[1],     &h->mom[0],   &h->mom[1], &h->word,  &h->node_of, &h->tile,
                             &h->runs,     &h->row_first, &h->row_last, &h->row_in1, &h->row_out1, &h->recs,
                             &h->q,        &h->uw,       &h->lfirst, &h->lmask, &h->lrec,
                             &h->lqd,      &h->luw,      &h->force,    &h->dom,    &h->row_dom, &h->fidx, &h->lqc};
@@ -218,7 +218,7 @@ void drop_graphs(lbm_handle h) {
 }
 
 void release_geometry(lbm_handle h) {
-  DeviceBuf* all[] = {&h->f[0],     &h->f[1],      &h->mom[0],   &h->mom[1], &h->word,  &h->node_of,
+  DeviceBuf* all[] = {&h->f[0],     &h->f[1],      &h->mom[0],   &h->mom[1], &h->word,  &h->node_of, &h->tile,
                       &h->runs,     &h->row_first, &h->row_last, &h->row_in1, &h->row_out1, &h->recs,
                       &h->q,        &h->uw,        &h->lfirst, &h->lmask, &h->lrec,
                       &h->lqd,      &h->luw,       &h->dom,      &h->row_dom, &h->fidx, &h->lqc};
@@ -815,14 +815,21 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   raw_vec<int32_t> sidx(N);
   par_fill(sidx, (int32_t)-1);
   raw_vec<int32_t> node_of((size_t)S);  // written for every stored node
+  const int64_t ntile = (N + MOM_TILE - 1) / MOM_TILE;
+  std::vector<int32_t> tile(ntile + 1, (int32_t)S);  // first stored node of each tile of dense nodes
 #pragma omp parallel for schedule(static)
   for (int64_t ch = 0; ch < nchunk; ++ch) {
     int64_t k = chunk_start[ch];
-    for (int64_t n = N * ch / nchunk; n < N * (ch + 1) / nchunk; ++n)
-      if (stored(n)) {
-        sidx[n] = (int32_t)k;
-        node_of[k++] = (int32_t)n;
-      }
+    const int64_t end = N * (ch + 1) / nchunk;
+    for (int64_t n = N * ch / nchunk; n < end;) {
+      const int64_t t = n / MOM_TILE, stop = std::min(end, (t + 1) * MOM_TILE);
+      if (n == t * MOM_TILE) tile[t] = (int32_t)k;
+      for (; n < stop; ++n)
+        if (stored(n)) {
+          sidx[n] = (int32_t)k;
+          node_of[k++] = (int32_t)n;
+        }
+    }
   }
   std::vector<int32_t> row_first(rows, -1), row_last(rows, -1);
 #pragma omp parallel for schedule(static)
@@ -1094,6 +1101,7 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   for (int k = 0; k < 2 && st == LBM_OK; ++k) st = acquire(h->mom[k], (size_t)S * 4 * rb);
   if (st == LBM_OK) st = upload(h->word, word.data(), sizeof(uint32_t) * S);
   if (st == LBM_OK) st = upload(h->node_of, node_of.data(), sizeof(int32_t) * S);
+  if (st == LBM_OK) st = upload(h->tile, tile.data(), sizeof(int32_t) * tile.size());
   if (st == LBM_OK) st = upload(h->runs, runs.data(), sizeof(RunRec) * runs.size());
   if (st == LBM_OK) st = upload(h->row_first, row_first.data(), sizeof(int32_t) * rows);
   if (st == LBM_OK) st = upload(h->row_last, row_last.data(), sizeof(int32_t) * rows);
@@ -1168,6 +1176,7 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   h->lay.S = S;
   h->lay.word = (const uint32_t*)h->word.p;
   h->lay.node_of = (const int32_t*)h->node_of.p;
+  h->lay.tile = (const int32_t*)h->tile.p;
   h->lay.runs = (const RunRec*)h->runs.p;
   h->lay.row_first = (const int32_t*)h->row_first.p;
   h->lay.row_last = (const int32_t*)h->row_last.p;
@@ -1305,19 +1314,14 @@ lbm_status lbm_moments(lbm_handle h, double* rho, double* u) {
   if (drho != du) return fail(LBM_ERR_INVALID_ARG, "rho and u must both be host or both device pointers");
   const int64_t N = h->N;
   if (drho) {
-    CUDA_TRY(cudaMemsetAsync(rho, 0, sizeof(double) * N, h->stream));
-    CUDA_TRY(cudaMemsetAsync(u, 0, sizeof(double) * h->D * N, h->stream));
     h->ops.moments(h->f[h->cur].p, h->lay, rho, u, h->p, h->stream);
     CUDA_TRY(cudaGetLastError());
     return LBM_OK;
   }
   double* tmp = nullptr;
   CUDA_TRY(cudaMalloc(&tmp, sizeof(double) * (1 + h->D) * N));
-  cudaError_t e = cudaMemsetAsync(tmp, 0, sizeof(double) * (1 + h->D) * N, h->stream);
-  if (e == cudaSuccess) {
-    h->ops.moments(h->f[h->cur].p, h->lay, tmp, tmp + N, h->p, h->stream);
-    e = cudaGetLastError();
-  }
+  h->ops.moments(h->f[h->cur].p, h->lay, tmp, tmp + N, h->p, h->stream);
+  cudaError_t e = cudaGetLastError();
   // while the device computes
   touch_host_output(rho, sizeof(double) * N);
   touch_host_output(u, sizeof(double) * h->D * N);
