@@ -488,7 +488,7 @@ __device__ __forceinline__ void adj_open_row(int t, typename P::T* __restrict__ 
   const size_t S = (size_t)lay.S;
   if (inlet_side && p.inlet) {
     // the inflow velocity does not depend on the row's storage: issued first
-    const T uin = (T)inlet_velocity(p, lay, y);
+    const T uin = ((const T*)lay.row_uin)[y];
     const int32_t k0 = lay.row_first[y];
     if (k0 >= 0 && (lay.word[k0] & W_OPEN)) {
       const uint32_t k1 = (uint32_t)k0 + 1;

@@ -46,11 +46,11 @@ inline void fold_fixed(FixedK& k, double omega, double fpre3, const double g[3],
   const double m = std::frexp(rho0, &e2);  // rho0 = m 2^e2, m in [1/2, 1)
   k.sc = m < 0.75 ? e2 - 1 : e2;
   bool on = e2 > -900 && e2 < 900;
+  if (on) k.step = std::ldexp(1.0, k.sc - 62);
   for (int a = 0; a < 3; ++a) on = on && std::fabs(g[a]) <= kFixedMaxForce * rho0;
   k.on = on ? 1 : 0;
   if (!on) return;
   const double unit = std::ldexp(1.0, 62 - k.sc);  // grid steps per 1
-  k.step = std::ldexp(1.0, k.sc - 62);
   auto steps = [&](double v) { return (int64_t)std::llrint(v * unit); };
   auto rate = [](double v) { return halves((int64_t)std::llrint(std::ldexp(v, 64))); };
   for (int a = 0; a < 3; ++a) k.hg[a] = steps(0.5 * g[a]);
@@ -326,6 +326,98 @@ __device__ __forceinline__ bool collide_grid(double (&f)[19], const FixedK& k, b
   pair(15, Byz + (uint64_t)Syz, my + mz);
   pair(17, Byz - (uint64_t)Syz, my - mz);
   m = NodeMom{r, ux, uy, uz};
+  return bad < 32u && wide == 0u && (int32_t)out >= 0;
+}
+
+// v (|v| < 1/2, else `wide`) in 2^-60, toward zero.
+__device__ __forceinline__ int64_t velocity_grid(double v, uint32_t& wide) {
+  const uint32_t lo = (uint32_t)__double2loint(v), hi = (uint32_t)__double2hiint(v);
+  const uint32_t e = (hi >> 20) & 0x7ffu;
+  wide |= e > 1021u ? 1u : 0u;
+  const uint32_t n = 1025u - e;  // places below the 63-bit significand; 0 and denormals vanish
+  const uint64_t m = ((uint64_t)((__funnelshift_l(lo, hi, 10) & 0x3fffffffu) | 0x40000000u) << 32) | (lo << 10);
+  const int64_t a = (int64_t)(n < 64u ? m >> n : 0ull), s = (int32_t)hi >> 31;
+  return (a ^ s) - s;
+}
+
+// e . (x, y, z) for a direction given as integers in {-1, 0, 1}.
+__device__ __forceinline__ int64_t dot_grid(const int (&e)[3], int64_t x, int64_t y, int64_t z) {
+  auto term = [](int c, int64_t v) {
+    const int64_t s = c >> 31, on = -(int64_t)(c & 1);
+    return ((v ^ s) & on) - s;
+  };
+  return term(e[0], x) + term(e[1], y) + term(e[2], z);
+}
+
+// VIBB link value (Sec. 3.1) on the grid.  With t = rho_d/rho at x_f and x_ff,
+// G = t f+_i' there, K(u) = 2 e.u + 3 (e.u)^2 - u.u and Delta the value at x_f
+// minus that at x_ff, the rule's feq(rho_d, u_d) + fneq_d is
+//   G_ff + 2 q Delta G + 3/2 w rho_d (K(u_d) - K(u_ff) - 2 q Delta K):
+// the equilibria's rest parts cancel, and every difference is formed exactly.
+// Eight FP64 operations (two reciprocals) in place of about 120, each of which
+// holds the FP64 pipe for 64 clocks of a warp's quarter of an SM.
+// wq: the link's velocity weights (cf, cff, cw) in 2^-62; diag: the
+// direction's weight is 1/36.  False: outside the grid's range, val unset.
+template <int SH, bool D3>
+__device__ __forceinline__ bool vibb_grid(const int (&e)[3], bool diag, double q, const int64_t (&wq)[3], double fpf,
+                                          double fpff, const double (&mf)[4], const double (&mff)[4], bool moving,
+                                          const double (&uw)[3], double wall, int local_rho, const FixedK& k,
+                                          double& val) {
+  constexpr int D = D3 ? 3 : 2;
+  uint32_t bad = 0, wide = 0;
+  const uint64_t F = to_grid<SH>(fpf, k.sc, bad), FF = to_grid<SH>(fpff, k.sc, bad);
+  const uint64_t R = to_grid<10>(mf[0], k.sc, bad), RR = to_grid<10>(mff[0], k.sc, bad);
+  const uint64_t Q = to_grid<10>(q, 0, bad);
+  const Halves hq = halves((int64_t)Q);
+  const uint64_t dR = R - RR;
+  wide |= beyond_rho(R) | beyond_rho(RR) | beyond<59>(dR);
+  const uint64_t rd = local_rho && Q > (1ull << 61) ? R : RR + (uint64_t)mul_grid<3>(hq, halves((int64_t)dR));
+  const Halves hd = halves((int64_t)rd);
+  // t - 1 in 2^-59
+  const int64_t tf = mul_grid<0>(hd, halves(reciprocal_grid(R))) - (1ll << 59);
+  const int64_t tff = mul_grid<0>(hd, halves(reciprocal_grid(RR))) - (1ll << 59);
+  wide |= beyond<57>((uint64_t)tf) | beyond<57>((uint64_t)tff);
+  const int64_t G = (int64_t)F + mul_grid<5>(halves((int64_t)F), halves(tf));
+  const int64_t GG = (int64_t)FF + mul_grid<5>(halves((int64_t)FF), halves(tff));
+  wide |= beyond<59>((uint64_t)(G - GG));
+  int64_t v = GG + mul_grid<3>(hq, halves(G - GG));
+  // K in 2^-59 of a velocity in 2^-60
+  auto K = [&](const int64_t (&u)[3]) {
+    const int64_t eu = dot_grid(e, u[0], u[1], u[2]);
+    wide |= beyond<59>((uint64_t)eu);
+    const Halves he = halves(eu);
+    int64_t r = eu + 3 * mul_grid<3>(he, he);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      const Halves h = halves(u[a]);
+      r -= mul_grid<3>(h, h);
+    }
+    return r;
+  };
+  int64_t u[3] = {0, 0, 0}, uu[3] = {0, 0, 0}, ud[3] = {0, 0, 0};
+  const Halves cf = halves(wq[0]), cff = halves(wq[1]), cw = halves(wq[2]);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    u[a] = velocity_grid(mf[1 + a], wide);
+    uu[a] = velocity_grid(mff[1 + a], wide);
+    ud[a] = mul_grid<2>(cf, halves(u[a])) + mul_grid<2>(cff, halves(uu[a]));
+    if (moving) ud[a] += mul_grid<2>(cw, halves(velocity_grid(uw[a], wide)));
+    wide |= beyond<59>((uint64_t)ud[a]);
+  }
+  const int64_t Kf = K(u), Kff = K(uu), Kd = K(ud);
+  wide |= beyond<59>((uint64_t)(Kf - Kff));
+  const int64_t X = Kd - Kff - mul_grid<3>(hq, halves(Kf - Kff));
+  wide |= beyond<57>((uint64_t)X);
+  // 3/2 w in 2^-64: 1/24 (diagonal), 1/12 or 1/6 (axis)
+  const Halves W = diag ? halves(0x0aaaaaaaaaaaaaabll) : (D3 ? halves(0x1555555555555555ll) : halves(0x2aaaaaaaaaaaaaabll));
+  v += mul_grid<5>(halves(mul_grid<0>(hd, W)), halves(X));
+  uint32_t out = 0;
+  if (moving) {
+    const double ws = wall / k.step;  // k.step is a power of two
+    wide |= ((uint32_t)__double2hiint(ws) & 0x7fffffffu) >= 0x43b00000u ? 1u : 0u;
+    v += __double2ll_rn(ws);
+  }
+  val = from_grid<true>((uint64_t)v, k.sc, out);
   return bad < 32u && wide == 0u && (int32_t)out >= 0;
 }
 

@@ -75,7 +75,9 @@ constexpr uint32_t W_GHOST = 1u << 31;
 // node k of the run sits at x = k + xk), its row (y, z), the domain the row
 // belongs to, and for each neighbour row (slot order below) dbase = the
 // storage index of (x0, row') minus k0 (so that the pull from (x + dx, row')
-// is k + dbase + dx).  48 B.
+// is k + dbase + dx).  48 B.  D2Q9 has two neighbour rows; dbase[2] holds the
+// run's open ends instead: bit 0 when it starts next to an open inlet node (at
+// x = 1), bit 1 when it ends at x = dbase[2] >> 2 next to an open outlet node.
 struct __align__(16) RunRec {
   int32_t xk, y, z, dom;
   int32_t dbase[8];
@@ -133,6 +135,9 @@ struct Layout {
   int32_t ndom;
   const uint32_t* fluid;       // [nfluid] storage indices of the fluid nodes (FP64 lattices), else null
   int64_t nfluid;
+  const void* row_uin;         // [ny] inlet velocity of each row, storage precision (open inlet)
+  const uint32_t* groups;      // D2Q9: 32-node groups with links (nlinked of them), then those without
+  int64_t nlinked, ngroups;
 };
 
 __device__ __forceinline__ Relax relax_params(const Params& p) {
@@ -161,6 +166,21 @@ struct __align__(16) LinkRec {
 };
 
 // --------------------------------------------------------------- helpers --
+
+// Clears the force slot of the next step (the grid's first block).
+template <int BT>
+__device__ __forceinline__ void clear_force(double* __restrict__ force_next, int nbody) {
+  if (force_next && blockIdx.x == 0)
+    for (int t = threadIdx.x; t < 3 * nbody; t += BT) force_next[t] = 0.0;
+}
+
+// Programmatic dependent launch: a step kernel lets its successor start as soon
+// as all its own blocks have, and the successor reads what no kernel writes
+// (node words, runs, link records) before it waits for the predecessor's
+// results.  On lattices that take microseconds a step the launch and those
+// loads are a third of it.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Equilibrium of Eq. (feq), C = 1, in storage form: r is rho (F64) or
 // rho - rho0 (F32S); rho is the full density.
@@ -477,6 +497,75 @@ __device__ __forceinline__ void pull_node(const T* __restrict__ fin, size_t S, u
   for (int i = 0; i < L::Q; ++i) f[i] = __ldg(fk + ((ptrdiff_t)i * (ptrdiff_t)S + d[i]));
 }
 
+// ------------------------------------------------------------ open sides --
+
+// Sec. 4.3: inlet column x = 0 (storage k0) by non-equilibrium extrapolation
+// from x = 1 with the parabolic velocity u_in(y) = 4 u_max (y - y0)(y1 - y)/
+// (y1 - y0)^2 (tabulated on the host: in doubles per step it took 30 FP64
+// instructions of a warp); f and mom hold the state of the fluid node at x = 1,
+// adjacent in storage.
+template <class L, class P>
+__device__ __forceinline__ void fill_inlet(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom,
+                                           size_t S, uint32_t k0, int y, const Layout& lay, const Params& p) {
+  using T = typename P::T;
+  const T uin = ((const T*)lay.row_uin)[y];
+  const uint32_t k1 = k0 + 1;
+  const Mom4<T> m1 = mom[k1];
+  const T rho1 = P::shifted ? par<T>(p.rho0, p.rho0_f) + m1.r : m1.r;
+  T v[L::Q];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) v[i] = f[i * S + k1];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i)
+    f[i * S + k0] = equilibrium<L, P>(i, m1.r, rho1, uin, (T)0, (T)0) +
+                    (v[i] - equilibrium<L, P>(i, m1.r, rho1, m1.ux, m1.uy, (T)0));
+}
+
+// Outlet column (storage kl): a copy of the fluid node before it.
+template <class L, class P>
+__device__ __forceinline__ void fill_outlet(typename P::T* __restrict__ f, size_t S, uint32_t kl) {
+  typename P::T v[L::Q];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) v[i] = f[i * S + kl - 1];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) f[i * S + kl] = v[i];
+}
+
+// The open columns of a state (f, mom), one thread per row and side (D2Q9):
+// the open node is the first (inlet) or last (outlet) stored node of its row.
+// Every state of a lattice with open columns holds them filled: by this kernel
+// after the initialisation, by the step kernels themselves (open_ends).
+template <class L, class P>
+__global__ void k_open(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom, Layout lay,
+                       Params p) {
+  // threads 0 .. ny-1: inlet rows; ny .. 2 ny - 1: outlet rows
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 2 * p.ny) return;
+  const size_t S = (size_t)lay.S;
+  if (t < p.ny) {
+    const int32_t k0 = lay.row_first[t];
+    if (p.inlet && k0 >= 0 && (lay.word[k0] & W_OPEN)) fill_inlet<L, P>(f, mom, S, (uint32_t)k0, t, lay, p);
+  } else {
+    const int32_t kl = lay.row_last[t - p.ny];
+    if (p.outlet && kl >= 0 && (lay.word[kl] & W_OPEN)) fill_outlet<L, P>(f, S, (uint32_t)kl);
+  }
+}
+
+// The open node beside fluid node k of run `run`, written by k's thread after
+// it stored k's state: the open columns of the next step cost no launch.  The
+// open slots' own threads store nothing.
+template <class L, class P>
+__device__ __forceinline__ void open_ends(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom,
+                                          size_t S, uint32_t k, const RunRec& run, const Layout& lay,
+                                          const Params& p) {
+  if constexpr (L::D == 2) {
+    if (!(p.inlet | p.outlet) || run.dbase[2] == 0) return;
+    const int x = (int)k + run.xk;
+    if ((run.dbase[2] & 1) && x == 1) fill_inlet<L, P>(f, mom, S, k - 1, run.y, lay, p);
+    if ((run.dbase[2] & 2) && x == (run.dbase[2] >> 2)) fill_outlet<L, P>(f, S, k + 1);
+  }
+}
+
 // ------------------------------------------------------------------ bulk --
 
 // Shapes of the bulk kernel the autotuner chooses from: threads per block,
@@ -529,41 +618,43 @@ constexpr int bulk_blocks_per_sm() {
   return base * 256 / BT < 1 ? 1 : base * 256 / BT;
 }
 
-// MULTI: the lattice holds several domains; each node's collision reads its
-// run's domain parameters.  Block (0) also clears the force slot of the
-// next step.
-template <class L, class P, bool MULTI, int BT, int NPT>
-__global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_bulk(const typename P::T* __restrict__ fin,
-                                                                       typename P::T* __restrict__ fout, Layout lay,
-                                                                       Mom4<typename P::T>* __restrict__ mom,
-                                                                       double* __restrict__ force_next, Params p) {
+// Pull, collision and store of NPT nodes k of a thread, all their pulls issued
+// before the first collision.  MULTI: the lattice holds several domains; each
+// node's collision reads its run's domain parameters.
+template <class L, class P, bool MULTI, int NPT>
+__device__ __forceinline__ void bulk_nodes(const uint32_t (&k)[NPT], const bool (&live)[NPT],
+                                           const typename P::T* __restrict__ fin, typename P::T* __restrict__ fout,
+                                           const Layout& lay, Mom4<typename P::T>* __restrict__ mom, const Params& p) {
   using T = typename P::T;
-  if (force_next && blockIdx.x == 0)
-    for (int t = threadIdx.x; t < 3 * p.nbody; t += BT) force_next[t] = 0.0;
-  const uint32_t t = blockIdx.x * BT + threadIdx.x;
   const size_t S = (size_t)lay.S;
-  const uint32_t stride = (uint32_t)((S + NPT - 1) / NPT);
-  uint32_t k[NPT], w[NPT];
+  uint32_t w[NPT];
   int dom[NPT];
-  bool live[NPT];
   T f[NPT][L::Q];
 #pragma unroll
-  for (int j = 0; j < NPT; ++j) {
-    k[j] = t + (uint32_t)j * stride;
-    live[j] = t < stride && (uint64_t)k[j] < S;
-    w[j] = live[j] ? __ldg(lay.word + k[j]) : W_GHOST;
-    dom[j] = 0;
-    if (live[j] && !(w[j] & (W_GHOST | W_OPEN))) {
-      const RunRec run = lay.runs[w[j] & W_RUN];
-      if (MULTI) dom[j] = run.dom;
-      pull_node<L>(fin, S, k[j], run, lay, p, f[j]);
+  for (int j = 0; j < NPT; ++j) w[j] = live[j] ? __ldg(lay.word + k[j]) : W_GHOST;
+  if constexpr (NPT == 1) {
+    RunRec run{};
+    if (live[0] && !(w[0] & (W_GHOST | W_OPEN))) run = lay.runs[w[0] & W_RUN];
+    dom[0] = run.dom;
+    wait_for_previous();
+    if (live[0] && !(w[0] & (W_GHOST | W_OPEN))) pull_node<L>(fin, S, k[0], run, lay, p, f[0]);
+  } else {
+    wait_for_previous();
+#pragma unroll
+    for (int j = 0; j < NPT; ++j) {
+      dom[j] = 0;
+      if (live[j] && !(w[j] & (W_GHOST | W_OPEN))) {
+        const RunRec run = lay.runs[w[j] & W_RUN];
+        if (MULTI) dom[j] = run.dom;
+        pull_node<L>(fin, S, k[j], run, lay, p, f[j]);
+      }
     }
   }
 #pragma unroll
   for (int j = 0; j < NPT; ++j) {
-    if (!live[j]) continue;
-    // ghost and open slots: zeros through the same stores (inputs at rest)
-    const bool fl = !(w[j] & (W_GHOST | W_OPEN));
+    if (!live[j] || (w[j] & W_OPEN)) continue;
+    // ghost slots: zeros through the same stores (inputs at rest)
+    const bool fl = !(w[j] & W_GHOST);
     auto rest = [&](T(&g)[L::Q]) {
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) g[i] = P::shifted ? (T)0 : (T)L::w(i);
@@ -575,7 +666,28 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_b
       else
         rest(g);
     });
+    if (L::D == 2 && fl && (p.inlet | p.outlet)) open_ends<L, P>(fout, mom, S, k[j], lay.runs[w[j] & W_RUN], lay, p);
   }
+}
+
+// Block (0) also clears the force slot of the next step.
+template <class L, class P, bool MULTI, int BT, int NPT>
+__global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_bulk(const typename P::T* __restrict__ fin,
+                                                                       typename P::T* __restrict__ fout, Layout lay,
+                                                                       Mom4<typename P::T>* __restrict__ mom,
+                                                                       double* __restrict__ force_next, Params p) {
+  let_next_start();
+  const uint32_t t = blockIdx.x * BT + threadIdx.x;
+  const uint32_t stride = (uint32_t)(((size_t)lay.S + NPT - 1) / NPT);
+  uint32_t k[NPT];
+  bool live[NPT];
+#pragma unroll
+  for (int j = 0; j < NPT; ++j) {
+    k[j] = t + (uint32_t)j * stride;
+    live[j] = t < stride && (uint64_t)k[j] < (uint64_t)lay.S;
+  }
+  bulk_nodes<L, P, MULTI, NPT>(k, live, fin, fout, lay, mom, p);
+  clear_force<BT>(force_next, p.nbody);
 }
 
 // FP64 bulk pass over the fluid nodes alone, one thread per entry of the
@@ -585,26 +697,29 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_b
 // cost as much as fluid nodes there; this pass has no such lanes.  It leaves
 // the ghost and open slots of the output unwritten: a ghost slot is read
 // only in its link's direction after the link kernel of the next step has
-// written it, and the open-column kernel rewrites the open slots before they
-// are pulled.
+// written it, and the fluid node beside an open slot writes it.
 template <class L, class P, bool MULTI, int BT>
 __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, 1>())) k_bulk_list(
     const typename P::T* __restrict__ fin, typename P::T* __restrict__ fout, Layout lay,
     Mom4<typename P::T>* __restrict__ mom, double* __restrict__ force_next, Params p) {
   using T = typename P::T;
-  if (force_next && blockIdx.x == 0)
-    for (int t = threadIdx.x; t < 3 * p.nbody; t += BT) force_next[t] = 0.0;
+  let_next_start();
   const int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
-  if (t >= lay.nfluid) return;
   const size_t S = (size_t)lay.S;
-  const uint32_t k = __ldg(lay.fluid + t);
-  const uint32_t w = __ldg(lay.word + k);
-  const RunRec run = lay.runs[w & W_RUN];
+  const bool live = t < lay.nfluid;
+  const uint32_t k = live ? __ldg(lay.fluid + t) : 0u;
+  const uint32_t w = live ? __ldg(lay.word + k) : 0u;
+  RunRec run{};
+  if (live) run = lay.runs[w & W_RUN];
+  wait_for_previous();
+  clear_force<BT>(force_next, p.nbody);
+  if (!live) return;
   T f[L::Q];
   pull_node<L>(fin, S, k, run, lay, p, f);
   collide_node<L, P, MULTI>(f, p, lay, run.dom, fout, S, k, mom, (w & W_CACHE) != 0, true, [&](T(&g)[L::Q]) {
     pull_node<L>(fin, S, k, lay.runs[w & W_RUN], lay, p, g);
   });
+  if (L::D == 2 && (p.inlet | p.outlet)) open_ends<L, P>(fout, mom, S, k, lay.runs[w & W_RUN], lay, p);
 }
 
 // Resident blocks per SM of the sequential walk (it keeps the next node's
@@ -640,8 +755,7 @@ __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_
     const typename P::T* __restrict__ fin, typename P::T* __restrict__ fout, Layout lay,
     Mom4<typename P::T>* __restrict__ mom, double* __restrict__ force_next, Params p) {
   using T = typename P::T;
-  if (force_next && blockIdx.x == 0)
-    for (int t = threadIdx.x; t < 3 * p.nbody; t += BT) force_next[t] = 0.0;
+  let_next_start();
   const size_t S = (size_t)lay.S;
   const uint32_t G = gridDim.x * BT;
   uint32_t k = blockIdx.x * BT + threadIdx.x;
@@ -649,6 +763,8 @@ __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_
   RunLite<L> run{};
   if (!(w & (W_GHOST | W_OPEN))) run = load_run_lite<L, MULTI>(lay.runs, w & W_RUN);
   uint32_t w2 = ((uint64_t)k + G < S) ? __ldg(lay.word + k + G) : W_GHOST;
+  wait_for_previous();
+  clear_force<BT>(force_next, p.nbody);
 #pragma unroll 1
   for (int it = 0; it < SEQ && (uint64_t)k < S; ++it, k += G) {
     T f[L::Q];
@@ -672,13 +788,14 @@ __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_
     const uint32_t w3 = ((uint64_t)k + 2ull * G < S) ? __ldg(lay.word + k + 2 * G) : W_GHOST;
     // (a separate zero-store branch here: the walk serves dense lattices,
     // where selecting zeros in every store measured about 2 % slower)
-    if (!fluid) {
+    if (w & W_GHOST) {
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) fout[(size_t)i * S + k] = (T)0;
-    } else {
+    } else if (fluid) {
       collide_node<L, P, MULTI>(f, p, lay, run.dom, fout, S, k, mom, (w & W_CACHE) != 0, true, [&](T(&g)[L::Q]) {
         pull_node<L>(fin, S, k, lay.runs[w & W_RUN], lay, p, g);
       });
+      if (p.inlet | p.outlet) open_ends<L, P>(fout, mom, S, k, lay.runs[w & W_RUN], lay, p);
     }
     // the next node's run record, loaded before its pulls are needed
     w = w2;
@@ -697,15 +814,24 @@ struct DirTable {
   int opp[Q];
   T w[Q];
   T e[Q][3];
+  int ie[Q][3];
 };
 
-// Equilibrium of direction d from table values (storage form, see above).
-template <class P>
-__device__ __forceinline__ typename P::T eq_dir(typename P::T w, typename P::T ex, typename P::T ey, typename P::T ez,
-                                                typename P::T r, typename P::T rho, typename P::T ux, typename P::T uy,
-                                                typename P::T uz) {
+// A direction as values (read from the table).
+template <class T>
+struct DirVal {
+  T wt, ex, ey, ez;
+  int e[3];  // the same as integers (FP64: a conversion costs as much as an addition)
+  __device__ __forceinline__ T w() const { return wt; }
+  __device__ __forceinline__ T dot(T x, T y, T z) const { return ex * x + ey * y + ez * z; }
+};
+// Equilibrium of direction `dir` (storage form, see above).
+template <class P, class Dir>
+__device__ __forceinline__ typename P::T eq_dir(const Dir& dir, typename P::T r, typename P::T rho, typename P::T ux,
+                                                typename P::T uy, typename P::T uz) {
   using T = typename P::T;
-  const T eu = ex * ux + ey * uy + ez * uz;
+  const T w = dir.w();
+  const T eu = dir.dot(ux, uy, uz);
   const T poly = (T)3 * eu + (T)4.5 * eu * eu - (T)1.5 * (ux * ux + uy * uy + uz * uz);
   return P::shifted ? w * (r + rho * poly) : w * rho * ((T)1 + poly);
 }
@@ -713,10 +839,9 @@ __device__ __forceinline__ typename P::T eq_dir(typename P::T w, typename P::T e
 // Missing population f_i(x_f, t+1) of one link in storage form (see the
 // rule list below).  fpf = f+_i'(x_f), fpff = f+_i'(x_ff), fpi = f+_i(x_f)
 // (only read by the rule that needs it, through the callbacks' values);
-// mf, mff: moments at time t at x_f and x_ff; (w, ex, ey, ez) of i'.
-template <class P>
-__device__ __forceinline__ typename P::T link_value(int rule, typename P::T q, typename P::T w, typename P::T ex,
-                                                    typename P::T ey, typename P::T ez, typename P::T fpf,
+// mf, mff: moments at time t at x_f and x_ff; dir: i'.
+template <class P, class Dir>
+__device__ __forceinline__ typename P::T link_value(int rule, typename P::T q, const Dir& dir, typename P::T fpf,
                                                     typename P::T fpff, typename P::T fpi, const Mom4<typename P::T>& mf,
                                                     const Mom4<typename P::T>& mff, typename P::T uw0,
                                                     typename P::T uw1, typename P::T uw2, typename P::T rho0,
@@ -726,7 +851,7 @@ __device__ __forceinline__ typename P::T link_value(int rule, typename P::T q, t
   // of the lattice moves (the same for every link of a launch: five FP64
   // instructions of about a hundred per link); FP32 forms it always (the
   // branch moved registers of the fused kernel into spills and cost 2 %)
-  const T wall = (P::shifted || moving) ? -(T)6 * w * rho0 * (ex * uw0 + ey * uw1 + ez * uw2) : (T)0;
+  const T wall = (P::shifted || moving) ? -(T)6 * dir.w() * rho0 * dir.dot(uw0, uw1, uw2) : (T)0;
   const T two_q = (T)2 * q;
   if (rule == 0) return fpf + wall;
   if (rule == 1) {
@@ -746,8 +871,8 @@ __device__ __forceinline__ typename P::T link_value(int rule, typename P::T q, t
   // Eq. (rhod) in storage form; optionally rho_d = rho_f when q > 1/2
   const T rd = (local_rho && q > (T)0.5) ? mf.r : two_q * mf.r + ((T)1 - two_q) * mff.r;
   const T rhod = P::shifted ? rho0 + rd : rd;
-  const T neq_f = fpf - eq_dir<P>(w, ex, ey, ez, mf.r, rhof, mf.ux, mf.uy, mf.uz);
-  const T neq_ff = fpff - eq_dir<P>(w, ex, ey, ez, mff.r, rhoff, mff.ux, mff.uy, mff.uz);
+  const T neq_f = fpf - eq_dir<P>(dir, mf.r, rhof, mf.ux, mf.uy, mf.uz);
+  const T neq_ff = fpff - eq_dir<P>(dir, mff.r, rhoff, mff.ux, mff.uy, mff.uz);
   // every quotient of the rule from one reciprocal, r = 1/(rho_f rho_ff D)
   // with D = q (1 + q) (q > 1/2) or 1 + q: 1/(rho_f rho_ff) = D r,
   // 1/D = rho_f rho_ff r, 1/(1 + q) and 1/q from 1/D
@@ -777,7 +902,7 @@ __device__ __forceinline__ typename P::T link_value(int rule, typename P::T q, t
   const T udx = cf * mf.ux + cff * mff.ux + cw * uw0;
   const T udy = cf * mf.uy + cff * mff.uy + cw * uw1;
   const T udz = cf * mf.uz + cff * mff.uz + cw * uw2;
-  return eq_dir<P>(w, ex, ey, ez, rd, rhod, udx, udy, udz) + nd + wall;
+  return eq_dir<P>(dir, rd, rhod, udx, udy, udz) + nd + wall;
 }
 
 // Direction table of the link kernels in shared memory (filled by the
@@ -792,25 +917,28 @@ __device__ __forceinline__ void fill_dir_table(DirTable<T, L::Q>& tab) {
     tab.e[d][0] = (T)L::cx(d);
     tab.e[d][1] = (T)L::cy(d);
     tab.e[d][2] = (T)L::cz(d);
+    tab.ie[d][0] = L::cx(d);
+    tab.ie[d][1] = L::cy(d);
+    tab.ie[d][2] = L::cz(d);
   }
 }
 
-// Missing population f_i(x_f, t+1) of the link (x_f = node, i' = ip) from
-// the post-collision state f (storage form, [Q][N]) and the moment cache at
-// time t; x_ff = ff (x_f when there is no second fluid node).  fpf receives
-// f+_i'(x_f, t), the link's other term of the momentum exchange.  Each rule
-// loads only what it reads.
+// Missing population f_i(x_f, t+1) of the link (x_f = node, i' = ip, opposite
+// i, as values dir) from the post-collision state (storage form, [Q][N]) and
+// the moment cache at time t; x_ff = ff (x_f when there is no second fluid
+// node).  fpf receives f+_i'(x_f, t), the link's other term of the momentum
+// exchange.  Each rule loads only what it reads.  FP64 VIBB runs on the
+// integer grid with the link's velocity weights wq[0], wq[nl], wq[2 nl] (in
+// 2^-62; q alone fixes them), in doubles where that says no.
 template <class L, class P>
-__device__ __forceinline__ typename P::T eval_link(const DirTable<typename P::T, L::Q>& tab,
+__device__ __forceinline__ typename P::T eval_link(const DirVal<typename P::T>& dir, int ip, int i,
                                                    const typename P::T* __restrict__ f,
-                                                   const Mom4<typename P::T>* __restrict__ mom, size_t N, int ip,
-                                                   int rule, typename P::T q, uint32_t node, uint32_t ff,
-                                                   typename P::T uw0, typename P::T uw1, typename P::T uw2,
-                                                   const Params& p, typename P::T& fpf, bool moving) {
+                                                   const Mom4<typename P::T>* __restrict__ mom, size_t N, int rule,
+                                                   typename P::T q, uint32_t node, uint32_t ff, typename P::T uw0,
+                                                   typename P::T uw1, typename P::T uw2, const Params& p,
+                                                   typename P::T& fpf, bool moving, const int64_t* __restrict__ wq,
+                                                   int64_t nl) {
   using T = typename P::T;
-  const int i = tab.opp[ip];
-  const T ex = tab.e[ip][0], ey = tab.e[ip][1], ez = tab.e[ip][2];
-  const T w = tab.w[ip];
   fpf = f[(size_t)ip * N + node];
   T fpff = 0, fpi = 0;
   Mom4<T> mf{0, 0, 0, 0}, mff{0, 0, 0, 0};
@@ -827,45 +955,84 @@ __device__ __forceinline__ typename P::T eval_link(const DirTable<typename P::T,
     fpff = f[(size_t)ip * N + ff];
     fpi = f[(size_t)i * N + node];
   }
-  return link_value<P>(rule, q, w, ex, ey, ez, fpf, fpff, fpi, mf, mff, uw0, uw1, uw2, par<T>(p.rho0, p.rho0_f),
+  if constexpr (!P::shifted) {
+    if (rule == 2 && p.kx.on) {
+      const int64_t c[3] = {wq[0], wq[nl], moving ? wq[2 * nl] : 0};
+      const double m0[4] = {mf.r, mf.ux, mf.uy, mf.uz}, m1[4] = {mff.r, mff.ux, mff.uy, mff.uz};
+      const double uw[3] = {uw0, uw1, uw2};
+      const double wall = moving ? -6.0 * dir.w() * p.rho0 * dir.dot(uw0, uw1, uw2) : 0.0;
+      double val;
+      if (vibb_grid<(L::D == 2 ? 8 : 7), L::D == 3>(dir.e, ip >= (L::D == 2 ? 5 : 7), q, c, fpf, fpff, m0, m1, moving, uw,
+                                                    wall, p.vibb_local_rho, p.kx, val))
+        return val;
+    }
+  }
+  return link_value<P>(rule, q, dir, fpf, fpff, fpi, mf, mff, uw0, uw1, uw2, par<T>(p.rho0, p.rho0_f),
                        p.vibb_local_rho, moving);
 }
 
-// VIBB (Sec. 3.1) with the velocity interpolation weights of the link given:
-// u_d = cf u_f + cff u_ff + cw u_w, where (cf, cff, cw) are the 1/3 : 2/3
-// blend of u*_d and u**_d and depend on q alone (the FP64 link kernel takes
-// them from a per-link array the host fills, instead of forming them from
-// 1/q and 1/(1+q) per link and step).  Otherwise as link_value's VIBB branch.
-template <class L, class P>
-__device__ __forceinline__ typename P::T vibb_weighted(const DirTable<typename P::T, L::Q>& tab,
-                                                       const typename P::T* __restrict__ f,
-                                                       const Mom4<typename P::T>* __restrict__ mom, size_t N, int ip,
-                                                       typename P::T q, uint32_t node, uint32_t ff, typename P::T uw0,
-                                                       typename P::T uw1, typename P::T uw2, const Params& p,
-                                                       typename P::T& fpf, bool moving, typename P::T cf,
-                                                       typename P::T cff, typename P::T cw) {
-  using T = typename P::T;
-  const T ex = tab.e[ip][0], ey = tab.e[ip][1], ez = tab.e[ip][2];
-  const T w = tab.w[ip];
-  fpf = f[(size_t)ip * N + node];
-  const T fpff = f[(size_t)ip * N + ff];
-  const Mom4<T> mf = mom[node], mff = mom[ff];
-  const T rho0 = par<T>(p.rho0, p.rho0_f);
-  const T wall = (P::shifted || moving) ? -(T)6 * w * rho0 * (ex * uw0 + ey * uw1 + ez * uw2) : (T)0;
-  const T two_q = (T)2 * q;
-  const T rhof = P::shifted ? rho0 + mf.r : mf.r;
-  const T rhoff = P::shifted ? rho0 + mff.r : mff.r;
-  const T rd = (p.vibb_local_rho && q > (T)0.5) ? mf.r : two_q * mf.r + ((T)1 - two_q) * mff.r;
-  const T rhod = P::shifted ? rho0 + rd : rd;
-  const T neq_f = fpf - eq_dir<P>(w, ex, ey, ez, mf.r, rhof, mf.ux, mf.uy, mf.uz);
-  const T neq_ff = fpff - eq_dir<P>(w, ex, ey, ez, mff.r, rhoff, mff.ux, mff.uy, mff.uz);
-  // fneq at d, each term rescaled by its density ratio
-  const T nd = rhod * (two_q * neq_f * rhoff + ((T)1 - two_q) * neq_ff * rhof) / (rhof * rhoff);
-  const T udx = cf * mf.ux + cff * mff.ux + cw * uw0;
-  const T udy = cf * mf.uy + cff * mff.uy + cw * uw1;
-  const T udz = cf * mf.uz + cff * mff.uz + cw * uw2;
-  return eq_dir<P>(w, ex, ey, ez, rd, rhod, udx, udy, udz) + nd + wall;
+// Direction ip from the table.
+template <class T, int Q>
+__device__ __forceinline__ DirVal<T> dir_of(const DirTable<T, Q>& tab, int ip) {
+  return DirVal<T>{tab.w[ip], tab.e[ip][0], tab.e[ip][1], tab.e[ip][2], {tab.ie[ip][0], tab.ie[ip][1], tab.ie[ip][2]}};
 }
+
+// A link's momentum exchange t e added to its body's slot by FP64 atomics.
+template <class T>
+__device__ __forceinline__ void add_force(double* __restrict__ force, int body, T t, const DirVal<T>& dir) {
+  if (dir.e[0]) atomicAdd(&force[3 * body + 0], (double)(t * dir.ex));
+  if (dir.e[1]) atomicAdd(&force[3 * body + 1], (double)(t * dir.ey));
+  if (dir.e[2]) atomicAdd(&force[3 * body + 2], (double)(t * dir.ez));
+}
+
+// Sum of the momentum exchange t e over links of one body.  FP32 adds in FP32;
+// FP64 adds integers in steps of 2^(sc - 55) (a warp's reduction of doubles is
+// 15 FP64 instructions, and rounds at the last place of the sum), and hands a
+// t of 2^(sc - 1) or more, or not a number, to `direct`, which adds it to the
+// body's slot by itself.  No sum of a warp's links reaches 2^63 steps: the
+// populations of a node add up to its density.
+template <class T>
+struct LinkForce {
+  T F[3] = {0, 0, 0};
+  template <class Direct>
+  __device__ __forceinline__ void add(T t, const DirVal<T>& dir, const FixedK&, Direct&&) {
+    F[0] += t * dir.ex;
+    F[1] += t * dir.ey;
+    F[2] += t * dir.ez;
+  }
+  __device__ __forceinline__ void reduce() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) F[a] += __shfl_down_sync(0xffffffffu, F[a], o);
+  }
+  __device__ __forceinline__ double value(int a, const FixedK&) const { return (double)F[a]; }
+};
+template <>
+struct LinkForce<double> {
+  int64_t F[3] = {0, 0, 0};
+  template <class Direct>
+  __device__ __forceinline__ void add(double t, const DirVal<double>& dir, const FixedK& k, Direct&& direct) {
+    const uint32_t hi = (uint32_t)__double2hiint(t), e = (hi >> 20) & 0x7ffu;
+    if (k.step == 0.0 || e >= (uint32_t)(1022 + k.sc)) return direct();
+    // t 2^(55 - sc) by its exponent (a t too small for that is none of a step)
+    const bool tiny = (int)e < 900 + k.sc || e == 0u;
+    const int64_t v = __double2ll_rn(
+        __hiloint2double((int)(hi + ((uint32_t)(55 - k.sc) << 20)), __double2loint(t)));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int64_t s = dir.e[a] >> 31, on = tiny ? 0 : -(int64_t)(dir.e[a] & 1);
+      F[a] += ((v ^ s) & on) - (s & on);
+    }
+  }
+  __device__ __forceinline__ void reduce() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) F[a] += __shfl_down_sync(0xffffffffu, F[a], o);
+  }
+  __device__ __forceinline__ double value(int a, const FixedK& k) const { return (double)F[a] * (k.step * 128.0); }
+};
 
 // One thread per link.  recs: storage indices and metadata; qv: q in
 // storage precision; uw: [D][nl] wall velocities or null.  force: the step's
@@ -880,12 +1047,13 @@ __device__ __forceinline__ typename P::T vibb_weighted(const DirTable<typename P
 //   Yu        (q f+_i'(x_f) + (1-q) f+_i'(x_ff) + wall)/(1+q) + q/(1+q) f+_i(x_f)  (Sec. 3)
 // with wall = 6 w rho0 (e_i . u_w).
 template <class L, class P, int SEQ>
-__global__ void __launch_bounds__(256) k_links(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom,
+__global__ void __launch_bounds__(256, (P::shifted ? 2 : 3)) k_links(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom,
                                                const LinkRec* __restrict__ recs, const typename P::T* __restrict__ qv,
                                                const typename P::T* __restrict__ uwv,
-                                               const typename P::T* __restrict__ qcv, int64_t nl,
+                                               const int64_t* __restrict__ wqv, int64_t nl,
                                                double* __restrict__ force, Params p, int64_t S_) {
   using T = typename P::T;
+  let_next_start();
   __shared__ DirTable<T, L::Q> tab;
   fill_dir_table<L>(tab);
   __syncthreads();
@@ -898,7 +1066,7 @@ __global__ void __launch_bounds__(256) k_links(typename P::T* __restrict__ f, co
   // terms with FP64 atomics directly
   const int b0 = (int)(__ldg(&recs[base].meta) >> 7) - 1;
   const size_t N = (size_t)S_;
-  T F0 = 0, F1 = 0, F2 = 0;
+  LinkForce<T> F;
   int64_t k = base + threadIdx.x;
   bool live = k < nl;
   LinkRec rec{0, 0, 0, 0};
@@ -907,6 +1075,7 @@ __global__ void __launch_bounds__(256) k_links(typename P::T* __restrict__ f, co
     rec = recs[k];
     q = qv[k];
   }
+  wait_for_previous();
 #pragma unroll 1
   for (int r = 0; r < SEQ; ++r) {
     const int64_t kn = k + blockDim.x;
@@ -927,37 +1096,21 @@ __global__ void __launch_bounds__(256) k_links(typename P::T* __restrict__ f, co
         uw1 = uwv[nl + k];
         if (L::D == 3) uw2 = uwv[2 * nl + k];
       }
-      T fpf, val;
-      // FP64 VIBB links take their velocity weights from qcv; the FP32 kernel
-      // keeps the one evaluation path (its rounding of the rule is what the
-      // FP32 adjoint's accuracy was measured with)
-      if constexpr (!P::shifted) {
-        if (qcv && rule == 2)
-          val = vibb_weighted<L, P>(tab, f, mom, N, ip, q, rec.kf, rec.kff, uw0, uw1, uw2, p, fpf, uwv != nullptr,
-                                    qcv[k], qcv[nl + k], qcv[2 * nl + k]);
-        else
-          val = eval_link<L, P>(tab, f, mom, N, ip, rule, q, rec.kf, rec.kff, uw0, uw1, uw2, p, fpf,
-                                uwv != nullptr);
-      } else {
-        val = eval_link<L, P>(tab, f, mom, N, ip, rule, q, rec.kf, rec.kff, uw0, uw1, uw2, p, fpf,
-                              uwv != nullptr);
-      }
+      T fpf;
+      const T val = eval_link<L, P>(dir_of(tab, ip), ip, tab.opp[ip], f, mom, N, rule, q, rec.kf, rec.kff, uw0, uw1,
+                                    uw2, p, fpf, uwv != nullptr, wqv + k, nl);
       f[(size_t)tab.opp[ip] * N + rec.ks] = val;
       if (body >= 0) {
         // momentum exchange (f+_i'(x_f,t) + f_i(x_f,t+1)) e_i'.  In shifted
         // storage this sums (h+_i' + h_i) e_i'; the rest part 2 w_i' rho0 e_i'
         // of every link is a geometric constant that the host adds in FP64.
         const T t = fpf + val;
-        const T ex = tab.e[ip][0], ey = tab.e[ip][1], ez = tab.e[ip][2];
-        if (body == b0) {
-          F0 += t * ex;
-          F1 += t * ey;
-          F2 += t * ez;
-        } else {
-          atomicAdd(&force[3 * body + 0], (double)(t * ex));
-          atomicAdd(&force[3 * body + 1], (double)(t * ey));
-          atomicAdd(&force[3 * body + 2], (double)(t * ez));
-        }
+        const DirVal<T> dir = dir_of(tab, ip);
+        auto direct = [&] { add_force(force, body, t, dir); };
+        if (body == b0)
+          F.add(t, dir, p.kx, direct);
+        else
+          direct();
       }
     }
     k = kn;
@@ -967,18 +1120,10 @@ __global__ void __launch_bounds__(256) k_links(typename P::T* __restrict__ f, co
   }
   if (b0 < 0) return;
   __shared__ double red[3][32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    F0 += __shfl_down_sync(0xffffffffu, F0, o);
-    F1 += __shfl_down_sync(0xffffffffu, F1, o);
-    F2 += __shfl_down_sync(0xffffffffu, F2, o);
-  }
+  F.reduce();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) {
-    red[0][warp] = (double)F0;
-    red[1][warp] = (double)F1;
-    red[2][warp] = (double)F2;
-  }
+  if (lane == 0)
+    for (int a = 0; a < 3; ++a) red[a][warp] = F.value(a, p.kx);
   __syncthreads();
   if (threadIdx.x < 3) {
     const int nw = (blockDim.x + 31) >> 5;
@@ -1007,6 +1152,7 @@ struct FusedLinks {
   const FusedRec* rec;     // [nl]
   const double* qd;        // [nl] (FP64 storage) or null
   const T* uw;             // [D][nl] wall velocities or null
+  const int64_t* wq;       // [3][nl] VIBB velocity weights in 2^-62 (FP64 storage) or null
   int64_t nl;
   int64_t ngroups;         // ceil(S / 32)
 };
@@ -1031,7 +1177,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 template <class L, class P, int BT>
 constexpr int fused_blocks_per_sm() {
   constexpr int base = !P::shifted ? 2 : (L::Q == 9 ? 4 : 5);
-  if (!P::shifted && BT == 128) return 5;
+  if (!P::shifted && BT == 128) return 4;
   return base * 256 / BT < 1 ? 1 : base * 256 / BT;
 }
 
@@ -1063,9 +1209,8 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
   __shared__ T stage[NW][L::Q][32];
   __shared__ DirTable<T, L::Q> tab;
   __shared__ double red[3][NW];
+  let_next_start();
   fill_dir_table<L>(tab);
-  if (force_next && blockIdx.x == 0)
-    for (int t = threadIdx.x; t < 3 * p.nbody; t += BT) force_next[t] = 0.0;
   __syncthreads();  // the direction table (every thread arrives here at once)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t base = blockIdx.x * BT;
@@ -1089,6 +1234,8 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
   const bool fluid = live && !(w & (W_GHOST | W_OPEN));
   T(&col)[L::Q][32] = stage[warp];
   int dom = 0;
+  wait_for_previous();
+  clear_force<BT>(force_next, p.nbody);
   if (fluid) {
     const RunRec run = lay.runs[w & W_RUN];
     if (MULTI) dom = run.dom;
@@ -1106,7 +1253,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
   }
   cp_async_commit();
   const int wb = total > 0 ? (int)(__ldg(&fl.rec[l0].meta) >> 8) - 1 : -1;
-  T F0 = 0, F1 = 0, F2 = 0;
+  LinkForce<T> F;
   for (int j = threadIdx.x; j < total; j += BT) {
     const int64_t li = l0 + j;
     const bool first_round = j == (int)threadIdx.x;
@@ -1122,37 +1269,25 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
       if (L::D == 3) uw2 = fl.uw[2 * fl.nl + li];
     }
     T fpf;
-    const T val = eval_link<L, P>(tab, fin, mom_in, S, ip, rule, q, r.kf, r.kff, uw0, uw1, uw2, p, fpf,
-                                  fl.uw != nullptr);
+    const T val = eval_link<L, P>(dir_of(tab, ip), ip, tab.opp[ip], fin, mom_in, S, rule, q, r.kf, r.kff, uw0, uw1,
+                                  uw2, p, fpf, fl.uw != nullptr, fl.wq + li, fl.nl);
     const uint32_t o = r.kf - base;  // the node's place in the block
     stage[o >> 5][tab.opp[ip]][o & 31] = val;
     if (body >= 0) {
       // momentum exchange as in k_links
       const T t = fpf + val;
-      const T ex = tab.e[ip][0], ey = tab.e[ip][1], ez = tab.e[ip][2];
-      if (body == wb) {
-        F0 += t * ex;
-        F1 += t * ey;
-        F2 += t * ez;
-      } else {
-        atomicAdd(&force[3 * body + 0], (double)(t * ex));
-        atomicAdd(&force[3 * body + 1], (double)(t * ey));
-        atomicAdd(&force[3 * body + 2], (double)(t * ez));
-      }
+      const DirVal<T> dir = dir_of(tab, ip);
+      auto direct = [&] { add_force(force, body, t, dir); };
+      if (body == wb)
+        F.add(t, dir, p.kx, direct);
+      else
+        direct();
     }
   }
   if (wb >= 0) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      F0 += __shfl_down_sync(0xffffffffu, F0, o);
-      F1 += __shfl_down_sync(0xffffffffu, F1, o);
-      F2 += __shfl_down_sync(0xffffffffu, F2, o);
-    }
-    if (lane == 0) {
-      red[0][warp] = (double)F0;
-      red[1][warp] = (double)F1;
-      red[2][warp] = (double)F2;
-    }
+    F.reduce();
+    if (lane == 0)
+      for (int a = 0; a < 3; ++a) red[a][warp] = F.value(a, p.kx);
   }
   cp_async_wait_all();
   __syncthreads();  // staged pulls, link values and warp sums of the whole block
@@ -1173,62 +1308,172 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
   }
 }
 
-// ------------------------------------------------------------ open sides --
+// ------------------------------------------------------------ inline step --
 
-// Inlet velocity of row y: 4 u_max (y - y0)(y1 - y)/(y1 - y0)^2, with y
-// counted from the first row of the row's domain.
-__device__ __forceinline__ double inlet_velocity(const Params& p, const Layout& lay, int y) {
-  double umax = p.inlet_umax, y0 = p.inlet_y0, y1 = p.inlet_y1, yy = (double)y;
-  if (lay.ndom > 1) {
-    const DomPar& d = lay.dom[lay.row_dom[y]];
-    umax = d.inlet_umax;
-    y0 = d.inlet_y0;
-    y1 = d.inlet_y1;
-    yy = (double)(y - d.lo);
-  }
-  const double h = y1 - y0;
-  return 4.0 * umax * (yy - y0) * (y1 - yy) / (h * h);
+// D2Q9 directions in a word each (two bits a direction): cx + 1, cy + 1; the
+// opposite of direction i in four bits.  Lanes holding different directions
+// unpack them without a table in memory.
+constexpr uint32_t d2q9_pack(bool y) {
+  uint32_t v = 0;
+  for (int i = 0; i < 9; ++i) v |= (uint32_t)((y ? D2Q9::cy(i) : D2Q9::cx(i)) + 1) << (2 * i);
+  return v;
+}
+constexpr uint64_t d2q9_opposites() {
+  uint64_t v = 0;
+  for (int i = 0; i < 9; ++i) v |= (uint64_t)D2Q9::opp(i) << (4 * i);
+  return v;
 }
 
-// Sec. 4.3: inlet column x = 0 by non-equilibrium extrapolation from x = 1
-// with the parabolic velocity u_in(y); outlet column x = nx-1 copies x = nx-2.
-// One thread per row and side (D2Q9); the open node is the first (inlet) or
-// last (outlet) stored node of its row and its fluid neighbour is adjacent.
-template <class L, class P>
-__global__ void k_open(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom, Layout lay,
-                       Params p) {
+// Nodes a warp without links takes at a time (two groups: 18 FP32 loads in
+// flight a thread).
+template <class P>
+constexpr int inline_free_groups() {
+  return P::shifted ? 2 : 1;
+}
+
+// One time step of a D2Q9 lattice with its links in the pull pass.  Cut links
+// are few in two dimensions (the boundary of an area: 0.06 per node in the
+// channel batch), so the groups of 32 stored nodes are listed by whether they
+// have any: the first blocks take those with links, a group per warp, the
+// others are k_bulk's pass, two groups per warp, with no mask, link range,
+// stage or barrier to read or wait for.  A warp with links evaluates them one
+// per lane (they are contiguous in the link list) while its pulls are in
+// flight, and hands the values to their nodes through its own part of shared
+// memory.  On a lattice with fewer groups with links than the chip holds
+// blocks (`spread`) a block takes one group and evaluates its links with all
+// its warps: a wall row has 96, three rounds of one warp.
+constexpr int64_t kInlineSpread = 2 * 152;
+__host__ __device__ __forceinline__ bool inline_spread(int64_t nlinked) { return nlinked <= kInlineSpread; }
+
+template <class L, class P, bool MULTI, int BT>
+__global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inline(
+    const typename P::T* __restrict__ fin, typename P::T* __restrict__ fout, Layout lay,
+    FusedLinks<typename P::T> fl, const Mom4<typename P::T>* __restrict__ mom_in,
+    Mom4<typename P::T>* __restrict__ mom_out, double* __restrict__ force, double* __restrict__ force_next,
+    Params p) {
   using T = typename P::T;
-  // threads 0 .. ny-1: inlet rows; ny .. 2 ny - 1: outlet rows
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 2 * p.ny) return;
-  const bool inlet_side = t < p.ny;
-  const int y = inlet_side ? t : t - p.ny;
+  constexpr int NW = BT / 32, NF = inline_free_groups<P>();
+  let_next_start();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const size_t S = (size_t)lay.S;
-  if (inlet_side && p.inlet) {
-    // the inflow velocity does not depend on the row's storage: issued first
-    const T uin = (T)inlet_velocity(p, lay, y);
-    const int32_t k0 = lay.row_first[y];
-    if (k0 >= 0 && (lay.word[k0] & W_OPEN)) {
-      const uint32_t k1 = (uint32_t)k0 + 1;
-      const Mom4<T> m1 = mom[k1];
-      const T rho1 = P::shifted ? par<T>(p.rho0, p.rho0_f) + m1.r : m1.r;
-      T v[L::Q];
+  const bool spread = inline_spread(lay.nlinked);
+  const int64_t nlb = spread ? lay.nlinked : (lay.nlinked + NW - 1) / NW;  // blocks with links
+  if ((int64_t)blockIdx.x >= nlb) {
+    const int64_t at = lay.nlinked + (((int64_t)blockIdx.x - nlb) * NW + warp) * NF;
+    uint32_t k[NF];
+    bool live[NF];
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) v[i] = f[i * S + k1];
-#pragma unroll
-      for (int i = 0; i < L::Q; ++i)
-        f[i * S + k0] = equilibrium<L, P>(i, m1.r, rho1, uin, (T)0, (T)0) +
-                        (v[i] - equilibrium<L, P>(i, m1.r, rho1, m1.ux, m1.uy, (T)0));
+    for (int j = 0; j < NF; ++j) {
+      k[j] = at + j < lay.ngroups ? 32u * __ldg(lay.groups + at + j) + lane : 0u;
+      live[j] = at + j < lay.ngroups && (uint64_t)k[j] < S;
+    }
+    bulk_nodes<L, P, MULTI, NF>(k, live, fin, fout, lay, mom_out, p);
+    clear_force<BT>(force_next, p.nbody);
+    return;
+  }
+  __shared__ T stage[NW][L::Q][32];
+  __shared__ double red[2][NW];
+  __shared__ int rbody[NW];
+  const int64_t at = spread ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * NW + warp;
+  const bool some = at < lay.nlinked;
+  // spread: the first warp holds the group's nodes, the others its links
+  const bool mine = !spread || warp == 0;
+  const int first = spread ? (int)threadIdx.x - 32 : lane, step = spread ? BT - 32 : 32;
+  const uint32_t g = some ? __ldg(lay.groups + at) : 0u;
+  const uint32_t k = 32u * g + lane;
+  const bool live = some && (uint64_t)k < S;
+  const int64_t l0 = some ? __ldg(fl.first + g) : 0, l1 = some ? __ldg(fl.first + g + 1) : 0;
+  FusedRec r{0, 0, 0, 0};
+  if (first >= 0 && l0 + first < l1) r = fl.rec[l0 + first];
+  const uint32_t w = live ? __ldg(lay.word + k) : W_GHOST;
+  const uint32_t mask = live ? __ldg(fl.mask + k) : 0u;
+  const bool fluid = !(w & (W_GHOST | W_OPEN));
+  T f[L::Q];
+  int dom = 0;
+  RunRec run{};
+  if (fluid && mine) run = lay.runs[w & W_RUN];
+  dom = run.dom;
+  wait_for_previous();
+  clear_force<BT>(force_next, p.nbody);
+  auto pull = [&] {
+    if (fluid && mine) pull_node<L>(fin, S, k, run, lay, p, f);
+  };
+  if (P::shifted || spread) pull();  // (else FP64: after the links, whose registers it would spill)
+  T(&col)[L::Q][32] = stage[spread ? 0 : warp];
+  // forces are summed for the body of the warp's first link
+  const int wb = (int)(__shfl_sync(0xffffffffu, r.meta, 0) >> 8) - 1;
+  LinkForce<T> F;
+  for (int64_t li = first < 0 ? l1 : l0 + first; li < l1; li += step) {
+    if (li != l0 + first) r = fl.rec[li];
+    const T q = P::shifted ? (T)__uint_as_float(r.q32) : (T)__ldg(fl.qd + li);
+    const int ip = (int)(r.meta & 31), rule = (int)((r.meta >> 5) & 7), body = (int)(r.meta >> 8) - 1;
+    const int i = (int)(d2q9_opposites() >> (4 * ip)) & 15;
+    const int ex = (int)((d2q9_pack(false) >> (2 * ip)) & 3) - 1, ey = (int)((d2q9_pack(true) >> (2 * ip)) & 3) - 1;
+    auto real = [](int e) { return e == 0 ? (T)0 : (e > 0 ? (T)1 : (T)-1); };
+    const DirVal<T> dir{ip < 5 ? (T)L::w(1) : (T)L::w(5), real(ex), real(ey), (T)0, {ex, ey, 0}};
+    T uw0 = 0, uw1 = 0;
+    if (fl.uw) {
+      uw0 = fl.uw[li];
+      uw1 = fl.uw[fl.nl + li];
+    }
+    T fpf;
+    const T val = eval_link<L, P>(dir, ip, i, fin, mom_in, S, rule, q, r.kf, r.kff, uw0, uw1, (T)0, p, fpf,
+                                  fl.uw != nullptr, fl.wq + li, fl.nl);
+    col[i][r.kf & 31] = val;
+    if (body >= 0) {
+      // momentum exchange as in k_links
+      const T t = fpf + val;
+      auto direct = [&] { add_force(force, body, t, dir); };
+      if (body == wb)
+        F.add(t, dir, p.kx, direct);
+      else
+        direct();
     }
   }
-  if (!inlet_side && p.outlet) {
-    const int32_t kl = lay.row_last[y];
-    if (kl >= 0 && (lay.word[kl] & W_OPEN)) {
-      T v[L::Q];
+  if (!P::shifted && !spread) pull();
+  if (spread)
+    __syncthreads();
+  else
+    __syncwarp();
+  // the populations of v that come from a wall
+  auto take = [&](T(&v)[L::Q]) {
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) v[i] = f[i * S + kl - 1];
+    for (int i = 1; i < L::Q; ++i)
+      if ((mask >> L::opp(i)) & 1u) v[i] = col[i][lane];
+  };
+  if (mask && mine) take(f);
+  if (live && mine && !(w & W_OPEN)) {
+    // ghost slots: zeros through the same stores (inputs at rest)
+    auto rest = [&](T(&v)[L::Q]) {
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) f[i * S + kl] = v[i];
+      for (int i = 0; i < L::Q; ++i) v[i] = P::shifted ? (T)0 : (T)L::w(i);
+    };
+    if (!fluid) rest(f);
+    collide_node<L, P, MULTI>(f, p, lay, dom, fout, S, k, mom_out, (w & W_CACHE) != 0, fluid, [&](T(&v)[L::Q]) {
+      if (!fluid) return rest(v);
+      pull_node<L>(fin, S, k, lay.runs[w & W_RUN], lay, p, v);
+      take(v);
+    });
+    if (fluid && (p.inlet | p.outlet)) open_ends<L, P>(fout, mom_out, S, k, lay.runs[w & W_RUN], lay, p);
+  }
+  if (wb >= 0) F.reduce();
+  if (lane == 0) {
+    red[0][warp] = F.value(0, p.kx);
+    red[1][warp] = F.value(1, p.kx);
+    rbody[warp] = wb;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    // one atomic per run of warps with one body
+    double acc = 0.0;
+#pragma unroll 1
+    for (int wi = 0; wi < NW; ++wi) {
+      const int b = rbody[wi];
+      acc += red[threadIdx.x][wi];
+      if (b >= 0 && (wi == NW - 1 || rbody[wi + 1] != b)) {
+        atomicAdd(&force[3 * b + threadIdx.x], acc);
+        acc = 0.0;
+      }
     }
   }
 }
@@ -1531,6 +1776,7 @@ struct FusedRaw {
   const FusedRec* rec;
   const double* qd;
   const void* uw;
+  const int64_t* wq;
   int64_t nl, ngroups;
 };
 
@@ -1543,7 +1789,7 @@ struct KernelOps {
   // 256); seq: links per thread of the link kernel (1 or 4)
   void (*bulk)(const void* fin, void* fout, const Layout& lay, void* mom, double* force_next, const Params& p,
                int shape, cudaStream_t s);
-  void (*links)(void* f, const void* mom, const LinkRec* recs, const void* q, const void* uw, const void* qc,
+  void (*links)(void* f, const void* mom, const LinkRec* recs, const void* q, const void* uw, const int64_t* wq,
                 int64_t nl, double* force, const Params& p, int64_t S, int threads, int seq, cudaStream_t s);
   // fused step (threads per block 128, 256 or 512; 512 runs as 256 for
   // FP64 D3Q19, whose link buffer would not fit the static shared memory)
@@ -1563,6 +1809,22 @@ struct KernelOps {
 
 inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
+// Launch of a step kernel that may start before its predecessor in the stream
+// has ended (it waits by itself).
+template <class... K, class... A>
+inline void launch_early(void (*kernel)(K...), unsigned grid, int block, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = s;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, (K)args...);
+}
+
 template <class L, class P>
 struct Launch {
   using T = typename P::T;
@@ -1571,19 +1833,19 @@ struct Launch {
                          const Params& p, cudaStream_t s) {
     if constexpr (!P::shifted && NPT == 1) {
       if (lay.fluid) {
-        k_bulk_list<L, P, M, BT><<<blocks_for(lay.nfluid > 0 ? lay.nfluid : 1, BT), BT, 0, s>>>(
-            (const T*)fin, (T*)fout, lay, (Mom4<T>*)mom, force_next, p);
+        launch_early(k_bulk_list<L, P, M, BT>, blocks_for(lay.nfluid > 0 ? lay.nfluid : 1, BT), BT, s, (const T*)fin,
+                     (T*)fout, lay, (Mom4<T>*)mom, force_next, p);
         return;
       }
     }
-    k_bulk<L, P, M, BT, NPT><<<blocks_for((lay.S + NPT - 1) / NPT, BT), BT, 0, s>>>((const T*)fin, (T*)fout, lay,
-                                                                                   (Mom4<T>*)mom, force_next, p);
+    launch_early(k_bulk<L, P, M, BT, NPT>, blocks_for((lay.S + NPT - 1) / NPT, BT), BT, s, (const T*)fin, (T*)fout, lay,
+                 (Mom4<T>*)mom, force_next, p);
   }
   template <bool M, int BT, int SEQ>
   static void bulk_seq(const void* fin, void* fout, const Layout& lay, void* mom, double* force_next,
                        const Params& p, cudaStream_t s) {
-    k_bulk_seq<L, P, M, BT, SEQ><<<blocks_for((lay.S + SEQ - 1) / SEQ, BT), BT, 0, s>>>(
-        (const T*)fin, (T*)fout, lay, (Mom4<T>*)mom, force_next, p);
+    launch_early(k_bulk_seq<L, P, M, BT, SEQ>, blocks_for((lay.S + SEQ - 1) / SEQ, BT), BT, s, (const T*)fin, (T*)fout,
+                 lay, (Mom4<T>*)mom, force_next, p);
   }
   template <bool M>
   static void bulk_m(const void* fin, void* fout, const Layout& lay, void* mom, double* fn, const Params& p,
@@ -1613,24 +1875,30 @@ struct Launch {
     else
       bulk_m<false>(fin, fout, lay, mom, force_next, p, shape, s);
   }
-  static void links(void* f, const void* mom, const LinkRec* recs, const void* q, const void* uw, const void* qc,
+  static void links(void* f, const void* mom, const LinkRec* recs, const void* q, const void* uw, const int64_t* wq,
                     int64_t nl, double* force, const Params& p, int64_t S, int threads, int seq, cudaStream_t s) {
     if (nl == 0) return;
     const int bt = (threads == 64 || threads == 128) ? threads : 256;
     if (seq == 4)
-      k_links<L, P, 4><<<blocks_for(nl, 4 * bt), bt, 0, s>>>((T*)f, (const Mom4<T>*)mom, recs, (const T*)q,
-                                                             (const T*)uw, (const T*)qc, nl, force, p, S);
+      launch_early(k_links<L, P, 4>, blocks_for(nl, 4 * bt), bt, s, (T*)f, (const Mom4<T>*)mom, recs, (const T*)q,
+                   (const T*)uw, wq, nl, force, p, S);
     else
-      k_links<L, P, 1><<<blocks_for(nl, bt), bt, 0, s>>>((T*)f, (const Mom4<T>*)mom, recs, (const T*)q,
-                                                         (const T*)uw, (const T*)qc, nl, force, p, S);
+      launch_early(k_links<L, P, 1>, blocks_for(nl, bt), bt, s, (T*)f, (const Mom4<T>*)mom, recs, (const T*)q,
+                   (const T*)uw, wq, nl, force, p, S);
   }
   template <bool M, int BT>
   static void fused_shape(const void* fin, void* fout, const Layout& lay, const FusedRaw& r, const void* mom_in,
                           void* mom_out, double* force, double* force_next, const Params& p, cudaStream_t s) {
-    const FusedLinks<T> fl{r.first, r.mask, r.rec, r.qd, (const T*)r.uw, r.nl, r.ngroups};
-    k_fused<L, P, M, BT><<<blocks_for(lay.S, BT), BT, 0, s>>>((const T*)fin, (T*)fout, lay, fl,
-                                                              (const Mom4<T>*)mom_in, (Mom4<T>*)mom_out, force,
-                                                              force_next, p);
+    const FusedLinks<T> fl{r.first, r.mask, r.rec, r.qd, (const T*)r.uw, r.wq, r.nl, r.ngroups};
+    if constexpr (L::Q == 9) {
+      const int64_t nw = BT / 32, nf = inline_free_groups<P>();
+      const int64_t nb = (inline_spread(lay.nlinked) ? lay.nlinked : (lay.nlinked + nw - 1) / nw) + (lay.ngroups - lay.nlinked + nw * nf - 1) / (nw * nf);
+      launch_early(k_inline<L, P, M, BT>, (unsigned)nb, BT, s, (const T*)fin, (T*)fout, lay, fl,
+                   (const Mom4<T>*)mom_in, (Mom4<T>*)mom_out, force, force_next, p);
+    } else {
+      launch_early(k_fused<L, P, M, BT>, blocks_for(lay.S, BT), BT, s, (const T*)fin, (T*)fout, lay, fl,
+                   (const Mom4<T>*)mom_in, (Mom4<T>*)mom_out, force, force_next, p);
+    }
   }
   template <bool M>
   static void fused_m(const void* fin, void* fout, const Layout& lay, const FusedRaw& r, const void* mom_in,

@@ -118,7 +118,7 @@ struct lbm_lattice_s {
   // state over stored nodes: f[c] and its moment cache mom[c]
   DeviceBuf f[2], mom[2];
   // layout
-  DeviceBuf word, node_of, tile, runs, row_first, row_last, row_in1, row_out1;
+  DeviceBuf word, node_of, tile, row_uin, groups, runs, row_first, row_last, row_in1, row_out1;
   Layout lay{};
   // batch: domains along the last axis (empty: one domain run by cfg)
   std::vector<lbm_domain> domains;
@@ -131,7 +131,9 @@ struct lbm_lattice_s {
   // links of the fused step kernel, in (node, dir) order (FusedLinks)
   DeviceBuf lfirst, lmask, lrec, lqd, luw;
   DeviceBuf fidx;  // FP64: storage indices of the fluid nodes (the bulk pass's thread map)
-  DeviceBuf lqc;   // FP64: per-link VIBB velocity weights [3][n_links] in the link kernel's order
+  // FP64: VIBB velocity weights [3][n_links] in the link kernel's order, and in
+  // the fused kernel's where that is another one
+  DeviceBuf lqc, lqf;
   int64_t n_links = 0, n_fluid = 0, n_cached = 0, n_runs = 0;
   DeviceBuf force;  // [2][nbody][3]
   // shifted storage: sum over each body's links of 2 w_i' rho0 e_i' (FP64),
@@ -162,10 +164,10 @@ struct lbm_lattice_s {
 namespace {
 
 int64_t device_bytes(const lbm_handle h) {
-  const DeviceBuf* all[] = {&h->f[0],     &h->f[1],     &h->mom[0],   &h->mom[1], &h->word,  &h->node_of, &h->tile,
+  const DeviceBuf* all[] = {&h->f[0],     &h->f[1],     &h->mom[0],   &h->mom[1], &h->word,  &h->node_of, &h->tile, &h->row_uin, &h->groups,
                             &h->runs,     &h->row_first, &h->row_last, &h->row_in1, &h->row_out1, &h->recs,
                             &h->q,        &h->uw,       &h->lfirst, &h->lmask, &h->lrec,
-                            &h->lqd,      &h->luw,      &h->force,    &h->dom,    &h->row_dom, &h->fidx, &h->lqc};
+                            &h->lqd,      &h->luw,      &h->force,    &h->dom,    &h->row_dom, &h->fidx, &h->lqc, &h->lqf};
   int64_t s = 0;
   for (auto* b : all) s += (int64_t)b->bytes;
   return s;
@@ -218,10 +220,10 @@ void drop_graphs(lbm_handle h) {
 }
 
 void release_geometry(lbm_handle h) {
-  DeviceBuf* all[] = {&h->f[0],     &h->f[1],      &h->mom[0],   &h->mom[1], &h->word,  &h->node_of, &h->tile,
+  DeviceBuf* all[] = {&h->f[0],     &h->f[1],      &h->mom[0],   &h->mom[1], &h->word,  &h->node_of, &h->tile, &h->row_uin, &h->groups,
                       &h->runs,     &h->row_first, &h->row_last, &h->row_in1, &h->row_out1, &h->recs,
                       &h->q,        &h->uw,        &h->lfirst, &h->lmask, &h->lrec,
-                      &h->lqd,      &h->luw,       &h->dom,      &h->row_dom, &h->fidx, &h->lqc};
+                      &h->lqd,      &h->luw,       &h->dom,      &h->row_dom, &h->fidx, &h->lqc, &h->lqf};
   for (auto* b : all) release(*b);
   h->lay = Layout{};
 }
@@ -247,7 +249,8 @@ void fold_all(lbm_handle h) {
 // the link rules run inside the pull pass (k_fused; mn must differ from mc),
 // else the link kernel writes the ghost slots of fc and the bulk kernel
 // pulls them (mn may equal mc: the link kernel reads mc before the bulk
-// kernel writes it).
+// kernel writes it).  fc's open columns are filled, and so are fn's after it
+// (by the threads of the nodes beside them).
 lbm_status enqueue_step_buf(lbm_handle h, void* fc, void* fn, void* mc, void* mn, double* slot, double* next,
                             bool timed, bool fused);
 
@@ -296,18 +299,15 @@ lbm_status enqueue_step_buf(lbm_handle h, void* fc, void* fn, void* mc, void* mn
   lbm_status st;
   if (!fused) {
     st = timed_launch(0, [&] {
-      h->ops.links(fc, mc, (const LinkRec*)h->recs.p, h->q.p, h->uw.p, h->lqc.p, h->n_links, slot, h->p, h->lay.S,
+      h->ops.links(fc, mc, (const LinkRec*)h->recs.p, h->q.p, h->uw.p, (const int64_t*)h->lqc.p, h->n_links, slot, h->p, h->lay.S,
                    h->tune.link_threads, h->tune.link_seq, h->stream);
     });
     if (st != LBM_OK) return st;
   }
-  if (h->p.inlet || h->p.outlet) {
-    st = timed_launch(1, [&] { h->ops.open(fc, mc, h->lay, h->p, h->stream); });
-    if (st != LBM_OK) return st;
-  }
   if (fused) {
     const FusedRaw fl{(const int32_t*)h->lfirst.p, (const uint32_t*)h->lmask.p, (const FusedRec*)h->lrec.p,
-                      (const double*)h->lqd.p, h->luw.p, h->n_links, (h->lay.S + 31) / 32};
+                      (const double*)h->lqd.p, h->luw.p,
+                      (const int64_t*)(h->lqf.p ? h->lqf.p : h->lqc.p), h->n_links, (h->lay.S + 31) / 32};
     st = timed_launch(2, [&] {
       h->ops.fused(fc, fn, h->lay, fl, mc, mn, slot, next, h->p, fused_threads(h), h->stream);
     });
@@ -443,6 +443,12 @@ lbm_status lbm_create_lattice(const lbm_config* cfg, lbm_handle* out) {
   for (int a = 0; a < 3; ++a) p.periodic[a] = c.periodic[a] ? 1 : 0;
   p.nbody = 1;
   h->tune.bulk_shape = h->ops.default_shape;
+  if (h->rb == 8 && h->Q == 19) {
+    // the FP64 link rule's registers take the fused kernel's warps (200^3 pack
+    // 0.87 ms fused, 0.68 ms with 64-thread link blocks and the bulk pass)
+    h->tune.fused = 0;
+    h->tune.link_threads = 64;
+  }
 
   if (c.cuda_stream) {
     h->stream = (cudaStream_t)c.cuda_stream;
@@ -904,6 +910,12 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
             }
         rec.dbase[sl] = base - sidx[n];
       }
+      if (D == 2) {
+        // open ends (see RunRec)
+        const int64_t xo = rwidth[r] - 1;
+        if (c.inlet && x == 1 && (m[nx * r] & H_OPEN)) rec.dbase[2] |= 1;
+        if (c.outlet && xe == xo - 1 && (m[nx * r + xo] & H_OPEN)) rec.dbase[2] |= 2 | (int32_t)(xe << 2);
+      }
       if (out) {
         const uint32_t rid = rid0 + (uint32_t)count;
         for (int64_t xx = x; xx <= xe; ++xx) {
@@ -1048,33 +1060,23 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
       split_rec(j, k, (uint32_t)sidx[links[k].node], (uint32_t)sidx[lk_ff[k]]);
     }
   }
-  // FP64: the VIBB velocity weights of each link in the link kernel's order
-  // (u*_d's and u**_d's weights of Sec. 3.1 blended 1/3 : 2/3; q alone
-  // fixes them)
-  raw_vec<double> qcw(h->rb == 8 ? 3 * (size_t)n_links : 0);
-  if (h->rb == 8) {
+  // FP64: the VIBB velocity weights of each link (u*_d's and u**_d's weights
+  // of Sec. 3.1 blended 1/3 : 2/3; q alone fixes them) in 2^-62, in the link
+  // kernel's order and, where it is another, in the fused kernel's
+  auto weights = [&](const int64_t* ord) {
+    raw_vec<int64_t> w(3 * (size_t)n_links);
 #pragma omp parallel for schedule(static)
     for (int64_t j = 0; j < n_links; ++j) {
-      const double q = links[order[j]].q, two_q = 2.0 * q;
-      double af, aff, aw;
-      if (q <= 0.5) {
-        af = two_q;
-        aff = 1.0 - two_q;
-        aw = 0.0;
-      } else {
-        const double iq = 1.0 / q;
-        af = (1.0 - q) * iq;
-        aff = 0.0;
-        aw = (two_q - 1.0) * iq;
-      }
-      const double i1q = 1.0 / (1.0 + q);
-      const double bff = (1.0 - q) * i1q, bw = two_q * i1q;
-      const double third = 1.0 / 3.0, two_thirds = 2.0 / 3.0;
-      qcw[j] = third * af;
-      qcw[n_links + j] = third * aff + two_thirds * bff;
-      qcw[2 * n_links + j] = third * aw + two_thirds * bw;
+      const double q = links[ord[j]].q, two_q = 2.0 * q, i1q = 1.0 / (1.0 + q);
+      const double af = q <= 0.5 ? two_q : (1.0 - q) / q, aff = q <= 0.5 ? 1.0 - two_q : 0.0;
+      const double aw = q <= 0.5 ? 0.0 : (two_q - 1.0) / q;
+      const double third = 1.0 / 3.0, unit = 0x1p62;
+      w[j] = (int64_t)std::llrint(third * af * unit);
+      w[n_links + j] = (int64_t)std::llrint((third * aff + 2.0 * third * (1.0 - q) * i1q) * unit);
+      w[2 * n_links + j] = (int64_t)std::llrint((third * aw + 2.0 * third * two_q * i1q) * unit);
     }
-  }
+    return w;
+  };
   // first link of each 32-node group: storage indices of x_f are
   // non-decreasing along (node, dir) order, so ffirst[g] (the first j with
   // kf_j >= 32 g) is j for every g in (kf_{j-1} / 32, kf_j / 32], and n_links
@@ -1088,6 +1090,29 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
     const int64_t glast = n_links > 0 ? (int64_t)(frec[n_links - 1].kf >> 5) : -1;
 #pragma omp parallel for schedule(static)
     for (int64_t t = glast + 1; t <= ngroups; ++t) ffirst[t] = (int32_t)n_links;
+  }
+
+  // D2Q9: the groups with links, then the others (k_inline)
+  raw_vec<uint32_t> groups(D == 2 && n_links > 0 ? (size_t)ngroups : 0);
+  int64_t nlinked = 0;
+  for (int pass = 0, at = 0; pass < 2 && !groups.empty(); ++pass) {
+    for (int64_t t = 0; t < ngroups; ++t)
+      if ((ffirst[t + 1] > ffirst[t]) == (pass == 0)) groups[at++] = (uint32_t)t;
+    if (pass == 0) nlinked = at;
+  }
+  // inlet velocity of every row, y counted from the first row of its domain
+  std::vector<double> uin(c.inlet ? (size_t)rows : 0);
+  for (int64_t r = 0; r < (int64_t)uin.size(); ++r) {
+    double umax = c.inlet_umax, y0 = c.inlet_y0, y1 = c.inlet_y1, yy = (double)r;
+    if (ndom > 0) {
+      const lbm_domain& q = h->domains[rdom[r]];
+      umax = q.inlet_umax;
+      y0 = q.inlet_y0;
+      y1 = q.inlet_y1;
+      yy = (double)(r - (ndom > 1 ? q.lo : 0));
+    }
+    const double hh = y1 - y0;
+    uin[r] = 4.0 * umax * (yy - y0) * (y1 - yy) / (hh * hh);
   }
 
   // ---- device
@@ -1113,7 +1138,10 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   if (st == LBM_OK) st = upload(h->lrec, frec.data(), sizeof(FusedRec) * n_links);
   if (st == LBM_OK) st = upload(h->lqd, fq.data(), sizeof(double) * fq.size());
   if (st == LBM_OK && nflist > 0) st = upload(h->fidx, flist.data(), sizeof(uint32_t) * nflist);
-  if (st == LBM_OK && h->rb == 8 && n_links > 0) st = upload(h->lqc, qcw.data(), sizeof(double) * 3 * n_links);
+  if (st == LBM_OK && h->rb == 8 && n_links > 0) {
+    st = upload(h->lqc, weights(order.data()).data(), sizeof(int64_t) * 3 * n_links);
+    if (st == LBM_OK && !same_order) st = upload(h->lqf, weights(ond).data(), sizeof(int64_t) * 3 * n_links);
+  }
   if (st == LBM_OK && ndom > 0) {
     std::vector<DomPar> dp(ndom);
     for (int k = 0; k < ndom; ++k) {
@@ -1161,6 +1189,8 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
       return upload(b, t.data(), 4 * t.size());
     };
     st = put(h->q, qs);
+    if (st == LBM_OK && !uin.empty()) st = put(h->row_uin, raw_vec<double>(uin.begin(), uin.end()));
+    if (st == LBM_OK && !groups.empty()) st = upload(h->groups, groups.data(), sizeof(uint32_t) * groups.size());
     if (st == LBM_OK && moving) st = put(h->uw, uws);
     if (st == LBM_OK && moving) st = put(h->luw, fuw);
   }
@@ -1187,6 +1217,10 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   h->lay.ndom = std::max(ndom, 1);
   h->lay.fluid = nflist > 0 ? (const uint32_t*)h->fidx.p : nullptr;
   h->lay.nfluid = nflist;
+  h->lay.row_uin = h->row_uin.p;
+  h->lay.groups = (const uint32_t*)h->groups.p;
+  h->lay.nlinked = nlinked;
+  h->lay.ngroups = ngroups;
   // a single domain runs through Params like an unsplit lattice
   Params& p = h->p;
   const lbm_domain one{0, 0, 0, 0, c.tau, {c.g[0], c.g[1], c.g[2]}, c.inlet_umax, c.inlet_y0, c.inlet_y1};
@@ -1233,6 +1267,7 @@ lbm_status lbm_init_equilibrium(lbm_handle h, const double* rho, const double* u
   if (e == cudaSuccess && h->mom[0].bytes) e = cudaMemsetAsync(h->mom[0].p, 0, h->mom[0].bytes, h->stream);
   if (e == cudaSuccess) {
     h->ops.init(h->f[0].p, h->mom[0].p, h->lay, drho, du, h->p, h->stream);
+    if (h->p.inlet || h->p.outlet) h->ops.open(h->f[0].p, h->mom[0].p, h->lay, h->p, h->stream);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(h->force.p, 0, h->force.bytes, h->stream);
@@ -1450,6 +1485,7 @@ lbm_status lbm_set_distributions(lbm_handle h, const double* f) {
   }
   if (e == cudaSuccess) {
     h->ops.refresh(h->f[h->cur].p, h->lay, h->mom[h->cur].p, h->p, h->stream);
+    if (h->p.inlet || h->p.outlet) h->ops.open(h->f[h->cur].p, h->mom[h->cur].p, h->lay, h->p, h->stream);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -1606,8 +1642,8 @@ lbm_status lbm_adjoint_step(lbm_handle h, int32_t body, const double dJ_dF[3], i
   // moments stay as they are)
   void* am = h->mom[h->cur ^ 1].p;
   // the states f+(s0) .. f+(s0 + m - 1) of a segment from its first state
-  // (copied into seg[0]); the link and open kernels leave the link values
-  // of step s0 + j in the ghost slots of seg[j] for j < m - 1
+  // (copied into seg[0], its open columns filled); the link kernel leaves the
+  // link values of step s0 + j in the ghost slots of seg[j] for j < m - 1
   auto enqueue_recompute = [&](int64_t m) -> lbm_status {
     h->ops.refresh(segp, h->lay, am, h->p, h->stream);
     for (int64_t j = 0; j + 1 < m; ++j) {
@@ -1629,9 +1665,8 @@ lbm_status lbm_adjoint_step(lbm_handle h, int32_t body, const double dJ_dF[3], i
         // cache holds the moments the recompute's last step wrote for it,
         // those its forward step used (a one-state segment: the refresh of
         // the recompute)
-        h->ops.links(state, am, (const LinkRec*)h->recs.p, h->q.p, h->uw.p, h->lqc.p, nl, fslot, h->p, S,
+        h->ops.links(state, am, (const LinkRec*)h->recs.p, h->q.p, h->uw.p, (const int64_t*)h->lqc.p, nl, fslot, h->p, S,
                      h->tune.link_threads, h->tune.link_seq, h->stream);
-        if (open) h->ops.open(state, am, h->lay, h->p, h->stream);
       }
       h->adj.bulk(state, lam[l].p, lam[l ^ 1].p, h->lay, h->p, dtau, am, h->stream);
       if (open)

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kBlock) k_force_partial(const double* __restri
     }
     const int rule = lk.bc >= 0 ? lk.bc : default_rule;
     const double fpf = f[ip * N + node];
-    const double val = lbm::link_value<P>(rule, lk.q, tab.w[ip], ex, ey, ez, fpf, f[ip * N + ff], f[i * N + node], m[0],
+    const double val = lbm::link_value<P>(rule, lk.q, lbm::DirVal<double>{tab.w[ip], ex, ey, ez, {}}, fpf, f[ip * N + ff], f[i * N + node], m[0],
                                           m[1], lk.uw[0], lk.uw[1], L::D == 3 ? lk.uw[2] : 0.0, p.rho0,
                                           p.vibb_local_rho);
     const double t = fpf + val;
