@@ -35,7 +35,8 @@ namespace lbm {
 constexpr double kFixedMaxForce = 1.0 / 512;
 
 __host__ __device__ __forceinline__ Halves halves(int64_t v) {
-  return Halves{(int32_t)(((uint64_t)v + 0x80000000ull) >> 32), (int32_t)(uint32_t)(uint64_t)v};
+  const uint32_t lo = (uint32_t)(uint64_t)v;
+  return Halves{(int32_t)((uint32_t)((uint64_t)v >> 32) + (lo >> 31)), (int32_t)lo};
 }
 
 // Fills the constants for stencil L; collision 1 is MRT (D2Q9).
@@ -147,11 +148,14 @@ __device__ __forceinline__ int64_t reciprocal_grid(uint64_t r) {
   return (int64_t)(((uint64_t)__funnelshift_r(mh, 0u, n) << 32) | __funnelshift_r(lo << 10, mh, n));
 }
 
-// 0 if v, as a signed number, lies in [-2^B, 2^B), B > 32.
+// Checks that signed numbers lie in [-2^B, 2^B), B > 32: the upper words moved
+// into [0, 2^(B - 31)) are or-ed together and looked at once.
 template <int B>
-__device__ __forceinline__ uint32_t beyond(uint64_t v) {
-  return ((uint32_t)(v >> 32) + (1u << (B - 32))) >> (B - 31);
-}
+struct Within {
+  uint32_t seen = 0;
+  __device__ __forceinline__ void operator()(uint64_t v) { seen |= (uint32_t)(v >> 32) + (1u << (B - 32)); }
+  __device__ __forceinline__ bool broken() const { return (seen >> (B - 31)) != 0u; }
+};
 
 // rho and u of a node: r in grid steps, u in 2^-60.
 struct NodeMom {
@@ -191,16 +195,24 @@ __device__ __forceinline__ bool collide_grid(double (&f)[9], const FixedK& k, bo
     jy += (uint64_t)k.hg[1];
   }
   // |X|, |Y| < 1/4, Sd < 1/2, |j| < 1/2
-  wide = beyond<60>(X) | beyond<60>(Y) | (uint32_t)(Sd >> 61) | beyond<61>(jx) | beyond<61>(jy) | beyond_rho(r);
+  Within<60> quarter;
+  Within<61> half;
+  quarter(X);
+  quarter(Y);
+  half(jx);
+  half(jy);
+  wide = (uint32_t)(Sd >> 61) | beyond_rho(r);
   const Halves inv = halves(reciprocal_grid(r));
   const Halves hx = halves((int64_t)(2 * jx)), hy = halves((int64_t)(2 * jy));
   const int64_t ux = mul_grid<0>(hx, inv), uy = mul_grid<0>(hy, inv);  // 2^-60
-  wide |= beyond<59>((uint64_t)ux) | beyond<59>((uint64_t)uy);         // |u| < 1/2
+  Within<59> slow;  // |u| < 1/2
+  slow((uint64_t)ux);
+  slow((uint64_t)uy);
   const Halves vx = halves(ux), vy = halves(uy);
   // rho u u in 2^-62: 2 j in 2^-62 times u in 2^-60 over 2^61
   const int64_t qxx = mul_grid<3>(hx, vx), qyy = mul_grid<3>(hy, vy), qxy = mul_grid<3>(hx, vy);
   const int64_t E = qxx + qyy;
-  wide |= beyond<60>((uint64_t)E);
+  quarter((uint64_t)E);
   const int64_t ne = -(int64_t)(2 * X + Y) - 3 * E;
   int64_t De = mul_grid<0>(halves(ne), k.c[0]), Dp = mul_grid<0>(halves((int64_t)X + E), k.c[1]);
   int64_t Dx = mul_grid<0>(halves((int64_t)(2 * bx - d13)), k.c[2]);
@@ -240,7 +252,7 @@ __device__ __forceinline__ bool collide_grid(double (&f)[9], const FixedK& k, bo
 #pragma unroll
   for (int i = 0; i < 9; ++i) f[i] = from_grid<true>(F[i], k.sc, out);
   m = NodeMom{r, ux, uy, 0};
-  return bad < 32u && wide == 0u && (int32_t)out >= 0;
+  return bad < 32u && wide == 0u && !(quarter.broken() || half.broken() || slow.broken()) && (int32_t)out >= 0;
 }
 
 // D3Q19 BGK: f+_i = (1 - omega) f_i + omega feq_i + src_i.  In units of a
@@ -271,11 +283,18 @@ __device__ __forceinline__ bool collide_grid(double (&f)[19], const FixedK& k, b
     jy += (uint64_t)k.hg[1];
     jz += (uint64_t)k.hg[2];
   }
-  wide = beyond_rho(r) | beyond<61>(jx) | beyond<61>(jy) | beyond<61>(jz);  // |j| < 1/2
+  wide = beyond_rho(r);
+  Within<61> half;  // |j| < 1/2
+  half(jx);
+  half(jy);
+  half(jz);
   const Halves inv = halves(reciprocal_grid(r));
   const Halves hx = halves((int64_t)(2 * jx)), hy = halves((int64_t)(2 * jy)), hz = halves((int64_t)(2 * jz));
   const int64_t ux = mul_grid<0>(hx, inv), uy = mul_grid<0>(hy, inv), uz = mul_grid<0>(hz, inv);  // 2^-60
-  wide |= beyond<59>((uint64_t)ux) | beyond<59>((uint64_t)uy) | beyond<59>((uint64_t)uz);         // |u| < 1/2
+  Within<59> slow;  // |u| < 1/2
+  slow((uint64_t)ux);
+  slow((uint64_t)uy);
+  slow((uint64_t)uz);
   const Halves vx = halves(ux), vy = halves(uy), vz = halves(uz);
   // 2 (omega/8) j; T in 2^-62: that times u in 2^-60 over 2^61
   int64_t Wx = mul_grid<0>(hx, k.c[0]), Wy = mul_grid<0>(hy, k.c[0]), Wz = mul_grid<0>(hz, k.c[0]);
@@ -294,7 +313,8 @@ __device__ __forceinline__ bool collide_grid(double (&f)[19], const FixedK& k, b
     Syz += 2 * (mul_grid<4>(vy, k.ge[2]) + mul_grid<4>(vz, k.ge[1]));
   }
   const int64_t tr = Txx + Tyy + Tzz;
-  wide |= beyond<57>((uint64_t)tr);  // (omega/8) rho u.u below 2^-5
+  Within<57> small;  // (omega/8) rho u.u below 2^-5
+  small((uint64_t)tr);
   const uint64_t B = (uint64_t)(mul_grid<0>(halves((int64_t)r), k.c[2]) - mul_grid<0>(halves(tr), k.c[3]));
   uint32_t out = 0;
   auto put = [&](int i, uint64_t c) {
@@ -326,7 +346,7 @@ __device__ __forceinline__ bool collide_grid(double (&f)[19], const FixedK& k, b
   pair(15, Byz + (uint64_t)Syz, my + mz);
   pair(17, Byz - (uint64_t)Syz, my - mz);
   m = NodeMom{r, ux, uy, uz};
-  return bad < 32u && wide == 0u && (int32_t)out >= 0;
+  return bad < 32u && wide == 0u && !(half.broken() || slow.broken() || small.broken()) && (int32_t)out >= 0;
 }
 
 // v (|v| < 1/2, else `wide`) in 2^-60, toward zero.
@@ -370,21 +390,25 @@ __device__ __forceinline__ bool vibb_grid(const int (&e)[3], bool diag, double q
   const uint64_t Q = to_grid<10>(q, 0, bad);
   const Halves hq = halves((int64_t)Q);
   const uint64_t dR = R - RR;
-  wide |= beyond_rho(R) | beyond_rho(RR) | beyond<59>(dR);
+  Within<59> w59;
+  Within<57> w57;
+  wide = beyond_rho(R) | beyond_rho(RR);
+  w59(dR);
   const uint64_t rd = local_rho && Q > (1ull << 61) ? R : RR + (uint64_t)mul_grid<3>(hq, halves((int64_t)dR));
   const Halves hd = halves((int64_t)rd);
   // t - 1 in 2^-59
   const int64_t tf = mul_grid<0>(hd, halves(reciprocal_grid(R))) - (1ll << 59);
   const int64_t tff = mul_grid<0>(hd, halves(reciprocal_grid(RR))) - (1ll << 59);
-  wide |= beyond<57>((uint64_t)tf) | beyond<57>((uint64_t)tff);
+  w57((uint64_t)tf);
+  w57((uint64_t)tff);
   const int64_t G = (int64_t)F + mul_grid<5>(halves((int64_t)F), halves(tf));
   const int64_t GG = (int64_t)FF + mul_grid<5>(halves((int64_t)FF), halves(tff));
-  wide |= beyond<59>((uint64_t)(G - GG));
+  w59((uint64_t)(G - GG));
   int64_t v = GG + mul_grid<3>(hq, halves(G - GG));
   // K in 2^-59 of a velocity in 2^-60
   auto K = [&](const int64_t (&u)[3]) {
     const int64_t eu = dot_grid(e, u[0], u[1], u[2]);
-    wide |= beyond<59>((uint64_t)eu);
+    w59((uint64_t)eu);
     const Halves he = halves(eu);
     int64_t r = eu + 3 * mul_grid<3>(he, he);
 #pragma unroll
@@ -402,12 +426,12 @@ __device__ __forceinline__ bool vibb_grid(const int (&e)[3], bool diag, double q
     uu[a] = velocity_grid(mff[1 + a], wide);
     ud[a] = mul_grid<2>(cf, halves(u[a])) + mul_grid<2>(cff, halves(uu[a]));
     if (moving) ud[a] += mul_grid<2>(cw, halves(velocity_grid(uw[a], wide)));
-    wide |= beyond<59>((uint64_t)ud[a]);
+    w59((uint64_t)ud[a]);
   }
   const int64_t Kf = K(u), Kff = K(uu), Kd = K(ud);
-  wide |= beyond<59>((uint64_t)(Kf - Kff));
+  w59((uint64_t)(Kf - Kff));
   const int64_t X = Kd - Kff - mul_grid<3>(hq, halves(Kf - Kff));
-  wide |= beyond<57>((uint64_t)X);
+  w57((uint64_t)X);
   // 3/2 w in 2^-64: 1/24 (diagonal), 1/12 or 1/6 (axis)
   const Halves W = diag ? halves(0x0aaaaaaaaaaaaaabll) : (D3 ? halves(0x1555555555555555ll) : halves(0x2aaaaaaaaaaaaaabll));
   v += mul_grid<5>(halves(mul_grid<0>(hd, W)), halves(X));
@@ -418,7 +442,7 @@ __device__ __forceinline__ bool vibb_grid(const int (&e)[3], bool diag, double q
     v += __double2ll_rn(ws);
   }
   val = from_grid<true>((uint64_t)v, k.sc, out);
-  return bad < 32u && wide == 0u && (int32_t)out >= 0;
+  return bad < 32u && wide == 0u && !(w59.broken() || w57.broken()) && (int32_t)out >= 0;
 }
 
 #endif  // __CUDACC__

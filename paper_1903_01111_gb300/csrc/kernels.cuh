@@ -977,6 +977,19 @@ __device__ __forceinline__ DirVal<T> dir_of(const DirTable<T, Q>& tab, int ip) {
   return DirVal<T>{tab.w[ip], tab.e[ip][0], tab.e[ip][1], tab.e[ip][2], {tab.ie[ip][0], tab.ie[ip][1], tab.ie[ip][2]}};
 }
 
+// The link's momentum exchange (f+_i'(x_f,t) + f_i(x_f,t+1)) e_i' without its
+// part at rest, 2 w_i' rho0, a geometric constant of the body that the host
+// adds in FP64: the sums stay as small as the force (over a closed body the
+// rest parts cancel, but not their roundings).  Shifted storage leaves it out
+// by itself.
+template <class P>
+__device__ __forceinline__ typename P::T exchange(typename P::T fpf, typename P::T val, const DirVal<typename P::T>& dir,
+                                                  const Params& p) {
+  if constexpr (P::shifted) return fpf + val;
+  const double c = dir.w() * p.rho0;
+  return (fpf - c) + (val - c);
+}
+
 // A link's momentum exchange t e added to its body's slot by FP64 atomics.
 template <class T>
 __device__ __forceinline__ void add_force(double* __restrict__ force, int body, T t, const DirVal<T>& dir) {
@@ -986,11 +999,10 @@ __device__ __forceinline__ void add_force(double* __restrict__ force, int body, 
 }
 
 // Sum of the momentum exchange t e over links of one body.  FP32 adds in FP32;
-// FP64 adds integers in steps of 2^(sc - 55) (a warp's reduction of doubles is
-// 15 FP64 instructions, and rounds at the last place of the sum), and hands a
-// t of 2^(sc - 1) or more, or not a number, to `direct`, which adds it to the
-// body's slot by itself.  No sum of a warp's links reaches 2^63 steps: the
-// populations of a node add up to its density.
+// FP64 adds integers in steps of 2^(sc - 57) (a warp's reduction of doubles is
+// 15 FP64 instructions), and hands a t of 2^(sc - 4) or more, or not a number,
+// to `direct`, which adds it to the body's slot by itself: no sum of the 576
+// links that a warp may hold reaches 2^63 steps.
 template <class T>
 struct LinkForce {
   T F[3] = {0, 0, 0};
@@ -1014,11 +1026,11 @@ struct LinkForce<double> {
   template <class Direct>
   __device__ __forceinline__ void add(double t, const DirVal<double>& dir, const FixedK& k, Direct&& direct) {
     const uint32_t hi = (uint32_t)__double2hiint(t), e = (hi >> 20) & 0x7ffu;
-    if (k.step == 0.0 || e >= (uint32_t)(1022 + k.sc)) return direct();
-    // t 2^(55 - sc) by its exponent (a t too small for that is none of a step)
+    if (k.step == 0.0 || e >= (uint32_t)(1019 + k.sc)) return direct();
+    // t 2^(57 - sc) by its exponent (a t too small for that is none of a step)
     const bool tiny = (int)e < 900 + k.sc || e == 0u;
     const int64_t v = __double2ll_rn(
-        __hiloint2double((int)(hi + ((uint32_t)(55 - k.sc) << 20)), __double2loint(t)));
+        __hiloint2double((int)(hi + ((uint32_t)(57 - k.sc) << 20)), __double2loint(t)));
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const int64_t s = dir.e[a] >> 31, on = tiny ? 0 : -(int64_t)(dir.e[a] & 1);
@@ -1031,7 +1043,7 @@ struct LinkForce<double> {
 #pragma unroll
       for (int a = 0; a < 3; ++a) F[a] += __shfl_down_sync(0xffffffffu, F[a], o);
   }
-  __device__ __forceinline__ double value(int a, const FixedK& k) const { return (double)F[a] * (k.step * 128.0); }
+  __device__ __forceinline__ double value(int a, const FixedK& k) const { return (double)F[a] * (k.step * 32.0); }
 };
 
 // One thread per link.  recs: storage indices and metadata; qv: q in
@@ -1101,11 +1113,8 @@ __global__ void __launch_bounds__(256, (P::shifted ? 2 : 3)) k_links(typename P:
                                     uw2, p, fpf, uwv != nullptr, wqv + k, nl);
       f[(size_t)tab.opp[ip] * N + rec.ks] = val;
       if (body >= 0) {
-        // momentum exchange (f+_i'(x_f,t) + f_i(x_f,t+1)) e_i'.  In shifted
-        // storage this sums (h+_i' + h_i) e_i'; the rest part 2 w_i' rho0 e_i'
-        // of every link is a geometric constant that the host adds in FP64.
-        const T t = fpf + val;
         const DirVal<T> dir = dir_of(tab, ip);
+        const T t = exchange<P>(fpf, val, dir, p);
         auto direct = [&] { add_force(force, body, t, dir); };
         if (body == b0)
           F.add(t, dir, p.kx, direct);
@@ -1275,8 +1284,8 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
     stage[o >> 5][tab.opp[ip]][o & 31] = val;
     if (body >= 0) {
       // momentum exchange as in k_links
-      const T t = fpf + val;
       const DirVal<T> dir = dir_of(tab, ip);
+      const T t = exchange<P>(fpf, val, dir, p);
       auto direct = [&] { add_force(force, body, t, dir); };
       if (body == wb)
         F.add(t, dir, p.kx, direct);
@@ -1384,7 +1393,11 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
   const bool live = some && (uint64_t)k < S;
   const int64_t l0 = some ? __ldg(fl.first + g) : 0, l1 = some ? __ldg(fl.first + g + 1) : 0;
   FusedRec r{0, 0, 0, 0};
-  if (first >= 0 && l0 + first < l1) r = fl.rec[l0 + first];
+  T q1 = 0;
+  if (first >= 0 && l0 + first < l1) {
+    r = fl.rec[l0 + first];
+    if (!P::shifted) q1 = (T)__ldg(fl.qd + l0 + first);
+  }
   const uint32_t w = live ? __ldg(lay.word + k) : W_GHOST;
   const uint32_t mask = live ? __ldg(fl.mask + k) : 0u;
   const bool fluid = !(w & (W_GHOST | W_OPEN));
@@ -1404,8 +1417,11 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
   const int wb = (int)(__shfl_sync(0xffffffffu, r.meta, 0) >> 8) - 1;
   LinkForce<T> F;
   for (int64_t li = first < 0 ? l1 : l0 + first; li < l1; li += step) {
-    if (li != l0 + first) r = fl.rec[li];
-    const T q = P::shifted ? (T)__uint_as_float(r.q32) : (T)__ldg(fl.qd + li);
+    if (li != l0 + first) {
+      r = fl.rec[li];
+      if (!P::shifted) q1 = (T)__ldg(fl.qd + li);
+    }
+    const T q = P::shifted ? (T)__uint_as_float(r.q32) : q1;
     const int ip = (int)(r.meta & 31), rule = (int)((r.meta >> 5) & 7), body = (int)(r.meta >> 8) - 1;
     const int i = (int)(d2q9_opposites() >> (4 * ip)) & 15;
     const int ex = (int)((d2q9_pack(false) >> (2 * ip)) & 3) - 1, ey = (int)((d2q9_pack(true) >> (2 * ip)) & 3) - 1;
@@ -1422,7 +1438,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
     col[i][r.kf & 31] = val;
     if (body >= 0) {
       // momentum exchange as in k_links
-      const T t = fpf + val;
+      const T t = exchange<P>(fpf, val, dir, p);
       auto direct = [&] { add_force(force, body, t, dir); };
       if (body == wb)
         F.add(t, dir, p.kx, direct);
@@ -1431,18 +1447,42 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
     }
   }
   if (!P::shifted && !spread) pull();
-  if (spread)
+  if (wb >= 0) F.reduce();
+  if (lane == 0) {
+    red[0][warp] = F.value(0, p.kx);
+    red[1][warp] = F.value(1, p.kx);
+    rbody[warp] = wb;
+  }
+  // the block's force: one atomic per run of warps with one body
+  auto add_block_force = [&](int a) {
+    double acc = 0.0;
+#pragma unroll 1
+    for (int wi = 0; wi < NW; ++wi) {
+      const int b = rbody[wi];
+      acc += red[a][wi];
+      if (b >= 0 && (wi == NW - 1 || rbody[wi + 1] != b)) {
+        atomicAdd(&force[3 * b + a], acc);
+        acc = 0.0;
+      }
+    }
+  };
+  if (spread) {
     __syncthreads();
-  else
+    if (!mine) {  // (the force off the first warp's way)
+      if (warp == 1 && lane < 2) add_block_force(lane);
+      return;
+    }
+  } else {
     __syncwarp();
+  }
   // the populations of v that come from a wall
   auto take = [&](T(&v)[L::Q]) {
 #pragma unroll
     for (int i = 1; i < L::Q; ++i)
       if ((mask >> L::opp(i)) & 1u) v[i] = col[i][lane];
   };
-  if (mask && mine) take(f);
-  if (live && mine && !(w & W_OPEN)) {
+  if (mask) take(f);
+  if (live && !(w & W_OPEN)) {
     // ghost slots: zeros through the same stores (inputs at rest)
     auto rest = [&](T(&v)[L::Q]) {
 #pragma unroll
@@ -1456,26 +1496,9 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
     });
     if (fluid && (p.inlet | p.outlet)) open_ends<L, P>(fout, mom_out, S, k, lay.runs[w & W_RUN], lay, p);
   }
-  if (wb >= 0) F.reduce();
-  if (lane == 0) {
-    red[0][warp] = F.value(0, p.kx);
-    red[1][warp] = F.value(1, p.kx);
-    rbody[warp] = wb;
-  }
+  if (spread) return;
   __syncthreads();
-  if (threadIdx.x < 2) {
-    // one atomic per run of warps with one body
-    double acc = 0.0;
-#pragma unroll 1
-    for (int wi = 0; wi < NW; ++wi) {
-      const int b = rbody[wi];
-      acc += red[threadIdx.x][wi];
-      if (b >= 0 && (wi == NW - 1 || rbody[wi + 1] != b)) {
-        atomicAdd(&force[3 * b + threadIdx.x], acc);
-        acc = 0.0;
-      }
-    }
-  }
+  if (threadIdx.x < 2) add_block_force((int)threadIdx.x);
 }
 
 // ------------------------------------------------------- init and fields --

@@ -6,8 +6,8 @@
 // the layout tables, the link records (in the link kernel's order and in the
 // fused step kernel's (node, direction) order), the domain table of a batch
 // and two FP64 force slots.  lbm_step replays
-// captured CUDA graphs (graph_steps steps, then two) and launches single
-// steps directly for an odd remainder; with profiling on it launches kernel
+// captured CUDA graphs of graph_steps steps (tuned above two) and launches the
+// rest step by step; with profiling on it launches kernel
 // by kernel between CUDA events.  lbm_autotune picks the launch shapes.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -136,9 +136,10 @@ struct lbm_lattice_s {
   DeviceBuf lqc, lqf;
   int64_t n_links = 0, n_fluid = 0, n_cached = 0, n_runs = 0;
   DeviceBuf force;  // [2][nbody][3]
-  // shifted storage: sum over each body's links of 2 w_i' rho0 e_i' (FP64),
-  // the rest part of the momentum exchange that the link kernel leaves out
+  // sum over each body's links of 2 w_i' rho0 e_i' (FP64), the rest part of the
+  // momentum exchange that the kernels leave out
   std::vector<double> force_rest = std::vector<double>(3, 0.0);
+  DeviceBuf force_hist;  // [steps][nbody][3]: the slots of the steps of one lbm_step_forces chunk
   // pinned host copy of the force slot read by lbm_force / lbm_forces (a
   // device-to-host copy into pageable memory is staged by the driver)
   double* force_host = nullptr;
@@ -150,7 +151,6 @@ struct lbm_lattice_s {
   bool has_geometry = false, has_state = false;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};   // two steps, per parity of the buffer
   cudaGraphExec_t graphG[2] = {nullptr, nullptr};  // tune.graph_steps steps
   // profiling
   bool profiling = false;
@@ -213,9 +213,8 @@ void touch_host_output(void* p, size_t bytes) {
 
 void drop_graphs(lbm_handle h) {
   for (int k = 0; k < 2; ++k) {
-    if (h->graph[k]) cudaGraphExecDestroy(h->graph[k]);
     if (h->graphG[k]) cudaGraphExecDestroy(h->graphG[k]);
-    h->graph[k] = h->graphG[k] = nullptr;
+    h->graphG[k] = nullptr;
   }
 }
 
@@ -266,9 +265,13 @@ int fused_threads(const lbm_handle h) {
 }
 
 // Enqueue one time step on the stream (parity = buffer holding f+(t)).
-lbm_status enqueue_step(lbm_handle h, int parity, int64_t step_index, bool timed) {
+lbm_status enqueue_step(lbm_handle h, int parity, int64_t step_index, bool timed, double* slot = nullptr) {
   double* force = (double*)h->force.p;
   const int64_t nb3 = 3 * (int64_t)h->nbody;
+  // a slot of the step's own (already zero): nothing to clear for the next
+  if (slot)
+    return enqueue_step_buf(h, h->f[parity].p, h->f[parity ^ 1].p, h->mom[parity].p, h->mom[parity ^ 1].p, slot,
+                            nullptr, timed, use_fused(h));
   return enqueue_step_buf(h, h->f[parity].p, h->f[parity ^ 1].p, h->mom[parity].p, h->mom[parity ^ 1].p,
                           force + nb3 * (step_index & 1), force + nb3 * ((step_index + 1) & 1), timed, use_fused(h));
 }
@@ -483,6 +486,7 @@ lbm_status lbm_destroy(lbm_handle h) {
   for (auto e : h->ev) cudaEventDestroy(e);
   release_geometry(h);
   release(h->force);
+  release(h->force_hist);
   if (h->force_host) cudaFreeHost(h->force_host);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
@@ -987,11 +991,11 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
         if (!(word[k] & (W_GHOST | W_OPEN))) flist[j++] = (uint32_t)k;
     }
   }
-  // rest part of the momentum exchange per body (shifted storage):
+  // rest part of the momentum exchange per body, left out by the kernels:
   // sum over the body's links of 2 w_i' rho0 e_i', from the exact count of
   // its links per direction (counted in parallel, summed in a fixed order)
   std::vector<double> rest(3 * (size_t)nbody, 0.0);
-  if (c.precision == LBM_FP32_SHIFTED && n_links > 0 && max_body >= 0) {
+  if (n_links > 0 && max_body >= 0) {
     const size_t nc = (size_t)(max_body + 1) * Q;
     std::vector<int64_t> cnt(nc, 0);
 #pragma omp parallel
@@ -1007,7 +1011,9 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
       for (int d = 1; d < Q; ++d) {
         const int64_t n = cnt[(size_t)b * Q + d];
         if (n == 0) continue;
-        const double t = (double)n * 2.0 * (Q == 9 ? D2Q9::w(d) : D3Q19::w(d)) * c.rho0;
+        const double w = Q == 9 ? D2Q9::w(d) : D3Q19::w(d);
+        // (FP64: n times what the kernels take off a link)
+        const double t = h->rb == 8 ? (double)n * (2.0 * (w * c.rho0)) : (double)n * 2.0 * w * c.rho0;
         rest[3 * b + 0] += t * cx_of(h, d);
         rest[3 * b + 1] += t * cy_of(h, d);
         rest[3 * b + 2] += t * cz_of(h, d);
@@ -1322,17 +1328,9 @@ lbm_status lbm_step(lbm_handle h, int64_t n) {
       h->step += G;
     }
   }
-  if (left >= 2) {
-    if (!h->graph[h->cur]) {
-      lbm_status st = build_graph(h, h->cur, 2, &h->graph[h->cur]);
-      if (st != LBM_OK) return st;
-    }
-    for (; left >= 2; left -= 2) {
-      CUDA_TRY(cudaGraphLaunch(h->graph[h->cur], h->stream));
-      h->step += 2;
-    }
-  }
-  if (left == 1) {
+  // step by step: each kernel lets the next start early, so that a graph of
+  // two steps (whose ends do not overlap) gains nothing over their launches
+  for (; left > 0; --left) {
     lbm_status st = enqueue_step(h, h->cur, h->step, false);
     if (st != LBM_OK) return st;
     h->cur ^= 1;
@@ -1410,35 +1408,47 @@ lbm_status lbm_step_forces(lbm_handle h, int64_t n, int32_t body, double* F) {
   if (!h || n < 0 || (n > 0 && !F)) return fail(LBM_ERR_INVALID_ARG, "null or negative argument");
   if (body < 0 || body >= MAX_BODIES) return fail(LBM_ERR_INVALID_ARG, "body %d out of range", body);
   if (!h->has_state) return fail(LBM_ERR_STATE, "initialise the state first");
-  constexpr int64_t kChunk = 4096;
+  // A chunk of steps adds its forces into slots of their own, cleared before
+  // and copied out after it (a copy per step cost its launch and kept every
+  // step from starting early: 35 -> 13 us per step on a 2000 x 400 channel).
+  const int64_t nb3 = 3 * (int64_t)h->nbody;
+  const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(4096, (int64_t)(8 << 20) / (8 * nb3)));
   const bool has = body < h->nbody;
   double* pinned = nullptr;
   if (n > 0) {
-    lbm_status st = force_host_buffer(h, 3 * (size_t)std::min(n, kChunk), &pinned);
+    const int64_t m = std::min(n, chunk);
+    lbm_status st = force_host_buffer(h, 3 * (size_t)m, &pinned);
+    if (st == LBM_OK && h->force_hist.bytes < sizeof(double) * nb3 * m)
+      st = acquire(h->force_hist, sizeof(double) * nb3 * m);
     if (st != LBM_OK) return st;
   }
-  for (int64_t k0 = 0; k0 < n; k0 += kChunk) {
-    const int64_t m = std::min(kChunk, n - k0);
+  double* hist = (double*)h->force_hist.p;
+  double* slots = (double*)h->force.p;
+  for (int64_t k0 = 0; k0 < n; k0 += chunk) {
+    const int64_t m = std::min(chunk, n - k0);
+    CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(double) * nb3 * m, h->stream));
     for (int64_t k = 0; k < m; ++k) {
-      lbm_status st = enqueue_step(h, h->cur, h->step, h->profiling);
+      lbm_status st = enqueue_step(h, h->cur, h->step, h->profiling, hist + nb3 * k);
       if (st != LBM_OK) return st;
       h->cur ^= 1;
       ++h->step;
-      // this step's slot: the next step clears the other one, the step
-      // after it this one, so the copy (queued before both) reads it whole
-      if (has) {
-        const double* slot = (const double*)h->force.p + 3 * (int64_t)h->nbody * ((h->step - 1) & 1) + 3 * body;
-        CUDA_TRY(cudaMemcpyAsync(pinned + 3 * k, slot, sizeof(double) * 3, cudaMemcpyDeviceToHost, h->stream));
-      }
       if (h->profiling && h->ev_used > (1u << 16)) {
         st = harvest_events(h);
         if (st != LBM_OK) return st;
       }
     }
+    // the state's own slots as lbm_step leaves them: the last step's force, and
+    // zeros for the next
+    CUDA_TRY(cudaMemcpyAsync(slots + nb3 * ((h->step - 1) & 1), hist + nb3 * (m - 1), sizeof(double) * nb3,
+                             cudaMemcpyDeviceToDevice, h->stream));
+    CUDA_TRY(cudaMemsetAsync(slots + nb3 * (h->step & 1), 0, sizeof(double) * nb3, h->stream));
+    if (has)
+      CUDA_TRY(cudaMemcpy2DAsync(pinned, sizeof(double) * 3, hist + 3 * body, sizeof(double) * nb3, sizeof(double) * 3,
+                                 m, cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     for (int64_t k = 0; k < m; ++k)
-      for (int a = 0; a < 3; ++a)
-        F[3 * (k0 + k) + a] = has ? pinned[3 * k + a] + h->force_rest[3 * body + a] : 0.0;
+      for (int c = 0; c < 3; ++c)
+        F[3 * (k0 + k) + c] = has ? pinned[3 * k + c] + h->force_rest[3 * body + c] : 0.0;
   }
   return LBM_OK;
 }
