@@ -188,6 +188,8 @@ __global__ void __launch_bounds__(256, (adj_bulk_blocks_per_sm<L, P>())) k_adj_b
   using T = typename P::T;
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   const size_t S = (size_t)lay.S;
+  prefetch_ahead<L::Q>(fin, lay, k & ~31u, 32, threadIdx.x & 31, 32);
+  prefetch_ahead<L::Q>((const T*)lam_next, lay, k & ~31u, 32, threadIdx.x & 31, 32);
   T dt = 0;
   int key = -1;
   if (k < (uint64_t)lay.S) {

@@ -121,7 +121,7 @@ __host__ __device__ constexpr int row_slot(int dy, int dz) {
 }
 
 struct Layout {
-  int64_t S;                   // stored nodes
+  int64_t S;                   // stored nodes, padded to a multiple of 32
   const uint32_t* word;        // [S]
   const int32_t* node_of;      // [S] dense node index
   const int32_t* tile;         // [ceil(N / MOM_TILE) + 1] first stored node of each tile of dense nodes
@@ -138,6 +138,7 @@ struct Layout {
   const void* row_uin;         // [ny] inlet velocity of each row, storage precision (open inlet)
   const uint32_t* groups;      // D2Q9: 32-node groups with links (nlinked of them), then those without
   int64_t nlinked, ngroups;
+  uint32_t ahead;              // nodes ahead that the step kernels prefetch into L2 (0: the state stays there)
 };
 
 __device__ __forceinline__ Relax relax_params(const Params& p) {
@@ -166,6 +167,27 @@ struct __align__(16) LinkRec {
 };
 
 // --------------------------------------------------------------- helpers --
+
+// Asks L2 for the populations of the N stored nodes from k (a multiple of 32)
+// on, `ahead` nodes further, by threads t = 0, 1, ... of nt: one request per
+// 128-byte line of a direction.  A block's pulls wait behind its node words and
+// runs, so too few of them are in flight to keep HBM busy (D2Q9 FP32 60 %);
+// brought into L2 a few microseconds early they wait a third as long.  ahead is
+// about 6 MB of state: 8192 x 4096 D2Q9 FP32 468 us per step without, 413 / 402 /
+// 399 / 407 at 1.4 / 2.8 / 5.6 / 11 MB; dense 301 x 257 x 259 506 -> 486, 526 at 24 MB
+// (the far half of L2 is used up); 384^3 pack 1298 -> 1266.
+template <int Q, class T>
+__device__ __forceinline__ void prefetch_ahead(const T* __restrict__ f, const Layout& lay, uint64_t k, int N, int t,
+                                               int nt) {
+  constexpr int per = 128 / (int)sizeof(T);
+  const uint64_t from = k + lay.ahead;
+  if (lay.ahead == 0u || from + N > (uint64_t)lay.S) return;
+  const int lines = N / per;
+  for (int j = t; j < lines * Q; j += nt) {
+    const int i = j / lines;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(f + (uint64_t)i * lay.S + from + (uint64_t)(j - i * lines) * per));
+  }
+}
 
 // Clears the force slot of the next step (the grid's first block).
 template <int BT>
@@ -685,6 +707,7 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_b
   for (int j = 0; j < NPT; ++j) {
     k[j] = t + (uint32_t)j * stride;
     live[j] = t < stride && (uint64_t)k[j] < (uint64_t)lay.S;
+    prefetch_ahead<L::Q>(fin, lay, (uint64_t)blockIdx.x * BT + (uint64_t)j * (stride / 32 * 32), BT, threadIdx.x, BT);
   }
   bulk_nodes<L, P, MULTI, NPT>(k, live, fin, fout, lay, mom, p);
   clear_force<BT>(force_next, p.nbody);
@@ -714,6 +737,8 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, 1>())) k_bul
   wait_for_previous();
   clear_force<BT>(force_next, p.nbody);
   if (!live) return;
+  // (the block's nodes lie at its share of the storage)
+  prefetch_ahead<L::Q>(fin, lay, (uint64_t)k / 32 * 32 - (threadIdx.x & ~31u), BT, threadIdx.x, BT);
   T f[L::Q];
   pull_node<L>(fin, S, k, run, lay, p, f);
   collide_node<L, P, MULTI>(f, p, lay, run.dom, fout, S, k, mom, (w & W_CACHE) != 0, true, [&](T(&g)[L::Q]) {
@@ -810,20 +835,26 @@ __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_
 // lanes holding different directions read it without serialisation.
 template <class T, int Q>
 struct DirTable {
-  int off[Q];   // cx + nx (cy + ny cz): node offset of e_d (32-bit)
   int opp[Q];
   T w[Q];
   T e[Q][3];
-  int ie[Q][3];
+  int ie[sizeof(T) == 8 ? Q : 1][3];  // the same as integers (FP64)
 };
 
-// A direction as values (read from the table).
+// A direction as values (read from the table); for FP64 as integers too (a
+// conversion costs as much as an addition).
 template <class T>
 struct DirVal {
   T wt, ex, ey, ez;
-  int e[3];  // the same as integers (FP64: a conversion costs as much as an addition)
   __device__ __forceinline__ T w() const { return wt; }
   __device__ __forceinline__ T dot(T x, T y, T z) const { return ex * x + ey * y + ez * z; }
+};
+template <>
+struct DirVal<double> {
+  double wt, ex, ey, ez;
+  int e[3];
+  __device__ __forceinline__ double w() const { return wt; }
+  __device__ __forceinline__ double dot(double x, double y, double z) const { return ex * x + ey * y + ez * z; }
 };
 // Equilibrium of direction `dir` (storage form, see above).
 template <class P, class Dir>
@@ -911,15 +942,16 @@ template <class L, class T>
 __device__ __forceinline__ void fill_dir_table(DirTable<T, L::Q>& tab) {
   if (threadIdx.x < L::Q) {
     const int d = threadIdx.x;
-    tab.off[d] = 0;
     tab.opp[d] = L::opp(d);
     tab.w[d] = (T)L::w(d);
     tab.e[d][0] = (T)L::cx(d);
     tab.e[d][1] = (T)L::cy(d);
     tab.e[d][2] = (T)L::cz(d);
-    tab.ie[d][0] = L::cx(d);
-    tab.ie[d][1] = L::cy(d);
-    tab.ie[d][2] = L::cz(d);
+    if constexpr (sizeof(T) == 8) {
+      tab.ie[d][0] = L::cx(d);
+      tab.ie[d][1] = L::cy(d);
+      tab.ie[d][2] = L::cz(d);
+    }
   }
 }
 
@@ -974,7 +1006,10 @@ __device__ __forceinline__ typename P::T eval_link(const DirVal<typename P::T>& 
 // Direction ip from the table.
 template <class T, int Q>
 __device__ __forceinline__ DirVal<T> dir_of(const DirTable<T, Q>& tab, int ip) {
-  return DirVal<T>{tab.w[ip], tab.e[ip][0], tab.e[ip][1], tab.e[ip][2], {tab.ie[ip][0], tab.ie[ip][1], tab.ie[ip][2]}};
+  if constexpr (sizeof(T) == 8)
+    return DirVal<T>{tab.w[ip], tab.e[ip][0], tab.e[ip][1], tab.e[ip][2], {tab.ie[ip][0], tab.ie[ip][1], tab.ie[ip][2]}};
+  else
+    return DirVal<T>{tab.w[ip], tab.e[ip][0], tab.e[ip][1], tab.e[ip][2]};
 }
 
 // The link's momentum exchange (f+_i'(x_f,t) + f_i(x_f,t+1)) e_i' without its
@@ -993,9 +1028,9 @@ __device__ __forceinline__ typename P::T exchange(typename P::T fpf, typename P:
 // A link's momentum exchange t e added to its body's slot by FP64 atomics.
 template <class T>
 __device__ __forceinline__ void add_force(double* __restrict__ force, int body, T t, const DirVal<T>& dir) {
-  if (dir.e[0]) atomicAdd(&force[3 * body + 0], (double)(t * dir.ex));
-  if (dir.e[1]) atomicAdd(&force[3 * body + 1], (double)(t * dir.ey));
-  if (dir.e[2]) atomicAdd(&force[3 * body + 2], (double)(t * dir.ez));
+  atomicAdd(&force[3 * body + 0], (double)(t * dir.ex));
+  atomicAdd(&force[3 * body + 1], (double)(t * dir.ey));
+  if (dir.ez != (T)0) atomicAdd(&force[3 * body + 2], (double)(t * dir.ez));
 }
 
 // Sum of the momentum exchange t e over links of one body.  FP32 adds in FP32;
@@ -1220,6 +1255,9 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
   __shared__ double red[3][NW];
   let_next_start();
   fill_dir_table<L>(tab);
+  // (waits before the link records: held back behind them it cost 2 %)
+  wait_for_previous();
+  clear_force<BT>(force_next, p.nbody);
   __syncthreads();  // the direction table (every thread arrives here at once)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t base = blockIdx.x * BT;
@@ -1228,6 +1266,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
   const bool live = (uint64_t)k < S;
   const uint32_t w = live ? __ldg(lay.word + k) : W_GHOST;
   const uint32_t mask = live ? __ldg(fl.mask + k) : 0u;
+  prefetch_ahead<L::Q>(fin, lay, base, BT, threadIdx.x, BT);
   // the block's range of the link list (the same two words in every thread)
   const int64_t g0 = base >> 5, g1 = g0 + NW < fl.ngroups ? g0 + NW : fl.ngroups;
   const int64_t l0 = __ldg(fl.first + g0), l1 = __ldg(fl.first + g1);
@@ -1243,8 +1282,6 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
   const bool fluid = live && !(w & (W_GHOST | W_OPEN));
   T(&col)[L::Q][32] = stage[warp];
   int dom = 0;
-  wait_for_previous();
-  clear_force<BT>(force_next, p.nbody);
   if (fluid) {
     const RunRec run = lay.runs[w & W_RUN];
     if (MULTI) dom = run.dom;
@@ -1255,10 +1292,11 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
     for (int i = 0; i < L::Q; ++i)
       // direction i comes from the solid side when its opposite is a link
       if (!((mask >> L::opp(i)) & 1u)) cp_async_real(&col[i][lane], fk + ((ptrdiff_t)i * (ptrdiff_t)S + d[i]));
-  } else if (live) {
-    // ghost and open slots: zeros through the same stores (inputs at rest)
+  } else if (live && !P::shifted) {
+    // ghost slots store zeros whatever their column holds; FP64 puts the rest
+    // state there, which its integer collision takes
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) col[i][lane] = P::shifted ? (T)0 : (T)L::w(i);
+    for (int i = 0; i < L::Q; ++i) col[i][lane] = (T)L::w(i);
   }
   cp_async_commit();
   const int wb = total > 0 ? (int)(__ldg(&fl.rec[l0].meta) >> 8) - 1 : -1;
@@ -1376,6 +1414,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
       k[j] = at + j < lay.ngroups ? 32u * __ldg(lay.groups + at + j) + lane : 0u;
       live[j] = at + j < lay.ngroups && (uint64_t)k[j] < S;
     }
+    prefetch_ahead<L::Q>(fin, lay, k[0] - lane, 32 * NF, lane, 32);
     bulk_nodes<L, P, MULTI, NF>(k, live, fin, fout, lay, mom_out, p);
     clear_force<BT>(force_next, p.nbody);
     return;
@@ -1426,7 +1465,16 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
     const int i = (int)(d2q9_opposites() >> (4 * ip)) & 15;
     const int ex = (int)((d2q9_pack(false) >> (2 * ip)) & 3) - 1, ey = (int)((d2q9_pack(true) >> (2 * ip)) & 3) - 1;
     auto real = [](int e) { return e == 0 ? (T)0 : (e > 0 ? (T)1 : (T)-1); };
-    const DirVal<T> dir{ip < 5 ? (T)L::w(1) : (T)L::w(5), real(ex), real(ey), (T)0, {ex, ey, 0}};
+    DirVal<T> dir;
+    dir.wt = ip < 5 ? (T)L::w(1) : (T)L::w(5);
+    dir.ex = real(ex);
+    dir.ey = real(ey);
+    dir.ez = (T)0;
+    if constexpr (!P::shifted) {
+      dir.e[0] = ex;
+      dir.e[1] = ey;
+      dir.e[2] = 0;
+    }
     T uw0 = 0, uw1 = 0;
     if (fl.uw) {
       uw0 = fl.uw[li];

@@ -134,7 +134,7 @@ struct lbm_lattice_s {
   // FP64: VIBB velocity weights [3][n_links] in the link kernel's order, and in
   // the fused kernel's where that is another one
   DeviceBuf lqc, lqf;
-  int64_t n_links = 0, n_fluid = 0, n_cached = 0, n_runs = 0;
+  int64_t n_links = 0, n_fluid = 0, n_stored = 0, n_cached = 0, n_runs = 0;
   DeviceBuf force;  // [2][nbody][3]
   // sum over each body's links of 2 w_i' rho0 e_i' (FP64), the rest part of the
   // momentum exchange that the kernels leave out
@@ -821,12 +821,16 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
     chunk_start[ch + 1] = cnt;
   }
   for (int64_t ch = 0; ch < nchunk; ++ch) chunk_start[ch + 1] += chunk_start[ch];
-  const int64_t S = chunk_start[nchunk];
+  // the slots of a direction are padded to whole groups of 32 (ghosts that no
+  // link writes and no node pulls), so that every direction's rows and pairs
+  // are aligned
+  const int64_t n_stored = chunk_start[nchunk], S = (n_stored + 31) / 32 * 32;
   raw_vec<int32_t> sidx(N);
   par_fill(sidx, (int32_t)-1);
   raw_vec<int32_t> node_of((size_t)S);  // written for every stored node
+  std::fill(node_of.begin() + n_stored, node_of.end(), 0);
   const int64_t ntile = (N + MOM_TILE - 1) / MOM_TILE;
-  std::vector<int32_t> tile(ntile + 1, (int32_t)S);  // first stored node of each tile of dense nodes
+  std::vector<int32_t> tile(ntile + 1, (int32_t)n_stored);  // first stored node of each tile of dense nodes
 #pragma omp parallel for schedule(static)
   for (int64_t ch = 0; ch < nchunk; ++ch) {
     int64_t k = chunk_start[ch];
@@ -952,7 +956,7 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   raw_vec<RunRec> runs((size_t)row_runs[rows]);
   par_fill(runs, RunRec{});
   raw_vec<uint32_t> word(S);
-  par_fill(word, 0u);
+  par_fill(word, (uint32_t)W_GHOST);
 #pragma omp parallel for schedule(dynamic, 64)
   for (int64_t r = 0; r < rows; ++r) {
     int64_t bad[2];
@@ -1227,6 +1231,9 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   h->lay.groups = (const uint32_t*)h->groups.p;
   h->lay.nlinked = nlinked;
   h->lay.ngroups = ngroups;
+  // two states beyond what L2 keeps from one step to the next: prefetch
+  const int64_t state = (int64_t)Q * S * (int64_t)rb;
+  h->lay.ahead = 2 * state > (96ll << 20) ? (uint32_t)((6ll << 20) / (Q * (int64_t)rb) / 32 * 32) : 0u;
   // a single domain runs through Params like an unsplit lattice
   Params& p = h->p;
   const lbm_domain one{0, 0, 0, 0, c.tau, {c.g[0], c.g[1], c.g[2]}, c.inlet_umax, c.inlet_y0, c.inlet_y1};
@@ -1245,6 +1252,7 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   h->sidx.swap(sidx);
   h->n_links = n_links;
   h->n_fluid = n_fluid;
+  h->n_stored = n_stored;
   h->n_cached = n_cached;
   h->n_runs = (int64_t)runs.size();
   h->force_rest.swap(rest);
@@ -1786,7 +1794,7 @@ lbm_status lbm_query(lbm_handle h, lbm_info* info) {
   info->D = h->D;
   info->precision = h->cfg.precision;
   info->real_bytes = (int32_t)h->rb;
-  info->n_stored = h->lay.S;
+  info->n_stored = h->n_stored;
   info->n_runs = h->n_runs;
   info->n_bodies = h->nbody;
   info->n_domains = std::max<int32_t>((int32_t)h->domains.size(), 1);

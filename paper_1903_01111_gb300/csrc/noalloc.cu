@@ -52,7 +52,6 @@ __global__ void __launch_bounds__(kBlock) k_force_partial(const double* __restri
   __shared__ double red[3][kBlock / 32];
   if (threadIdx.x < L::Q) {
     const int d = threadIdx.x;
-    tab.off[d] = 0;
     tab.opp[d] = L::opp(d);
     tab.w[d] = L::w(d);
     tab.e[d][0] = L::cx(d);
