@@ -40,6 +40,7 @@
 
 #include "fixed64.cuh"
 #include "lattice.cuh"
+#include "pair32.cuh"
 
 namespace lbm {
 
@@ -250,6 +251,48 @@ __device__ __forceinline__ const FixedK& fixed_of(const Params& p, const Layout&
     return p.kx;
 }
 
+// FP32 D2Q9 BGK parameters of one node from its run parameters and folded
+// constants, and those of two nodes.
+__device__ __forceinline__ Bgk32<float> bgk32_params(float rho0, const Relax& rx, const Folded& kc, bool force) {
+  Bgk32<float> c;
+  c.rho0 = rho0;
+  c.om = rx.omega_f;
+  if (force) {
+    constexpr int dir[4] = {1, 2, 5, 6};
+    c.hx = kc.hg_f[0];
+    c.hy = kc.hg_f[1];
+    c.gx = rx.g_f[0];
+    c.gy = rx.g_f[1];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) c.kf[i] = kc.kf_f[i];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      c.kt[i] = kc.kt_f[dir[i]];
+      c.ke[i] = kc.ke_f[dir[i]];
+    }
+  }
+  return c;
+}
+__device__ __forceinline__ Bgk32<F2> bgk32_pair(const Bgk32<float>& a, const Bgk32<float>& b, bool force) {
+  Bgk32<F2> c;
+  c.rho0 = pack2(a.rho0, b.rho0);
+  c.om = pack2(a.om, b.om);
+  if (force) {
+    c.hx = pack2(a.hx, b.hx);
+    c.hy = pack2(a.hy, b.hy);
+    c.gx = pack2(a.gx, b.gx);
+    c.gy = pack2(a.gy, b.gy);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) c.kf[i] = pack2(a.kf[i], b.kf[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      c.kt[i] = pack2(a.kt[i], b.kt[i]);
+      c.ke[i] = pack2(a.ke[i], b.ke[i]);
+    }
+  }
+  return c;
+}
+
 // Collision and store of one node: moments of f, Guo-forced BGK (or D2Q9
 // MRT) with the run parameters rx and the folded constants kc, the node's
 // moment cache entry when flagged.
@@ -261,6 +304,17 @@ __device__ __forceinline__ void collide_store(typename P::T (&f)[L::Q], const Pa
                                               typename P::T* __restrict__ fout, size_t S, uint32_t n_,
                                               Mom4<typename P::T>* __restrict__ mom, bool cache, bool keep = true) {
   using T = typename P::T;
+  if constexpr (P::shifted && L::Q == 9) {
+    if (p.collision == 0) {
+      const bool force = rx.has_force != 0;
+      float r, ux, uy;
+      bgk_d2q9(f, bgk32_params(p.rho0_f, rx, kc, force), force, r, ux, uy);
+      if (cache && keep) mom[n_] = Mom4<float>{r, ux, uy, 0.f};
+#pragma unroll
+      for (int i = 0; i < 9; ++i) fout[(size_t)i * S + n_] = keep ? f[i] : 0.f;
+      return;
+    }
+  }
   T r = 0, jx = 0, jy = 0, jz = 0;
   if constexpr (!P::shifted) {
     // FP64 (bound by the FP64 pipe, where every add, multiply or FMA takes
@@ -623,7 +677,7 @@ constexpr unsigned bulk_shape_mask() {
 // 339 with two nodes per thread, whose registers halve the warps in flight).
 template <class L, class P>
 constexpr int bulk_default_shape() {
-  return L::Q == 9 && P::shifted ? 3 : 1;
+  return L::Q == 9 && P::shifted ? 4 : 1;
 }
 
 // Resident blocks per SM a shape is compiled for, from a register budget per
@@ -692,6 +746,105 @@ __device__ __forceinline__ void bulk_nodes(const uint32_t (&k)[NPT], const bool 
   }
 }
 
+// The neighbouring nodes k (even) and k + 1 of one thread, FP32 D2Q9 BGK (see
+// pair32.cuh): their words, and the runs of those that are fluid.
+struct PairNodes {
+  uint2 w;
+  RunRec ra, rb;
+  __device__ __forceinline__ bool fa() const { return !(w.x & (W_GHOST | W_OPEN)); }
+  __device__ __forceinline__ bool fb() const { return !(w.y & (W_GHOST | W_OPEN)); }
+  __device__ __forceinline__ bool same() const { return fa() && fb() && ((w.x ^ w.y) & W_RUN) == 0; }
+};
+__device__ __forceinline__ PairNodes pair_nodes(uint32_t k, bool live, const Layout& lay) {
+  PairNodes n{};
+  n.w = live ? __ldg((const uint2*)(lay.word + k)) : make_uint2(W_GHOST, W_GHOST);
+  if (n.fa()) n.ra = lay.runs[n.w.x & W_RUN];
+  if (n.same())
+    n.rb = n.ra;
+  else if (n.fb())
+    n.rb = lay.runs[n.w.y & W_RUN];
+  return n;
+}
+
+// Their pulls.  Inside one fluid run, away from the periodic seam, the second
+// node's sources are those of the first moved by one; any other pair gathers
+// its nodes one by one.
+__device__ __forceinline__ void pair_pull(uint32_t k, const PairNodes& n, const float* __restrict__ fin,
+                                          const Layout& lay, const Params& p, F2 (&f)[9]) {
+  using L = D2Q9;
+  const size_t S = (size_t)lay.S;
+  const int x = (int)k + n.ra.xk;
+  if (n.same() && x > 0 && x + 1 < p.nx - 1) {
+    const float* __restrict__ fk = fin + k;
+    f[0].v = __ldg((const unsigned long long*)fk);
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      const int dx = -L::cx(i), dy = -L::cy(i);
+      const float* __restrict__ s =
+          fk + ((ptrdiff_t)i * (ptrdiff_t)S + (dy == 0 ? dx : n.ra.dbase[row_slot(dy, 0)] + dx));
+      f[i] = pack2(__ldg(s), __ldg(s + 1));
+    }
+  } else {
+    float a[9] = {0}, b[9] = {0};
+    if (n.fa()) pull_node<L>(fin, S, k, n.ra, lay, p, a);
+    if (n.fb()) pull_node<L>(fin, S, k + 1, n.rb, lay, p, b);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = pack2(a[i], b[i]);
+  }
+}
+
+// Their collision and store.
+template <bool MULTI>
+__device__ __forceinline__ void pair_finish(uint32_t k, bool live, const PairNodes& n, F2 (&f)[9],
+                                            float* __restrict__ fout, const Layout& lay,
+                                            Mom4<float>* __restrict__ mom, const Params& p) {
+  const size_t S = (size_t)lay.S;
+  const bool fa = n.fa(), fb = n.fb();
+  const int da = n.ra.dom, db = n.rb.dom;
+  const Relax xa = MULTI ? relax_domain(lay.dom, da) : relax_params(p);
+  bool force = xa.has_force != 0;
+  Bgk32<float> ca, cb;
+  if (MULTI && da != db) {
+    const Relax xb = relax_domain(lay.dom, db);
+    force = force || xb.has_force != 0;
+    ca = bgk32_params(p.rho0_f, xa, folded_of<MULTI>(p, lay, da), force);
+    cb = bgk32_params(p.rho0_f, xb, folded_of<MULTI>(p, lay, db), force);
+  } else {
+    ca = cb = bgk32_params(p.rho0_f, xa, folded_of<MULTI>(p, lay, da), force);
+  }
+  F2 r, ux, uy;
+  bgk_d2q9(f, bgk32_pair(ca, cb, force), force, r, ux, uy);
+  if ((n.w.x & W_CACHE) && fa) mom[k] = Mom4<float>{low(r), low(ux), low(uy), 0.f};
+  if ((n.w.y & W_CACHE) && fb) mom[k + 1] = Mom4<float>{high(r), high(ux), high(uy), 0.f};
+  float* __restrict__ ok = fout + k;
+  if (fa && fb) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) *(unsigned long long*)(ok + (size_t)i * S) = f[i].v;
+  } else if (live) {
+    // ghost slots take zeros (whole sectors), open slots their neighbour's thread
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      if (!(n.w.x & W_OPEN)) ok[(size_t)i * S] = fa ? low(f[i]) : 0.f;
+      if (!(n.w.y & W_OPEN)) ok[(size_t)i * S + 1] = fb ? high(f[i]) : 0.f;
+    }
+  }
+  if (p.inlet | p.outlet) {
+    if (fa) open_ends<D2Q9, F32S>(fout, mom, S, k, n.ra, lay, p);
+    if (fb) open_ends<D2Q9, F32S>(fout, mom, S, k + 1, n.rb, lay, p);
+  }
+}
+
+template <bool MULTI>
+__device__ __forceinline__ void bulk_pair(uint32_t k, bool live, const float* __restrict__ fin,
+                                          float* __restrict__ fout, const Layout& lay, Mom4<float>* __restrict__ mom,
+                                          const Params& p) {
+  const PairNodes n = pair_nodes(k, live, lay);
+  wait_for_previous();
+  F2 f[9];
+  pair_pull(k, n, fin, lay, p, f);
+  pair_finish<MULTI>(k, live, n, f, fout, lay, mom, p);
+}
+
 // Block (0) also clears the force slot of the next step.
 template <class L, class P, bool MULTI, int BT, int NPT>
 __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_bulk(const typename P::T* __restrict__ fin,
@@ -700,6 +853,14 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_b
                                                                        double* __restrict__ force_next, Params p) {
   let_next_start();
   const uint32_t t = blockIdx.x * BT + threadIdx.x;
+  if constexpr (NPT == 2 && P::shifted && L::Q == 9) {
+    if (p.collision == 0) {
+      prefetch_ahead<L::Q>(fin, lay, 2ull * blockIdx.x * BT, 2 * BT, threadIdx.x, BT);
+      bulk_pair<MULTI>(2 * t, 2ull * t < (uint64_t)lay.S, fin, fout, lay, mom, p);
+      clear_force<BT>(force_next, p.nbody);
+      return;
+    }
+  }
   const uint32_t stride = (uint32_t)(((size_t)lay.S + NPT - 1) / NPT);
   uint32_t k[NPT];
   bool live[NPT];
@@ -1407,6 +1568,18 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
   const int64_t nlb = spread ? lay.nlinked : (lay.nlinked + NW - 1) / NW;  // blocks with links
   if ((int64_t)blockIdx.x >= nlb) {
     const int64_t at = lay.nlinked + (((int64_t)blockIdx.x - nlb) * NW + warp) * NF;
+    if constexpr (P::shifted) {
+      if (p.collision == 0) {
+        // two groups a warp, a pair of neighbours a lane
+        const int64_t mine = at + (lane >> 4);
+        const bool some = mine < lay.ngroups;
+        const uint32_t k = (some ? 32u * __ldg(lay.groups + mine) : 0u) + 2u * (lane & 15);
+        prefetch_ahead<L::Q>(fin, lay, k & ~31u, 32, lane & 15, 16);
+        bulk_pair<MULTI>(k, some, fin, fout, lay, mom_out, p);
+        clear_force<BT>(force_next, p.nbody);
+        return;
+      }
+    }
     uint32_t k[NF];
     bool live[NF];
 #pragma unroll
