@@ -188,14 +188,17 @@ __global__ void __launch_bounds__(256, (adj_bulk_blocks_per_sm<L, P>())) k_adj_b
   using T = typename P::T;
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   const size_t S = (size_t)lay.S;
+  let_next_start();
+  const uint32_t w = k < (uint64_t)lay.S ? __ldg(lay.word + k) : W_GHOST;
+  RunRec run{};
+  if (!(w & (W_GHOST | W_OPEN))) run = lay.runs[w & W_RUN];
+  wait_for_previous();
   prefetch_ahead<L::Q>(fin, lay, k & ~31u, 32, threadIdx.x & 31, 32);
   prefetch_ahead<L::Q>((const T*)lam_next, lay, k & ~31u, 32, threadIdx.x & 31, 32);
   T dt = 0;
   int key = -1;
-  if (k < (uint64_t)lay.S) {
-    const uint32_t w = lay.word[k];
+  {
     if (!(w & (W_GHOST | W_OPEN))) {
-      const RunRec run = lay.runs[w & W_RUN];
       key = lay.ndom > 1 ? run.dom : 0;
       const Relax rx = lay.ndom > 1 ? relax_domain(lay.dom, key) : relax_params(p);
       int d[L::Q];
@@ -315,6 +318,7 @@ __device__ __forceinline__ void adj_link(int64_t k, const DirTable<typename P::T
     uw1 = uwv[nl + k];
     if (L::D == 3) uw2 = uwv[2 * nl + k];
   }
+  wait_for_previous();
   T om = lam[(size_t)i * S + ks];  // weight of this link's value (consumed here)
   if (final_step && body >= 0) {
     // J = w_b . sum (f+_i'(x_f) + L) e_i'
@@ -443,12 +447,17 @@ __global__ void __launch_bounds__(256) k_adj_links(const typename P::T* __restri
                                                    const typename P::T* __restrict__ uwv, int64_t nl, Params p,
                                                    int64_t S_, double* __restrict__ dq_acc, int final_step,
                                                    const double* __restrict__ wbody) {
+  let_next_start();
   __shared__ DirTable<typename P::T, L::Q> tab;
   fill_dir_table<L>(tab);
   __syncthreads();
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   MomAdj<typename P::T> ma{~0u, 0, 0, 0, 0, {0, 0, 0, 0}, 1};
-  if (k < nl) adj_link<L, P>(k, tab, f, mom, lam, lam_in, recs, qv, uwv, nl, p, S_, dq_acc, final_step, wbody, ma);
+  // (waits for its predecessor once its record is there)
+  if (k < nl)
+    adj_link<L, P>(k, tab, f, mom, lam, lam_in, recs, qv, uwv, nl, p, S_, dq_acc, final_step, wbody, ma);
+  else
+    wait_for_previous();
   spread_moment_adjoints<L>(lam, (size_t)S_, ma);
 }
 
@@ -552,15 +561,20 @@ __global__ void __launch_bounds__(256) k_adj_links_open(const typename P::T* __r
                                                         const typename P::T* __restrict__ uwv, int64_t nl, Params p,
                                                         int64_t S_, double* __restrict__ dq_acc, int final_step,
                                                         const double* __restrict__ wbody, Layout lay, int nbo) {
+  let_next_start();
   if ((int)blockIdx.x >= nbo) {
     __shared__ DirTable<typename P::T, L::Q> tab;
     fill_dir_table<L>(tab);
     __syncthreads();
     const int64_t k = (blockIdx.x - nbo) * (int64_t)blockDim.x + threadIdx.x;
     MomAdj<typename P::T> ma{~0u, 0, 0, 0, 0, {0, 0, 0, 0}, 1};
-    if (k < nl) adj_link<L, P>(k, tab, f, mom, lam, lam_in, recs, qv, uwv, nl, p, S_, dq_acc, final_step, wbody, ma);
+    if (k < nl)
+      adj_link<L, P>(k, tab, f, mom, lam, lam_in, recs, qv, uwv, nl, p, S_, dq_acc, final_step, wbody, ma);
+    else
+      wait_for_previous();
     spread_moment_adjoints<L>(lam, (size_t)S_, ma);
   } else {
+    wait_for_previous();
     adj_open_row<L, P>((int)(blockIdx.x * blockDim.x + threadIdx.x), lam, lam_in, mom, lay, p);
   }
 }
@@ -580,6 +594,12 @@ __global__ void __launch_bounds__(256) k_adj_init(const typename P::T* __restric
     const uint32_t run = lay.word[k] & W_RUN;
     key = lay.ndom > 1 ? lay.runs[run].dom : 0;
     const Relax rx = relax_of_run(p, lay, run);
+    // without a force u = u_in, and f+(0) = feq whatever tau is (3.4 ms of FP64
+    // zeros on 96 channels)
+    if (!rx.has_force) key = -1;
+  }
+  if (key >= 0) {
+    const Relax rx = relax_of_run(p, lay, lay.word[k] & W_RUN);
     const double g[3] = {rx.g[0], rx.g[1], rx.g[2]};
     double r = 0.0, j[3] = {0.0, 0.0, 0.0};
 #pragma unroll
@@ -631,25 +651,23 @@ struct AdjointLaunch {
   static void bulk(const void* fin, void* lam_next, void* lam_out, const Layout& lay, const Params& p, double* dtau,
                    void* mom, cudaStream_t s) {
     if (lay.S == 0) return;
-    k_adj_bulk<L, P><<<blocks_for(lay.S, 256), 256, 0, s>>>((const T*)fin, (T*)lam_next, (T*)lam_out, lay, p, dtau,
-                                                           (Mom4<T>*)mom);
+    launch_early(k_adj_bulk<L, P>, blocks_for(lay.S, 256), 256, s, (const T*)fin, (T*)lam_next, (T*)lam_out, lay, p, dtau,
+                 (Mom4<T>*)mom);
   }
   static void links(const void* f, const void* mom, void* lam, void* lam_in, const LinkRec* recs, const void* q,
                     const void* uw, int64_t nl, const Params& p, int64_t S, double* dq_acc, int final_step,
                     const double* wbody, cudaStream_t s) {
     if (nl == 0) return;
-    k_adj_links<L, P><<<blocks_for(nl, 256), 256, 0, s>>>((const T*)f, (const Mom4<T>*)mom, (T*)lam, (T*)lam_in,
-                                                         recs, (const T*)q, (const T*)uw, nl, p, S, dq_acc,
-                                                         final_step, wbody);
+    launch_early(k_adj_links<L, P>, blocks_for(nl, 256), 256, s, (const T*)f, (const Mom4<T>*)mom, (T*)lam, (T*)lam_in,
+                 recs, (const T*)q, (const T*)uw, nl, p, S, dq_acc, final_step, wbody);
   }
   static void links_open(const void* f, const void* mom, void* lam, void* lam_in, const LinkRec* recs, const void* q,
                          const void* uw, int64_t nl, const Params& p, int64_t S, double* dq_acc, int final_step,
                          const double* wbody, const Layout& lay, cudaStream_t s) {
     const int nbl = (int)blocks_for(nl, 256);
     const int nbo = (int)blocks_for(2 * (int64_t)p.ny, 256);
-    k_adj_links_open<L, P><<<nbl + nbo, 256, 0, s>>>((const T*)f, (const Mom4<T>*)mom, (T*)lam, (T*)lam_in, recs,
-                                                     (const T*)q, (const T*)uw, nl, p, S, dq_acc, final_step, wbody,
-                                                     lay, nbo);
+    launch_early(k_adj_links_open<L, P>, (unsigned)(nbl + nbo), 256, s, (const T*)f, (const Mom4<T>*)mom, (T*)lam,
+                 (T*)lam_in, recs, (const T*)q, (const T*)uw, nl, p, S, dq_acc, final_step, wbody, lay, nbo);
   }
   static void open(void* lam, void* lam_in, const void* mom, const Layout& lay, const Params& p, cudaStream_t s) {
     k_adj_open<L, P><<<blocks_for(2 * (int64_t)p.ny, 128), 128, 0, s>>>((T*)lam, (T*)lam_in, (const Mom4<T>*)mom, lay, p);

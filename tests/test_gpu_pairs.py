@@ -1,0 +1,109 @@
+"""D2Q9 step kernels at their edges: pairs of neighbouring nodes against one
+node per thread (FP32 BGK: the same bits), groups with links taken by a warp or
+by a whole block, and open columns written by their neighbours' threads."""
+import numpy as np
+import pytest
+
+from paper_1903_01111_gb300 import batch as B
+from paper_1903_01111_gb300 import geometry as G
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1903_01111_gb300 import lbm
+
+    return lbm
+
+
+def _start(geo, seed):
+    rng = np.random.default_rng(seed)
+    u = np.zeros((geo.N, 3))
+    u[:, :2] = rng.uniform(-0.03, 0.03, (geo.N, 2))
+    u[geo.solid != 0] = 0
+    return 1.0 + rng.uniform(-0.01, 0.01, geo.N), u
+
+
+def _run(L, geo, steps, domains=None, tuning=None, **kw):
+    lat = L.Lattice(geo, domains=domains, **kw)
+    if tuning:
+        lat.set_tuning(**tuning)
+    lat.init_equilibrium(*_start(geo, 3))
+    lat.step(steps)
+    out = lat.distributions(), lat.forces()
+    lat.close()
+    return out
+
+
+def _geometries():
+    yield "box 1x1", G.build(0, (1, 1, 1), (1, 1, 1), []), None, {}
+    yield "box 2x3", G.build(0, (2, 3, 1), (1, 1, 1), []), None, {}
+    yield "box 31x5", G.build(0, (31, 5, 1), (1, 1, 1), []), None, {}
+    yield "box 33x64", G.build(0, (33, 64, 1), (1, 1, 1), []), None, {}
+    yield "rotor 45x33", G.build(0, (45, 33, 1), (1, 1, 1), [G.ball((20.37, 15.61, 0), 6.3, omega=(0, 0, 0.004))]), None, {}
+    geo = G.cylinder_channel(nx=121, ny_fluid=30, center=(30.37, 15.61), radius=4.3)
+    yield "channel", geo, None, dict(inlet_umax=0.05, inlet_y0=0.5, inlet_y1=30.5)
+    b = B.stack(B.draw_channels(3, seed=2, nx_range=(40, 61), ny_range=(24, 31), r_range=(3.0, 4.0), n_cyl=(1, 2)))
+    yield "batch", b.geometry, b.domains, dict(inlet_y0=0.0, inlet_y1=1.0)
+
+
+CASES = list(_geometries())
+
+
+@pytest.mark.parametrize("g", [(0.0, 0.0, 0.0), (2e-5, -1e-5, 0.0)])
+@pytest.mark.parametrize("case", range(len(CASES)), ids=[c[0] for c in CASES])
+def test_pairs_have_the_bits_of_single_nodes(L, case, g):
+    _, geo, domains, kw = CASES[case]
+    if domains is not None:
+        domains = [dict(d, g=g) for d in domains]
+    ref = None
+    for shape in (1, 0, 2, 3, 4, 5, 6, 7):
+        f, F = _run(L, geo, 7, domains, dict(bulk_shape=shape, fused=0), precision=L.LBM_FP32_SHIFTED, tau=0.7, g=g, **kw)
+        if ref is None:
+            ref = f
+        assert np.array_equal(f, ref), shape
+
+
+@pytest.mark.parametrize("collision", ["bgk", "mrt"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32s"])
+@pytest.mark.parametrize("name", ["whole blocks", "warps", "warps, one body per wall"])
+def test_linked_groups_by_warps_and_by_blocks(L, name, prec, collision):
+    """The step with the links in the pull pass against the link kernel and the
+    bulk pass: few groups with links (a block on each) and more than the chip
+    holds blocks (a warp on each); FP64 differs in the order of a few roundings
+    (20 steps, 1e-13), FP32 by 4 steps eps of the deviations, as in the parity
+    tests."""
+    if name == "whole blocks":
+        geo = G.cylinder_channel(nx=200, ny_fluid=40, center=(50.37, 20.61), radius=6.3)
+    else:
+        two = name != "warps"
+        geo = G.channel(0, 6007, 24, q_lo=0.3, q_hi=0.7, u_hi=(0.01, 0, 0), force_lo=0, force_hi=1 if two else 0)
+    kw = dict(precision=L.LBM_FP64 if prec == "fp64" else L.LBM_FP32_SHIFTED, tau=0.7,
+              collision=L.LBM_MRT if collision == "mrt" else L.LBM_BGK)
+    if geo.open_x[0]:
+        kw.update(inlet_umax=0.05, inlet_y0=0.5, inlet_y1=40.5)
+    else:
+        kw.update(g=(1e-5, 0, 0))
+    steps = 20
+    (fa, Fa), (fb, Fb) = (_run(L, geo, steps, None, dict(bulk_shape=1, fused=k), **kw) for k in (1, 0))
+    w = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None]
+    fl = geo.solid == 0
+    if prec == "fp64":
+        tol = 1e-13
+    else:
+        tol = 4 * steps * float(np.finfo(np.float32).eps) * np.abs((fb - w)[:, fl]).max()
+    assert np.abs(fa - fb).max() <= tol
+    assert np.abs(Fa - Fb).max() <= max(np.abs(Fb).max(), 1e-3) * (1e-10 if prec == "fp64" else 1e-4) + len(geo.links) * tol
+    # the monitored loop leaves the same state and the last force
+    lat = L.Lattice(geo, **kw)
+    lat.set_tuning(bulk_shape=1, fused=1)
+    lat.init_equilibrium(*_start(geo, 3))
+    series = lat.step_forces(steps, 0)
+    assert np.array_equal(lat.distributions(), fa)
+    np.testing.assert_allclose(series[-1], lat.force(0), rtol=0, atol=0)
+    lat.close()
