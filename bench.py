@@ -488,7 +488,7 @@ def run_batch(lbm, torch, peak, n_domains=256, seed=0, steps=2000, warmup=10, ad
     nf = b.n_fluid
     s = 4
     fused = bool(tuning.fused) and info.n_links > 0
-    main_name = "k_fused" if fused else "k_bulk"
+    main_name = "k_inline" if fused else "k_bulk"
     main_ms = kms[2] / max(nlaunch[2], 1)
     main_bytes = nf * (2 * 9 * s + 1) + info.n_cached * 4 * s
     if fused:

@@ -169,26 +169,33 @@ typedef struct {
  *                 then (128,1) with each thread walking 4 or 8 nodes in
  *                 sequence over the grid, the next node's addressing loaded
  *                 while the current node's pulls are in flight;
- *                 3..7 are D2Q9 only.  -1 on input: the stencil's default,
- *                 3 for D2Q9 and 1 for D3Q19 (the shape a new lattice has).
+ *                 3..7 are D2Q9 only (FP32 BGK with two nodes per thread
+ *                 takes neighbours, in packed arithmetic; the other kinds
+ *                 nodes half a lattice apart).  -1 on input: the shape a new
+ *                 lattice has, 4 for D2Q9 FP32 and 1 otherwise.
  *  link_threads   64, 128 or 256 threads per block of the link kernel.
  *  graph_steps    time steps per CUDA graph replayed by lbm_step (even,
- *                 2..64).
+ *                 2..64); at 2 (the default) steps are launched one by one,
+ *                 each letting the next start early, without a graph.
  *  link_seq       links per thread of the link kernel, 1 or 4 (a block
  *                 takes link_seq rounds of consecutive links, loading the
  *                 next round's record while it evaluates the current one);
  *                 0 on input means 1.
- *  fused          1 (the default): a lattice with cut links runs each step
- *                 as one kernel: a block stages its nodes' pulls in shared
- *                 memory, evaluates the link rules of its nodes into the
- *                 staged slots of the link directions and collides from
- *                 there (the link values never go through device memory);
- *                 the bulk shape then only gives its threads per block (256
- *                 for the shapes with two or sequential nodes per thread).
+ *  fused          1: a lattice with cut links runs each step
+ *                 as one kernel.  D3Q19: a block stages its nodes' pulls in
+ *                 shared memory, evaluates the link rules of its nodes into
+ *                 the staged slots of the link directions and collides from
+ *                 there; D2Q9: the groups of nodes that have links evaluate
+ *                 them beside their pulls (either way the link values never
+ *                 go through device memory); the bulk shape then only gives
+ *                 its threads per block.
  *                 0: a link kernel writes each link's value into the ghost
  *                 slot of its solid neighbour and the bulk kernel pulls it
  *                 (the adjoint's recompute always takes this form).  Both
- *                 give the same populations up to rounding.
+ *                 give the same populations up to rounding.  A new lattice
+ *                 has 1, but 0 in FP64 D3Q19 (with 64 link threads) and on
+ *                 D2Q9 FP32 lattices of which more than 1 in 12 groups of 32
+ *                 stored nodes has links, unless the caller set it.
  * Shapes of the same kernel (same nodes per thread in parallel and in
  * sequence, same links per thread) give the same bits (force sums may differ
  * in the last place, as FP64 atomics are unordered); different kernels are
@@ -267,13 +274,14 @@ lbm_status lbm_forces(lbm_handle h, int32_t n, double* F);
 
 /* n >= 0 steps as lbm_step, with the force on body `body` after each of
  * them (lbm_force of that step) written to F[3*k + a], k = 0 .. n-1: a
- * monitoring loop without a host synchronisation per step.  Each step's
- * force is copied behind that step on the lattice's stream into a pinned
- * staging buffer the lattice owns (grown to at most 4096 steps x 3
- * doubles), so the device runs the steps back to back; the call waits once
- * per 4096 steps and returns when every value has landed.  Steps run one
- * launch sequence each (no multi-step graphs), so states and forces are
- * those of lbm_step(1) repeated, bit for bit.  F: 3 n doubles on the host;
+ * monitoring loop without a host synchronisation per step.  A chunk of
+ * steps (at most 4096, and 8 MB of force slots) adds its forces into slots
+ * of their own, copied once behind it on the lattice's stream into a pinned
+ * staging buffer the lattice owns, so the device runs the steps back to back;
+ * the call waits once per chunk and returns when every value has landed.
+ * Steps run one launch sequence each (no multi-step graphs), so states are
+ * those of lbm_step(1) repeated, bit for bit, and forces to the order of
+ * their FP64 atomics.  F: 3 n doubles on the host;
  * a body without links gives zeros.
  * Errors: STATE (no state), INVALID_ARG, OOM, CUDA. */
 lbm_status lbm_step_forces(lbm_handle h, int64_t n, int32_t body, double* F);
@@ -336,8 +344,9 @@ lbm_status lbm_query(lbm_handle h, lbm_info* info);
 /* Kernel timing for measurement.  While on, lbm_step launches the kernels
  * one by one (no CUDA graph) with a CUDA event pair around each launch on
  * the lattice's stream.  lbm_kernel_times synchronises and returns, per
- * kernel k (0 = links, 1 = open columns, 2 = bulk, or the fused step kernel
- * when the tuning's fused form runs, in which case slot 0 stays empty), the
+ * kernel k (0 = links, 1 = open columns (empty: the step kernels fill them),
+ * 2 = bulk, or the fused step kernel when the tuning's fused form runs, in
+ * which case slot 0 stays empty), the
  * number of timed launches and their summed duration in milliseconds since
  * profiling was switched on.  Errors: STATE, CUDA, OOM. */
 lbm_status lbm_set_profiling(lbm_handle h, int32_t on);

@@ -10,7 +10,8 @@
 // f+(s) before the adjoint step), so that every dependence is through f+(s).
 //
 // Per step (one stream, in this order):
-//   k_adj_bulk   per fluid node x: pre-collision f(s+1) from the pull sources
+//   k_adj_bulk   (FP32 D2Q9: k_adj_pair, two neighbouring nodes a thread)
+//                per fluid node x: pre-collision f(s+1) from the pull sources
 //                (ghost slots hold the link values of step s), the collision
 //                transpose mu = (dC/df)^T lambda(s+1)(x), and mu_i scattered to
 //                the pull source of direction i -- streaming is a permutation,
@@ -171,13 +172,12 @@ __device__ __forceinline__ void block_add_keyed(T v, int key, double* target) {
   }
 }
 
-// Resident 256-thread blocks per SM of the adjoint bulk kernel: 5 (48
-// registers, a few spilled words) for FP32 D2Q9 — measured faster than 4 at
-// 64 registers on the channel batch (backward 0.667 -> 0.641 ms per step) —,
-// 2 (up to 128 registers) for FP64 D2Q9 and FP32 D3Q19, 1 for FP64 D3Q19.
+// Resident 256-thread blocks per SM of the adjoint bulk kernel: 2 (up to 128
+// registers) for FP64 D2Q9 and FP32 D3Q19, 1 for FP64 D3Q19.  FP32 D2Q9 runs
+// k_adj_pair.
 template <class L, class P>
 constexpr int adj_bulk_blocks_per_sm() {
-  return L::Q == 9 ? (P::shifted ? 5 : 2) : (P::shifted ? 2 : 1);
+  return L::Q == 9 || P::shifted ? 2 : 1;
 }
 
 template <class L, class P>
@@ -231,6 +231,103 @@ __global__ void __launch_bounds__(256, (adj_bulk_blocks_per_sm<L, P>())) k_adj_b
     }
   }
   block_add_keyed<T>(dt, key, dtau);
+}
+
+// As k_adj_bulk for FP32 D2Q9, two neighbouring nodes a thread in packed
+// arithmetic (pair32.cuh): the bytes bound it, but one node a lane spent 565
+// instructions per 32 nodes on them, 56 % of the issue slots.  Batch of 64
+// channels, 64 steps: 6.85 -> 6.02 ms for the sweep's adjoint part; channel
+// 1024 x 256, 200 steps: 3.41 -> 3.08 ms.  10 blocks of 64 threads an SM (96
+// registers); with blocks of 128: 5 an SM 6.16 / 3.04 ms, 6 (80 registers)
+// 6.10 / 3.23, 7 6.17 / 3.45.
+template <class P>
+__global__ void __launch_bounds__(64, 10) k_adj_pair(const float* __restrict__ fin, float* __restrict__ lam_next,
+                                                     float* __restrict__ lam_out, Layout lay, Params p,
+                                                     double* __restrict__ dtau, Mom4<float>* __restrict__ mom) {
+  using L = D2Q9;
+  let_next_start();
+  const uint32_t k = 2u * (blockIdx.x * blockDim.x + threadIdx.x);
+  const size_t S = (size_t)lay.S;
+  const bool live = (uint64_t)k < (uint64_t)lay.S;
+  const PairNodes n = pair_nodes(k, live, lay);
+  const bool fa = n.fa(), fb = n.fb();
+  wait_for_previous();
+  {
+    const int lane = threadIdx.x & 31;
+    prefetch_ahead<L::Q>(fin, lay, k & ~63u, 64, lane, 32);
+    prefetch_ahead<L::Q>((const float*)lam_next, lay, k & ~63u, 64, lane, 32);
+  }
+  float dt = 0.f;
+  int key = -1;
+  if (fa || fb) {
+    F2 f[9], lam[9], mu[9];
+    pair_pull(k, n, fin, lay, p, f);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) lam[i].v = *(const unsigned long long*)(lam_next + (size_t)i * S + k);
+    // moments of f+(s) at cached nodes (the k_refresh formula)
+    auto refresh = [&](uint32_t m, const Relax& rx) {
+      float r = 0, jx = 0, jy = 0;
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        const float v = fin[(size_t)i * S + m];
+        r += v;
+        jx += (float)L::cx(i) * v;
+        jy += (float)L::cy(i) * v;
+      }
+      const float rho = p.rho0_f + r;
+      mom[m] = Mom4<float>{r, (jx - rx.hg_f[0]) / rho, (jy - rx.hg_f[1]) / rho, 0.f};
+    };
+    const bool multi = lay.ndom > 1;
+    const int da = fa ? n.ra.dom : n.rb.dom, db = fb ? n.rb.dom : da;
+    const Relax xa = multi ? relax_domain(lay.dom, da) : relax_params(p);
+    const Relax xb = multi && db != da ? relax_domain(lay.dom, db) : xa;
+    if (fa && (n.w.x & W_CACHE)) refresh(k, xa);
+    if (fb && (n.w.y & W_CACHE)) refresh(k + 1, xb);
+    const bool force = xa.has_force != 0 || xb.has_force != 0;
+    Bgk32<F2> c;
+    c.rho0 = Num<F2>::all(p.rho0_f);
+    c.om = pack2(xa.omega_f, xb.omega_f);
+    if (force) {
+      c.hx = pack2(xa.hg_f[0], xb.hg_f[0]);
+      c.hy = pack2(xa.hg_f[1], xb.hg_f[1]);
+      c.gx = pack2(xa.g_f[0], xb.g_f[0]);
+      c.gy = pack2(xa.g_f[1], xb.g_f[1]);
+    }
+    const F2 t = adjoint_d2q9(f, lam, mu, c, force);
+    // a pair across two domains adds its second node's term by itself
+    key = multi ? da : 0;
+    dt = fa ? low(t) : 0.f;
+    if (fb) {
+      if (db == da || !multi)
+        dt += high(t);
+      else
+        atomicAdd(dtau + db, (double)high(t));
+    }
+    const int x = (int)k + n.ra.xk;
+    if (n.same() && x > 0 && x + 1 < p.nx - 1) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        const int dx = -L::cx(i), dy = -L::cy(i);
+        float* __restrict__ o =
+            lam_out + k + ((ptrdiff_t)i * (ptrdiff_t)S + (dy == 0 ? dx : n.ra.dbase[row_slot(dy, 0)] + dx));
+        o[0] = low(mu[i]);
+        o[1] = high(mu[i]);
+      }
+    } else {
+      int d[9];
+      if (fa) {
+        pull_offsets<L>(k, n.ra, lay, p, d);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) lam_out[(ptrdiff_t)i * (ptrdiff_t)S + (ptrdiff_t)k + d[i]] = low(mu[i]);
+      }
+      if (fb) {
+        pull_offsets<L>(k + 1, n.rb, lay, p, d);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) lam_out[(ptrdiff_t)i * (ptrdiff_t)S + (ptrdiff_t)k + 1 + d[i]] = high(mu[i]);
+      }
+    }
+  }
+  block_add_keyed<float>(dt, key, dtau);
 }
 
 // Adds (a_r, a_u) -- adjoints of a node's moments rho and u -- to all
@@ -651,8 +748,12 @@ struct AdjointLaunch {
   static void bulk(const void* fin, void* lam_next, void* lam_out, const Layout& lay, const Params& p, double* dtau,
                    void* mom, cudaStream_t s) {
     if (lay.S == 0) return;
-    launch_early(k_adj_bulk<L, P>, blocks_for(lay.S, 256), 256, s, (const T*)fin, (T*)lam_next, (T*)lam_out, lay, p, dtau,
-                 (Mom4<T>*)mom);
+    if constexpr (P::shifted && L::Q == 9)
+      launch_early(k_adj_pair<P>, blocks_for(lay.S / 2, 64), 64, s, (const float*)fin, (float*)lam_next,
+                   (float*)lam_out, lay, p, dtau, (Mom4<float>*)mom);
+    else
+      launch_early(k_adj_bulk<L, P>, blocks_for(lay.S, 256), 256, s, (const T*)fin, (T*)lam_next, (T*)lam_out, lay, p,
+                   dtau, (Mom4<T>*)mom);
   }
   static void links(const void* f, const void* mom, void* lam, void* lam_in, const LinkRec* recs, const void* q,
                     const void* uw, int64_t nl, const Params& p, int64_t S, double* dq_acc, int final_step,

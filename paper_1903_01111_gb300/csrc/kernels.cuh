@@ -16,23 +16,29 @@
 // fluid node; ghost slots are filled by the link kernel before the bulk
 // kernel pulls them.
 //
-// Step t -> t+1, on one stream, in one of two forms.  Fused (the default on
-// lattices with cut links): k_fused stages each block's pulls in shared
-// memory, evaluates the block's link rules into the staged slots and
-// collides (after k_open where there are open columns).  Split (the
-// adjoint's recompute, and wherever the autotuner finds it faster):
+// Every state of a lattice with open columns (D2Q9) holds them filled: by
+// k_open after the initialisation, by the threads of the nodes beside them in
+// every step (open_ends).
+//
+// Step t -> t+1, on one stream, in one of two forms.  Fused: D3Q19 k_fused
+// stages each block's pulls in shared memory, evaluates the block's link rules
+// into the staged slots and collides; D2Q9 k_inline does so for the groups of
+// nodes that have links and pulls the others straight.  Split (the adjoint's
+// recompute, FP64 D3Q19, D2Q9 lattices with links all over, and wherever the
+// autotuner finds it faster):
 //   k_links: per cut link (x_f, i'), the missing f_i(x_f, t+1), i = opp(i'),
 //            from f+ and the moment cache at x_f and x_ff (Sec. 3 and 3.1),
 //            written to the ghost slot f[i][k_s] (read only by x_f);
 //            momentum exchange force in FP64.
-//   k_open:  inlet/outlet columns (Sec. 4.3), D2Q9 only.
 //   k_bulk:  pull streaming f_i(x, t+1) = f+_i(x - e_i, t) (Eq. 1), moments,
 //            Guo-forced BGK (Sec. 2, Eq. feq) -> f+(t+1) into the other
 //            buffer; rho, u(t+1) into the moment cache where flagged.  Ghost
-//            and open slots of the output get zeros (through the same store
+//            slots of the output get zeros (through the same store
 //            instructions as the fluid slots) so that every written sector
 //            is complete.  FP64 one-node shapes run k_bulk_list instead, over
 //            the fluid nodes alone.
+// FP64 collides and evaluates VIBB links in 64-bit integers (fixed64.cuh),
+// FP32 D2Q9 BGK in packed pairs (pair32.cuh).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -44,18 +50,13 @@
 
 namespace lbm {
 
-// bulk_min_blocks: resident 256-thread blocks per SM the bulk kernel is
-// compiled for (FP32: 5, FP64: 2; 6 for FP32 forces spills and ran slower on
-// the porous workload).
 struct F64 {
   using T = double;
   static constexpr bool shifted = false;
-  static constexpr int bulk_min_blocks = 2;
 };
 struct F32S {
   using T = float;
   static constexpr bool shifted = true;
-  static constexpr int bulk_min_blocks = 5;
 };
 
 // One moment-cache record per node: (r, ux, uy, uz) with r = rho (F64) or
@@ -669,11 +670,10 @@ constexpr unsigned bulk_shape_mask() {
   return L::Q == 9 ? 0xffu : 0x07u;
 }
 
-// Default shape: two nodes per thread in 256-thread blocks for D2Q9; one
-// node per thread in 128-thread blocks for D3Q19 (the autotuner's choice on
-// dense and porous D3Q19 lattices in both precisions, and the fused step's
-// best block: 1.30 ms per step on a 384^3 pack against 1.37 at 256) and for
-// FP64 D2Q9 (integer collision: 280 us per step on 4097 x 2049 nodes against
+// Default shape, 128-thread blocks: two neighbouring nodes per thread for FP32
+// D2Q9 (8192 x 4096 nodes 382 us per step, 388 in 256-thread blocks, 408 with
+// one node per thread); one node per thread for D3Q19 (the fused step's best
+// block: 1.26 ms per step on a 384^3 pack against 1.33 at 256) and for FP64 D2Q9 (integer collision: 280 us per step on 4097 x 2049 nodes against
 // 339 with two nodes per thread, whose registers halve the warps in flight).
 template <class L, class P>
 constexpr int bulk_default_shape() {

@@ -135,6 +135,76 @@ __device__ __forceinline__ void bgk_d2q9(V (&f)[9], const Bgk32<V>& c, bool forc
   pair(6, 8, 2, w2, N::sub(uy, ux), 3);
 }
 
+// Transpose of the collision at one node or two (see collide_adjoint, whose
+// moments of d_i = lambda_i - mean lambda these are, with opposite directions
+// paired): mu from the pre-collision f and lambda(s+1); returns the node's
+// sum_i lambda_i dC_i/dtau.
+template <class V>
+__device__ __forceinline__ V adjoint_d2q9(const V (&f)[9], const V (&lam)[9], V (&mu)[9], const Bgk32<V>& c,
+                                          bool force) {
+  using N = Num<V>;
+  constexpr float w0 = (float)(4.0 / 9.0), w1 = (float)(1.0 / 9.0), w2 = (float)(1.0 / 36.0);
+  const V d13 = N::sub(f[1], f[3]), d24 = N::sub(f[2], f[4]), d57 = N::sub(f[5], f[7]), d68 = N::sub(f[6], f[8]);
+  const V r = N::add(f[0], N::add(N::add(N::add(f[1], f[3]), N::add(f[2], f[4])),
+                                  N::add(N::add(f[5], f[7]), N::add(f[6], f[8]))));
+  const V jx = N::add(d13, N::sub(d57, d68)), jy = N::add(d24, N::add(d57, d68));
+  const V rho = N::add(c.rho0, r);
+  V ir = N::rcp_seed(rho);
+  ir = N::fma(ir, N::fma(N::mul(rho, N::all(-1.f)), ir, N::all(1.f)), ir);
+  const V ux = N::mul(force ? N::add(jx, c.hx) : jx, ir), uy = N::mul(force ? N::add(jy, c.hy) : jy, ir);
+  const V nu = N::mul(N::all(-1.5f), N::fma(ux, ux, N::mul(uy, uy)));
+  const V lbar = N::mul(
+      N::all((float)(1.0 / 9.0)),
+      N::add(lam[0], N::add(N::add(N::add(lam[1], lam[3]), N::add(lam[2], lam[4])),
+                            N::add(N::add(lam[5], lam[7]), N::add(lam[6], lam[8])))));
+  V d[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) d[i] = N::sub(lam[i], lbar);
+  V lf = N::mul(d[0], f[0]);
+#pragma unroll
+  for (int i = 1; i < 9; ++i) lf = N::fma(d[i], f[i], lf);
+  const V p13 = N::add(d[1], d[3]), p24 = N::add(d[2], d[4]), p57 = N::add(d[5], d[7]), p68 = N::add(d[6], d[8]);
+  const V m57 = N::sub(d[5], d[7]), m68 = N::sub(d[6], d[8]);
+  const V diag = N::mul(N::all(w2), N::add(p57, p68));
+  const V S0 = N::fma(N::all(w0), d[0], N::fma(N::all(w1), N::add(p13, p24), diag));
+  const V Sx = N::fma(N::all(w1), N::sub(d[1], d[3]), N::mul(N::all(w2), N::sub(m57, m68)));
+  const V Sy = N::fma(N::all(w1), N::sub(d[2], d[4]), N::mul(N::all(w2), N::add(m57, m68)));
+  const V Txx = N::fma(N::all(w1), p13, diag), Tyy = N::fma(N::all(w1), p24, diag);
+  const V Txy = N::mul(N::all(w2), N::sub(p57, p68));
+  const V Tux = N::fma(Txx, ux, N::mul(Txy, uy)), Tuy = N::fma(Txy, ux, N::mul(Tyy, uy));
+  const V uS = N::fma(ux, Sx, N::mul(uy, Sy)), uTu = N::fma(ux, Tux, N::mul(uy, Tuy));
+  const V dpoly = N::fma(nu, S0, N::fma(N::all(4.5f), uTu, N::mul(N::all(3.f), uS)));
+  const V A = N::add(N::add(S0, dpoly), lbar);
+  const V orho = N::mul(c.om, rho), s3 = N::mul(N::all(-3.f), S0);
+  V B0 = N::mul(orho, N::fma(s3, ux, N::fma(N::all(9.f), Tux, N::mul(N::all(3.f), Sx))));
+  V B1 = N::mul(orho, N::fma(s3, uy, N::fma(N::all(9.f), Tuy, N::mul(N::all(3.f), Sy))));
+  V dt = N::sub(lf, N::fma(rho, dpoly, N::mul(r, S0)));
+  if (force) {
+    const V c2 = N::fma(N::all(-0.5f), c.om, N::all(1.f));
+    const V Tgx = N::fma(Txx, c.gx, N::mul(Txy, c.gy)), Tgy = N::fma(Txy, c.gx, N::mul(Tyy, c.gy));
+    B0 = N::fma(c2, N::fma(s3, c.gx, N::mul(N::all(9.f), Tgx)), B0);
+    B1 = N::fma(c2, N::fma(s3, c.gy, N::mul(N::all(9.f), Tgy)), B1);
+    // sum d_i src_i = 3 g.S - 3 (u.g) S0 + 9 u.T.g
+    const V ug = N::fma(ux, c.gx, N::mul(uy, c.gy));
+    V src = N::mul(N::all(3.f), N::fma(c.gx, Sx, N::mul(c.gy, Sy)));
+    src = N::fma(N::all(9.f), N::fma(ux, Tgx, N::mul(uy, Tgy)), N::fma(s3, ug, src));
+    dt = N::fma(N::all(0.5f), src, dt);
+  }
+  const V om1 = N::sub(N::all(1.f), c.om), bx = N::mul(B0, ir), by = N::mul(B1, ir);
+  const V C = N::sub(N::mul(c.om, A), N::fma(bx, ux, N::mul(by, uy)));
+  mu[0] = N::fma(om1, lam[0], C);
+  mu[1] = N::fma(om1, lam[1], N::add(C, bx));
+  mu[3] = N::fma(om1, lam[3], N::sub(C, bx));
+  mu[2] = N::fma(om1, lam[2], N::add(C, by));
+  mu[4] = N::fma(om1, lam[4], N::sub(C, by));
+  const V s = N::add(bx, by), t = N::sub(bx, by);
+  mu[5] = N::fma(om1, lam[5], N::add(C, s));
+  mu[7] = N::fma(om1, lam[7], N::sub(C, s));
+  mu[8] = N::fma(om1, lam[8], N::add(C, t));
+  mu[6] = N::fma(om1, lam[6], N::sub(C, t));
+  return N::mul(dt, N::mul(c.om, c.om));
+}
+
 #endif  // __CUDACC__
 
 }  // namespace lbm

@@ -317,7 +317,7 @@ def lbm_forces(h, n: int) -> np.ndarray:
 
 def lbm_step_forces(h, n: int, body: int = 0) -> np.ndarray:
     """n steps, and the force (n, 3) on `body` after each of them (copied
-    behind each step, one synchronisation per 4096 steps)."""
+    behind a chunk of at most 4096 steps)."""
     out = np.zeros((max(int(n), 1), 3))
     _check(_lib.lbm_step_forces(h, int(n), int(body), out.ctypes.data))
     return out[:int(n)]
@@ -413,7 +413,7 @@ def _ptr_or_int(a):
 
 LBM_NOALLOC_MAX_LINKS = 16777216
 
-KERNEL_NAMES = ("k_links", "k_open", "k_bulk or k_fused")
+KERNEL_NAMES = ("k_links", "k_open", "k_bulk, k_fused or k_inline")
 
 
 class Lattice:

@@ -107,3 +107,36 @@ def test_linked_groups_by_warps_and_by_blocks(L, name, prec, collision):
     assert np.array_equal(lat.distributions(), fa)
     np.testing.assert_allclose(series[-1], lat.force(0), rtol=0, atol=0)
     lat.close()
+
+
+@pytest.mark.parametrize("g", [(0.0, 0.0, 0.0), (2e-5, -1e-5, 0.0)])
+@pytest.mark.parametrize("case", [c for c in range(len(CASES)) if not CASES[c][0].startswith("box")],
+                         ids=[c[0] for c in CASES if not c[0].startswith("box")])
+def test_adjoint_pairs_against_one_node_in_doubles(L, case, g):
+    """The FP32 D2Q9 adjoint (pairs; odd row lengths, seams, open columns,
+    domains with rates of their own) against FP64's one node per thread, every
+    link and every domain: 1e-3 of the largest entry, the bound of the FP32
+    adjoint test at 300 steps."""
+    _, geo, domains, kw = CASES[case]
+    if domains is not None:
+        domains = [dict(d, g=g) for d in domains]
+    out = []
+    for prec in (L.LBM_FP64, L.LBM_FP32_SHIFTED):
+        with L.Lattice(geo, domains=domains, precision=prec, tau=0.7, g=g, **kw) as lat:
+            lat.init_equilibrium(u=_smooth(geo))
+            w = np.tile([1.0, 0.3, 0.0], (lat.info().n_bodies, 1))
+            out.append(L.lbm_adjoint_step(lat.h, -1, w, 40, 9))
+    (_, qa, ta, _), (_, qb, tb, _) = out
+    assert np.abs(qa).max() > 0 and np.abs(qb - qa).max() <= 1e-3 * np.abs(qa).max()
+    ta, tb = np.atleast_1d(ta), np.atleast_1d(tb)
+    assert np.abs(ta).max() > 0 and np.abs(tb - ta).max() <= 1e-3 * np.abs(ta).max()
+
+
+def _smooth(geo):
+    x = np.arange(geo.N) % geo.nx
+    y = np.arange(geo.N) // geo.nx
+    u = np.zeros((geo.N, 3))
+    u[:, 0] = 0.03 + 0.01 * np.sin(2 * np.pi * y / geo.ny)
+    u[:, 1] = 0.01 * np.cos(2 * np.pi * x / geo.nx)
+    u[geo.solid != 0] = 0
+    return u
