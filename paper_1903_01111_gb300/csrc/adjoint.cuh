@@ -181,10 +181,10 @@ constexpr int adj_bulk_blocks_per_sm() {
 }
 
 template <class L, class P>
-__global__ void __launch_bounds__(256, (adj_bulk_blocks_per_sm<L, P>())) k_adj_bulk(const typename P::T* __restrict__ fin,
-                                                  typename P::T* __restrict__ lam_next,
-                                                  typename P::T* __restrict__ lam_out, Layout lay, Params p,
-                                                  double* __restrict__ dtau, Mom4<typename P::T>* __restrict__ mom) {
+__global__ void __launch_bounds__(256, (adj_bulk_blocks_per_sm<L, P>())) k_adj_bulk(const typename P::T* fin,
+                                                  typename P::T* lam_next,
+                                                  typename P::T* lam_out, Layout lay, Params p,
+                                                  double* dtau, Mom4<typename P::T>* __restrict__ mom) {
   using T = typename P::T;
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   const size_t S = (size_t)lay.S;
@@ -241,9 +241,9 @@ __global__ void __launch_bounds__(256, (adj_bulk_blocks_per_sm<L, P>())) k_adj_b
 // registers); with blocks of 128: 5 an SM 6.16 / 3.04 ms, 6 (80 registers)
 // 6.10 / 3.23, 7 6.17 / 3.45.
 template <class P>
-__global__ void __launch_bounds__(64, 10) k_adj_pair(const float* __restrict__ fin, float* __restrict__ lam_next,
+__global__ void __launch_bounds__(64, 10) k_adj_pair(const float* fin, float* lam_next,
                                                      float* __restrict__ lam_out, Layout lay, Params p,
-                                                     double* __restrict__ dtau, Mom4<float>* __restrict__ mom) {
+                                                     double* dtau, Mom4<float>* __restrict__ mom) {
   using L = D2Q9;
   let_next_start();
   const uint32_t k = 2u * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(64, 10) k_adj_pair(const float* __restrict__ f
 // Adds (a_r, a_u) -- adjoints of a node's moments rho and u -- to all
 // directions of that node: d rho/df+_j = 1, d u_a/df+_j = (e_ja - u_a)/rho.
 template <class L, class T>
-__device__ __forceinline__ void scatter_moment_adjoint(T* __restrict__ lam, size_t S, uint32_t k, T ar, T a0, T a1,
+__device__ __forceinline__ void scatter_moment_adjoint(T* lam, size_t S, uint32_t k, T ar, T a0, T a1,
                                                        T a2, const Mom4<T>& m, T rho) {
   const T ir = (T)1 / rho;
 #pragma unroll
@@ -365,7 +365,7 @@ struct MomAdj {
 // directions (one set of atomics per node instead of one per link).  All 32
 // lanes of the warp take part.
 template <class L, class T>
-__device__ __forceinline__ void spread_moment_adjoints(T* __restrict__ lam, size_t S, MomAdj<T> a) {
+__device__ __forceinline__ void spread_moment_adjoints(T* lam, size_t S, MomAdj<T> a) {
   const int lane = threadIdx.x & 31;
   const uint32_t prev = __shfl_up_sync(0xffffffffu, a.key, 1);
   const uint32_t next = __shfl_down_sync(0xffffffffu, a.key, 1);
@@ -391,11 +391,11 @@ __device__ __forceinline__ void spread_moment_adjoints(T* __restrict__ lam, size
 // adjoint of x_f's moments is left in ma (spread by the caller).
 template <class L, class P>
 __device__ __forceinline__ void adj_link(int64_t k, const DirTable<typename P::T, L::Q>& tab,
-                                         const typename P::T* __restrict__ f,
-                                         const Mom4<typename P::T>* __restrict__ mom, typename P::T* __restrict__ lam,
-                                         typename P::T* __restrict__ lam_in, const LinkRec* __restrict__ recs,
+                                         const typename P::T* f,
+                                         const Mom4<typename P::T>* mom, typename P::T* lam,
+                                         typename P::T* lam_in, const LinkRec* __restrict__ recs,
                                          const typename P::T* __restrict__ qv, const typename P::T* __restrict__ uwv,
-                                         int64_t nl, const Params& p, int64_t S_, double* __restrict__ dq_acc,
+                                         int64_t nl, const Params& p, int64_t S_, double* dq_acc,
                                          int final_step, const double* __restrict__ wbody,
                                          MomAdj<typename P::T>& ma) {
   using T = typename P::T;
@@ -536,13 +536,13 @@ __device__ __forceinline__ void adj_link(int64_t k, const DirTable<typename P::T
 // objective's direct terms J = sum_b wbody[b] . F_b(step) (wbody: [nbody][3]
 // FP64).
 template <class L, class P>
-__global__ void __launch_bounds__(256) k_adj_links(const typename P::T* __restrict__ f,
-                                                   const Mom4<typename P::T>* __restrict__ mom,
-                                                   typename P::T* __restrict__ lam, typename P::T* __restrict__ lam_in,
+__global__ void __launch_bounds__(256) k_adj_links(const typename P::T* f,
+                                                   const Mom4<typename P::T>* mom,
+                                                   typename P::T* lam, typename P::T* lam_in,
                                                    const LinkRec* __restrict__ recs,
                                                    const typename P::T* __restrict__ qv,
                                                    const typename P::T* __restrict__ uwv, int64_t nl, Params p,
-                                                   int64_t S_, double* __restrict__ dq_acc, int final_step,
+                                                   int64_t S_, double* dq_acc, int final_step,
                                                    const double* __restrict__ wbody) {
   let_next_start();
   __shared__ DirTable<typename P::T, L::Q> tab;
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(256) k_adj_links(const typename P::T* __restri
 // next to the open column in row y - cy(j) (table: row_in1 for the inlet,
 // cx = -1; row_out1 for the outlet, cx = +1).
 template <class L, class T>
-__device__ __forceinline__ void clear_open_neighbours(T* __restrict__ lam_in, const Layout& lay, const Params& p, int y,
+__device__ __forceinline__ void clear_open_neighbours(T* lam_in, const Layout& lay, const Params& p, int y,
                                                       int cx) {
   const int32_t* __restrict__ next = cx < 0 ? lay.row_in1 : lay.row_out1;
 #pragma unroll
@@ -586,8 +586,8 @@ __device__ __forceinline__ void clear_open_neighbours(T* __restrict__ lam_in, co
 // entries of lambda(s+1) (lam_in, read by k_adj_bulk) that point into an
 // open node.  t < ny: inlet of row t; ny <= t < 2 ny: outlet of row t - ny.
 template <class L, class P>
-__device__ __forceinline__ void adj_open_row(int t, typename P::T* __restrict__ lam, typename P::T* __restrict__ lam_in,
-                                             const Mom4<typename P::T>* __restrict__ mom, const Layout& lay,
+__device__ __forceinline__ void adj_open_row(int t, typename P::T* lam, typename P::T* lam_in,
+                                             const Mom4<typename P::T>* mom, const Layout& lay,
                                              const Params& p) {
   using T = typename P::T;
   if (t >= 2 * p.ny) return;
@@ -639,8 +639,8 @@ __device__ __forceinline__ void adj_open_row(int t, typename P::T* __restrict__ 
 }
 
 template <class L, class P>
-__global__ void k_adj_open(typename P::T* __restrict__ lam, typename P::T* __restrict__ lam_in,
-                           const Mom4<typename P::T>* __restrict__ mom, Layout lay, Params p) {
+__global__ void k_adj_open(typename P::T* lam, typename P::T* lam_in,
+                           const Mom4<typename P::T>* mom, Layout lay, Params p) {
   adj_open_row<L, P>(blockIdx.x * blockDim.x + threadIdx.x, lam, lam_in, mom, lay, p);
 }
 
@@ -649,14 +649,14 @@ __global__ void k_adj_open(typename P::T* __restrict__ lam, typename P::T* __res
 // accesses overlap the link blocks), the others the links (as
 // k_adj_links); the two parts touch common entries only through atomics.
 template <class L, class P>
-__global__ void __launch_bounds__(256) k_adj_links_open(const typename P::T* __restrict__ f,
-                                                        const Mom4<typename P::T>* __restrict__ mom,
-                                                        typename P::T* __restrict__ lam,
-                                                        typename P::T* __restrict__ lam_in,
+__global__ void __launch_bounds__(256) k_adj_links_open(const typename P::T* f,
+                                                        const Mom4<typename P::T>* mom,
+                                                        typename P::T* lam,
+                                                        typename P::T* lam_in,
                                                         const LinkRec* __restrict__ recs,
                                                         const typename P::T* __restrict__ qv,
                                                         const typename P::T* __restrict__ uwv, int64_t nl, Params p,
-                                                        int64_t S_, double* __restrict__ dq_acc, int final_step,
+                                                        int64_t S_, double* dq_acc, int final_step,
                                                         const double* __restrict__ wbody, Layout lay, int nbo) {
   let_next_start();
   if ((int)blockIdx.x >= nbo) {
@@ -680,8 +680,8 @@ __global__ void __launch_bounds__(256) k_adj_links_open(const typename P::T* __r
 // rho and u_in recovered from f+(0): rho = sum f+, u_in = (sum f+ e - g)/rho.
 template <class L, class P>
 __global__ void __launch_bounds__(256) k_adj_init(const typename P::T* __restrict__ f0,
-                                                  const typename P::T* __restrict__ lam, Layout lay, Params p,
-                                                  double* __restrict__ dtau) {
+                                                  const typename P::T* lam, Layout lay, Params p,
+                                                  double* dtau) {
   using T = typename P::T;
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   const size_t S = (size_t)lay.S;

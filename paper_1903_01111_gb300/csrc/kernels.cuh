@@ -179,7 +179,7 @@ struct __align__(16) LinkRec {
 // 399 / 407 at 1.4 / 2.8 / 5.6 / 11 MB; dense 301 x 257 x 259 506 -> 486, 526 at 24 MB
 // (the far half of L2 is used up); 384^3 pack 1298 -> 1266.
 template <int Q, class T>
-__device__ __forceinline__ void prefetch_ahead(const T* __restrict__ f, const Layout& lay, uint64_t k, int N, int t,
+__device__ __forceinline__ void prefetch_ahead(const T* f, const Layout& lay, uint64_t k, int N, int t,
                                                int nt) {
   constexpr int per = 128 / (int)sizeof(T);
   const uint64_t from = k + lay.ahead;
@@ -193,7 +193,7 @@ __device__ __forceinline__ void prefetch_ahead(const T* __restrict__ f, const La
 
 // Clears the force slot of the next step (the grid's first block).
 template <int BT>
-__device__ __forceinline__ void clear_force(double* __restrict__ force_next, int nbody) {
+__device__ __forceinline__ void clear_force(double* force_next, int nbody) {
   if (force_next && blockIdx.x == 0)
     for (int t = threadIdx.x; t < 3 * nbody; t += BT) force_next[t] = 0.0;
 }
@@ -203,6 +203,16 @@ __device__ __forceinline__ void clear_force(double* __restrict__ force_next, int
 // (node words, runs, link records) before it waits for the predecessor's
 // results.  On lattices that take microseconds a step the launch and those
 // loads are a third of it.
+//
+// A kernel started so is resident while its predecessor still writes the
+// populations, the moment cache and the multipliers it will read.  Such memory
+// is not read-only for the kernel's lifetime, so it is loaded by plain loads
+// after the wait, never by __ldg, and never through a __restrict__ pointer
+// (which lets the compiler take a non-coherent load, or move a load above the
+// wait): the wait makes the predecessor's writes visible to plain loads only.
+// __ldg and const __restrict__ are kept for what the host alone writes, and
+// __restrict__ for outputs of which a thread reads back no more than its own
+// stores.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -565,13 +575,13 @@ __device__ __forceinline__ void pull_offsets(uint32_t k, const RunRec& run, cons
 
 // The populations f_i(x, t+1) = f+_i(x - e_i, t) of fluid node k of run `run`.
 template <class L, class T>
-__device__ __forceinline__ void pull_node(const T* __restrict__ fin, size_t S, uint32_t k, const RunRec& run,
+__device__ __forceinline__ void pull_node(const T* fin, size_t S, uint32_t k, const RunRec& run,
                                           const Layout& lay, const Params& p, T (&f)[L::Q]) {
   int d[L::Q];
   pull_offsets<L>(k, run, lay, p, d);
-  const T* __restrict__ fk = fin + k;
+  const T* fk = fin + k;
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) f[i] = __ldg(fk + ((ptrdiff_t)i * (ptrdiff_t)S + d[i]));
+  for (int i = 0; i < L::Q; ++i) f[i] = fk[(ptrdiff_t)i * (ptrdiff_t)S + d[i]];
 }
 
 // ------------------------------------------------------------ open sides --
@@ -582,7 +592,7 @@ __device__ __forceinline__ void pull_node(const T* __restrict__ fin, size_t S, u
 // instructions of a warp); f and mom hold the state of the fluid node at x = 1,
 // adjacent in storage.
 template <class L, class P>
-__device__ __forceinline__ void fill_inlet(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom,
+__device__ __forceinline__ void fill_inlet(typename P::T* f, const Mom4<typename P::T>* mom,
                                            size_t S, uint32_t k0, int y, const Layout& lay, const Params& p) {
   using T = typename P::T;
   const T uin = ((const T*)lay.row_uin)[y];
@@ -600,7 +610,7 @@ __device__ __forceinline__ void fill_inlet(typename P::T* __restrict__ f, const 
 
 // Outlet column (storage kl): a copy of the fluid node before it.
 template <class L, class P>
-__device__ __forceinline__ void fill_outlet(typename P::T* __restrict__ f, size_t S, uint32_t kl) {
+__device__ __forceinline__ void fill_outlet(typename P::T* f, size_t S, uint32_t kl) {
   typename P::T v[L::Q];
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) v[i] = f[i * S + kl - 1];
@@ -632,7 +642,7 @@ __global__ void k_open(typename P::T* __restrict__ f, const Mom4<typename P::T>*
 // it stored k's state: the open columns of the next step cost no launch.  The
 // open slots' own threads store nothing.
 template <class L, class P>
-__device__ __forceinline__ void open_ends(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom,
+__device__ __forceinline__ void open_ends(typename P::T* f, const Mom4<typename P::T>* mom,
                                           size_t S, uint32_t k, const RunRec& run, const Layout& lay,
                                           const Params& p) {
   if constexpr (L::D == 2) {
@@ -699,7 +709,7 @@ constexpr int bulk_blocks_per_sm() {
 // node's collision reads its run's domain parameters.
 template <class L, class P, bool MULTI, int NPT>
 __device__ __forceinline__ void bulk_nodes(const uint32_t (&k)[NPT], const bool (&live)[NPT],
-                                           const typename P::T* __restrict__ fin, typename P::T* __restrict__ fout,
+                                           const typename P::T* fin, typename P::T* __restrict__ fout,
                                            const Layout& lay, Mom4<typename P::T>* __restrict__ mom, const Params& p) {
   using T = typename P::T;
   const size_t S = (size_t)lay.S;
@@ -769,20 +779,20 @@ __device__ __forceinline__ PairNodes pair_nodes(uint32_t k, bool live, const Lay
 // Their pulls.  Inside one fluid run, away from the periodic seam, the second
 // node's sources are those of the first moved by one; any other pair gathers
 // its nodes one by one.
-__device__ __forceinline__ void pair_pull(uint32_t k, const PairNodes& n, const float* __restrict__ fin,
+__device__ __forceinline__ void pair_pull(uint32_t k, const PairNodes& n, const float* fin,
                                           const Layout& lay, const Params& p, F2 (&f)[9]) {
   using L = D2Q9;
   const size_t S = (size_t)lay.S;
   const int x = (int)k + n.ra.xk;
   if (n.same() && x > 0 && x + 1 < p.nx - 1) {
-    const float* __restrict__ fk = fin + k;
-    f[0].v = __ldg((const unsigned long long*)fk);
+    const float* fk = fin + k;
+    f[0].v = *(const unsigned long long*)fk;
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
       const int dx = -L::cx(i), dy = -L::cy(i);
-      const float* __restrict__ s =
+      const float* s =
           fk + ((ptrdiff_t)i * (ptrdiff_t)S + (dy == 0 ? dx : n.ra.dbase[row_slot(dy, 0)] + dx));
-      f[i] = pack2(__ldg(s), __ldg(s + 1));
+      f[i] = pack2(s[0], s[1]);
     }
   } else {
     float a[9] = {0}, b[9] = {0};
@@ -835,7 +845,7 @@ __device__ __forceinline__ void pair_finish(uint32_t k, bool live, const PairNod
 }
 
 template <bool MULTI>
-__device__ __forceinline__ void bulk_pair(uint32_t k, bool live, const float* __restrict__ fin,
+__device__ __forceinline__ void bulk_pair(uint32_t k, bool live, const float* fin,
                                           float* __restrict__ fout, const Layout& lay, Mom4<float>* __restrict__ mom,
                                           const Params& p) {
   const PairNodes n = pair_nodes(k, live, lay);
@@ -847,10 +857,10 @@ __device__ __forceinline__ void bulk_pair(uint32_t k, bool live, const float* __
 
 // Block (0) also clears the force slot of the next step.
 template <class L, class P, bool MULTI, int BT, int NPT>
-__global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_bulk(const typename P::T* __restrict__ fin,
+__global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_bulk(const typename P::T* fin,
                                                                        typename P::T* __restrict__ fout, Layout lay,
                                                                        Mom4<typename P::T>* __restrict__ mom,
-                                                                       double* __restrict__ force_next, Params p) {
+                                                                       double* force_next, Params p) {
   let_next_start();
   const uint32_t t = blockIdx.x * BT + threadIdx.x;
   if constexpr (NPT == 2 && P::shifted && L::Q == 9) {
@@ -884,8 +894,8 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_b
 // written it, and the fluid node beside an open slot writes it.
 template <class L, class P, bool MULTI, int BT>
 __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, 1>())) k_bulk_list(
-    const typename P::T* __restrict__ fin, typename P::T* __restrict__ fout, Layout lay,
-    Mom4<typename P::T>* __restrict__ mom, double* __restrict__ force_next, Params p) {
+    const typename P::T* fin, typename P::T* __restrict__ fout, Layout lay,
+    Mom4<typename P::T>* __restrict__ mom, double* force_next, Params p) {
   using T = typename P::T;
   let_next_start();
   const int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
@@ -938,8 +948,8 @@ __device__ __forceinline__ RunLite<L> load_run_lite(const RunRec* __restrict__ r
 // record right after the current node's stores (D2Q9).
 template <class L, class P, bool MULTI, int BT, int SEQ>
 __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_seq(
-    const typename P::T* __restrict__ fin, typename P::T* __restrict__ fout, Layout lay,
-    Mom4<typename P::T>* __restrict__ mom, double* __restrict__ force_next, Params p) {
+    const typename P::T* fin, typename P::T* __restrict__ fout, Layout lay,
+    Mom4<typename P::T>* __restrict__ mom, double* force_next, Params p) {
   using T = typename P::T;
   let_next_start();
   const size_t S = (size_t)lay.S;
@@ -967,9 +977,9 @@ __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_
       } else {
         pull_offsets<L>(k, lay.runs[w & W_RUN], lay, p, d);
       }
-      const T* __restrict__ fk = fin + k;
+      const T* fk = fin + k;
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) f[i] = __ldg(fk + ((ptrdiff_t)i * (ptrdiff_t)S + d[i]));
+      for (int i = 0; i < L::Q; ++i) f[i] = fk[(ptrdiff_t)i * (ptrdiff_t)S + d[i]];
     }
     const uint32_t w3 = ((uint64_t)k + 2ull * G < S) ? __ldg(lay.word + k + 2 * G) : W_GHOST;
     // (a separate zero-store branch here: the walk serves dense lattices,
@@ -1125,8 +1135,7 @@ __device__ __forceinline__ void fill_dir_table(DirTable<T, L::Q>& tab) {
 // 2^-62; q alone fixes them), in doubles where that says no.
 template <class L, class P>
 __device__ __forceinline__ typename P::T eval_link(const DirVal<typename P::T>& dir, int ip, int i,
-                                                   const typename P::T* __restrict__ f,
-                                                   const Mom4<typename P::T>* __restrict__ mom, size_t N, int rule,
+                                                   const typename P::T* f, const Mom4<typename P::T>* mom, size_t N, int rule,
                                                    typename P::T q, uint32_t node, uint32_t ff, typename P::T uw0,
                                                    typename P::T uw1, typename P::T uw2, const Params& p,
                                                    typename P::T& fpf, bool moving, const int64_t* __restrict__ wq,
@@ -1188,7 +1197,7 @@ __device__ __forceinline__ typename P::T exchange(typename P::T fpf, typename P:
 
 // A link's momentum exchange t e added to its body's slot by FP64 atomics.
 template <class T>
-__device__ __forceinline__ void add_force(double* __restrict__ force, int body, T t, const DirVal<T>& dir) {
+__device__ __forceinline__ void add_force(double* force, int body, T t, const DirVal<T>& dir) {
   atomicAdd(&force[3 * body + 0], (double)(t * dir.ex));
   atomicAdd(&force[3 * body + 1], (double)(t * dir.ey));
   if (dir.ez != (T)0) atomicAdd(&force[3 * body + 2], (double)(t * dir.ez));
@@ -1255,11 +1264,11 @@ struct LinkForce<double> {
 //   Yu        (q f+_i'(x_f) + (1-q) f+_i'(x_ff) + wall)/(1+q) + q/(1+q) f+_i(x_f)  (Sec. 3)
 // with wall = 6 w rho0 (e_i . u_w).
 template <class L, class P, int SEQ>
-__global__ void __launch_bounds__(256, (P::shifted ? 2 : 3)) k_links(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom,
+__global__ void __launch_bounds__(256, (P::shifted ? 2 : 3)) k_links(typename P::T* f, const Mom4<typename P::T>* mom,
                                                const LinkRec* __restrict__ recs, const typename P::T* __restrict__ qv,
                                                const typename P::T* __restrict__ uwv,
                                                const int64_t* __restrict__ wqv, int64_t nl,
-                                               double* __restrict__ force, Params p, int64_t S_) {
+                                               double* force, Params p, int64_t S_) {
   using T = typename P::T;
   let_next_start();
   __shared__ DirTable<T, L::Q> tab;
@@ -1405,9 +1414,9 @@ constexpr int fused_blocks_per_sm() {
 // other bodies add their terms with FP64 atomics directly.
 template <class L, class P, bool MULTI, int BT>
 __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused(
-    const typename P::T* __restrict__ fin, typename P::T* __restrict__ fout, Layout lay,
-    FusedLinks<typename P::T> fl, const Mom4<typename P::T>* __restrict__ mom_in,
-    Mom4<typename P::T>* __restrict__ mom_out, double* __restrict__ force, double* __restrict__ force_next,
+    const typename P::T* fin, typename P::T* __restrict__ fout, Layout lay,
+    FusedLinks<typename P::T> fl, const Mom4<typename P::T>* mom_in,
+    Mom4<typename P::T>* __restrict__ mom_out, double* force, double* force_next,
     Params p) {
   using T = typename P::T;
   constexpr int NW = BT / 32;
@@ -1448,7 +1457,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
     if (MULTI) dom = run.dom;
     int d[L::Q];
     pull_offsets<L>(k, run, lay, p, d);
-    const T* __restrict__ fk = fin + k;
+    const T* fk = fin + k;
 #pragma unroll
     for (int i = 0; i < L::Q; ++i)
       // direction i comes from the solid side when its opposite is a link
@@ -1555,9 +1564,9 @@ __host__ __device__ __forceinline__ bool inline_spread(int64_t nlinked) { return
 
 template <class L, class P, bool MULTI, int BT>
 __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inline(
-    const typename P::T* __restrict__ fin, typename P::T* __restrict__ fout, Layout lay,
-    FusedLinks<typename P::T> fl, const Mom4<typename P::T>* __restrict__ mom_in,
-    Mom4<typename P::T>* __restrict__ mom_out, double* __restrict__ force, double* __restrict__ force_next,
+    const typename P::T* fin, typename P::T* __restrict__ fout, Layout lay,
+    FusedLinks<typename P::T> fl, const Mom4<typename P::T>* mom_in,
+    Mom4<typename P::T>* __restrict__ mom_out, double* force, double* force_next,
     Params p) {
   using T = typename P::T;
   constexpr int NW = BT / 32, NF = inline_free_groups<P>();
