@@ -263,7 +263,10 @@ __global__ void __launch_bounds__(64, 10) k_adj_pair(const float* fin, float* la
     F2 f[9], lam[9], mu[9];
     pair_pull(k, n, fin, lay, p, f);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) lam[i].v = *(const unsigned long long*)(lam_next + (size_t)i * S + k);
+    for (int i = 0; i < 9; ++i) {
+      const float2 l = *(const float2*)(lam_next + (size_t)i * S + k);
+      lam[i] = pack2(l.x, l.y);
+    }
     // moments of f+(s) at cached nodes (the k_refresh formula)
     auto refresh = [&](uint32_t m, const Relax& rx) {
       float r = 0, jx = 0, jy = 0;

@@ -786,7 +786,8 @@ __device__ __forceinline__ void pair_pull(uint32_t k, const PairNodes& n, const 
   const int x = (int)k + n.ra.xk;
   if (n.same() && x > 0 && x + 1 < p.nx - 1) {
     const float* fk = fin + k;
-    f[0].v = *(const unsigned long long*)fk;
+    const float2 own = *(const float2*)fk;
+    f[0] = pack2(own.x, own.y);
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
       const int dx = -L::cx(i), dy = -L::cy(i);
@@ -828,8 +829,9 @@ __device__ __forceinline__ void pair_finish(uint32_t k, bool live, const PairNod
   if ((n.w.y & W_CACHE) && fb) mom[k + 1] = Mom4<float>{high(r), high(ux), high(uy), 0.f};
   float* __restrict__ ok = fout + k;
   if (fa && fb) {
+    // (stored as floats: open_ends reads them back as such)
 #pragma unroll
-    for (int i = 0; i < 9; ++i) *(unsigned long long*)(ok + (size_t)i * S) = f[i].v;
+    for (int i = 0; i < 9; ++i) *(float2*)(ok + (size_t)i * S) = make_float2(low(f[i]), high(f[i]));
   } else if (live) {
     // ghost slots take zeros (whole sectors), open slots their neighbour's thread
 #pragma unroll

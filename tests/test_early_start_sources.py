@@ -80,3 +80,12 @@ def test_early_kernels_load_what_others_write_coherently(what):
                 if decl[1] not in (TABLES if decl[0].strip().startswith("const") else OUTPUTS):
                     wrong.append((n, decl[1]))
     assert not wrong, wrong
+
+
+def test_no_population_is_accessed_through_another_type():
+    """A pair of floats stored as one 64-bit integer and read back as a float by
+    the same thread (the open node beside it) is undefined: the compiler may take
+    the two for different objects and move the load above the store."""
+    for f in ("kernels.cuh", "adjoint.cuh", "pair32.cuh"):
+        text = re.sub(r"//[^\n]*", "", (CSRC / f).read_text())
+        assert not re.search(r"\*\s*\(\s*(const )?(unsigned long long|uint64_t|double|int64_t)\s*\*\s*\)", text), f
