@@ -1814,7 +1814,10 @@ __device__ __forceinline__ void node_moments(const typename P::T* __restrict__ f
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) h[i] = f[(size_t)i * S + k];
   if constexpr (!P::shifted) {
-    if (p.kx.on) {
+    // (a domain whose force is beyond the grid's has no grid constants)
+    bool on = p.kx.on != 0;
+    if (lay.ndom > 1) on = lay.dom[lay.runs[w & W_RUN].dom].kx.on != 0;
+    if (on) {
       uint64_t r = 0, j[3] = {0, 0, 0};
       uint32_t bad = 0;
 #pragma unroll

@@ -186,3 +186,52 @@ def test_field_read_out_at_tile_edges(L, shape, body, prec):
     assert np.all(np.abs(rho - r)[fl] <= 64 * eps * S[fl])
     amp = (1 + np.abs(ur).max(0)) / np.abs(r)
     assert np.all(np.abs(u - ur)[:, fl] <= 64 * eps * (S * amp)[fl])
+
+
+def _masked(stencil, shape, solid, q=0.5, bc=0, body=-1):
+    """A periodic lattice with a mask: a link wherever a direction of a fluid
+    node points into the solid, all of one rule."""
+    nx, ny, nz = shape
+    m = solid.reshape(nz, ny, nx)
+    e = G.velocity_set(stencil)
+    links = []
+    for d in range(1, len(e)):
+        hit = (m == 0) & (np.roll(m, tuple(-e[d][::-1]), (0, 1, 2)) != 0)
+        lk = np.zeros(int(hit.sum()), G.LINK_DTYPE)
+        lk["node"], lk["dir"], lk["bc"], lk["body"], lk["q"] = np.flatnonzero(hit), d, bc, body, q
+        links.append(lk)
+    links = np.concatenate(links)
+    links = links[np.lexsort((links["dir"], links["node"]))]
+    return G.Geometry(stencil, nx, ny, nz, (True, True, True), solid, links, (False, False), None, {})
+
+
+@pytest.mark.parametrize("cfg_g", [0.0, 0.02])
+@pytest.mark.parametrize("stencil", [G.D2Q9, G.D3Q19])
+def test_fp64_read_out_of_domains_with_weak_and_strong_forces(L, stencil, cfg_g):
+    """rho and u of a batch's domains from their own populations, forces inside
+    and beyond the grid's (|g| > rho0 / 512) side by side, whatever the lattice's
+    own unused force is: 64 eps, as above."""
+    forces = [(0.0, 0.0, 0.0), (1e-4, -3e-5, 2e-5), (0.01, -0.004, 0.003), (0.0, 0.05, 0.0), (1e-3, 0.0, 0.0)]
+    n, nx, D = 7, 19, 2 if stencil == G.D2Q9 else 3
+    shape = (nx, n * len(forces), 1) if D == 2 else (nx, 6, n * len(forces))
+    rows = shape[D - 1]
+    solid = np.zeros((rows, int(np.prod(shape)) // rows), np.uint8)
+    solid[::n] = 1
+    solid[n - 1::n] = 1
+    geo = _masked(stencil, shape, solid.reshape(-1))
+    fl = geo.solid == 0
+    lat = L.Lattice(geo, domains=[dict(lo=n * k, n=n, nx=nx, tau=0.7, g=g) for k, g in enumerate(forces)],
+                    precision=L.LBM_FP64, tau=0.7, g=(cfg_g, 0.0, 0.0))
+    lat.init_equilibrium()
+    lat.set_distributions(_state(stencil, geo.N, 1.0, "plain", np.random.default_rng(3)) * fl)
+    f = lat.distributions()
+    rho, u = lat.moments()
+    lat.close()
+    e, _ = _weights(stencil)
+    g = np.repeat(np.array(forces), geo.N // len(forces), 0).T
+    r = np.where(fl, f.sum(0), 1.0)
+    ur = ((e.T @ f - 0.5 * g) / r)[:D]
+    S = np.abs(f).sum(0) + np.abs(g).sum(0)
+    u = u.reshape(D, -1)
+    assert np.all(np.abs(rho.reshape(-1) - r)[fl] <= 64 * EPS * S[fl])
+    assert np.all(np.abs(u - ur)[:, fl] <= 64 * EPS * (S / r * (1 + np.abs(ur).max(0)))[fl])
