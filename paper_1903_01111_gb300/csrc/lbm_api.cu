@@ -706,8 +706,8 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   // open inlet reads the moments of the first fluid column
   if (c.inlet)
     for (int64_t y = 0; y < ny; ++y)
-      if ((m[nx * y] & H_OPEN) && nx > 1) {
-        if (m[nx * y + 1] & (H_SOLID | H_OPEN))
+      if (m[nx * y] & H_OPEN) {
+        if (nx < 2 || (m[nx * y + 1] & (H_SOLID | H_OPEN)))
           return fail(LBM_ERR_INVALID_ARG, "inlet node (0,%lld) has no fluid node at x = 1", (long long)y);
         m[nx * y + 1] |= H_CACHE;
       }

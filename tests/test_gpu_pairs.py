@@ -140,3 +140,16 @@ def _smooth(geo):
     u[:, 1] = 0.01 * np.cos(2 * np.pi * x / geo.nx)
     u[geo.solid != 0] = 0
     return u
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32s"])
+def test_inlet_needs_a_second_column(L, prec):
+    """The inlet column is filled from the fluid node at x = 1; a lattice of one
+    column has none, and the node after its last row would be beyond the storage
+    (32 rows fill it exactly)."""
+    lat = L.Lattice(None, stencil=0, nx=1, ny=32, nz=1, periodic=(0, 1, 1), tau=0.8, inlet=1, inlet_umax=0.05, inlet_y0=-0.5,
+                    inlet_y1=31.5, precision=L.LBM_FP64 if prec == "fp64" else L.LBM_FP32_SHIFTED)
+    with pytest.raises(L.LBMError) as ex:
+        lat.set_geometry(np.zeros(32, np.uint8), np.zeros(0, G.LINK_DTYPE))
+    assert ex.value.status == L.LBM_ERR_INVALID_ARG and "inlet" in str(ex.value)
+    lat.close()
