@@ -493,8 +493,9 @@ __device__ __forceinline__ void collide_store(typename P::T (&f)[L::Q], const Pa
 #undef LBM_KI
 
 // Collision and store of one node in the step kernels.  FP64 collides on the
-// integer grid (fixed64.cuh) and, where the node is outside its range, takes
-// the populations again (again(f) fills f as it was) and collides in doubles.
+// integer grid (fixed64.cuh) and, where a kept node is outside its range,
+// takes the populations again (again(f) fills f as it was) and collides in
+// doubles.
 template <class L, class P, bool MULTI, class Again>
 __device__ __forceinline__ void collide_node(typename P::T (&f)[L::Q], const Params& p, const Layout& lay, int dom,
                                              typename P::T* __restrict__ fout, size_t S, uint32_t k,
@@ -505,7 +506,8 @@ __device__ __forceinline__ void collide_node(typename P::T (&f)[L::Q], const Par
     const FixedK& kx = fixed_of<MULTI>(p, lay, dom);
     if (kx.on) {
       NodeMom m;
-      if (collide_grid(f, kx, rx.has_force != 0, m)) {
+      // (a slot that is not kept stores zeros whatever comes out)
+      if (collide_grid(f, kx, rx.has_force != 0, m) || !keep) {
         if (cache && keep) mom[k] = Mom4<double>{(double)m.r * kx.step, m.u(m.ux), m.u(m.uy), m.u(m.uz)};
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) fout[(size_t)i * S + k] = keep ? f[i] : 0.0;
@@ -741,16 +743,12 @@ __device__ __forceinline__ void bulk_nodes(const uint32_t (&k)[NPT], const bool 
     if (!live[j] || (w[j] & W_OPEN)) continue;
     // ghost slots: zeros through the same stores (inputs at rest)
     const bool fl = !(w[j] & W_GHOST);
-    auto rest = [&](T(&g)[L::Q]) {
+    if (!fl) {
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) g[i] = P::shifted ? (T)0 : (T)L::w(i);
-    };
-    if (!fl) rest(f[j]);
+      for (int i = 0; i < L::Q; ++i) f[j][i] = P::shifted ? (T)0 : (T)L::w(i);
+    }
     collide_node<L, P, MULTI>(f[j], p, lay, dom[j], fout, S, k[j], mom, (w[j] & W_CACHE) != 0, fl, [&](T(&g)[L::Q]) {
-      if (fl)
-        pull_node<L>(fin, S, k[j], lay.runs[w[j] & W_RUN], lay, p, g);
-      else
-        rest(g);
+      pull_node<L>(fin, S, k[j], lay.runs[w[j] & W_RUN], lay, p, g);
     });
     if (L::D == 2 && fl && (p.inlet | p.outlet)) open_ends<L, P>(fout, mom, S, k[j], lay.runs[w[j] & W_RUN], lay, p);
   }
@@ -1716,13 +1714,11 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
   if (mask) take(f);
   if (live && !(w & W_OPEN)) {
     // ghost slots: zeros through the same stores (inputs at rest)
-    auto rest = [&](T(&v)[L::Q]) {
+    if (!fluid) {
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) v[i] = P::shifted ? (T)0 : (T)L::w(i);
-    };
-    if (!fluid) rest(f);
+      for (int i = 0; i < L::Q; ++i) f[i] = P::shifted ? (T)0 : (T)L::w(i);
+    }
     collide_node<L, P, MULTI>(f, p, lay, dom, fout, S, k, mom_out, (w & W_CACHE) != 0, fluid, [&](T(&v)[L::Q]) {
-      if (!fluid) return rest(v);
       pull_node<L>(fin, S, k, lay.runs[w & W_RUN], lay, p, v);
       take(v);
     });
