@@ -1203,16 +1203,38 @@ __device__ __forceinline__ void add_force(double* force, int body, T t, const Di
   if (dir.ez != (T)0) atomicAdd(&force[3 * body + 2], (double)(t * dir.ez));
 }
 
-// Sum of the momentum exchange t e over links of one body.  FP32 adds in FP32;
-// FP64 adds integers in steps of 2^(sc - 57) (a warp's reduction of doubles is
-// 15 FP64 instructions), and hands a t of 2^(sc - 4) or more, or not a number,
-// to `direct`, which adds it to the body's slot by itself: no sum of the 576
-// links that a warp may hold reaches 2^63 steps.
-template <class T>
+// As add_force for the lanes that are here, one atomic per body and component
+// (out of line and by values, so that the usual case keeps its registers).
+static __device__ __noinline__ void add_force_together(double* force, int body, double t, int ex, int ey, int ez) {
+  const unsigned m = __match_any_sync(__activemask(), body);
+  const int lane = threadIdx.x & 31;
+  double v[3] = {t * ex, t * ey, t * ez};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (m == 0xffffffffu) {
+      for (int o = 16; o > 0; o >>= 1) v[a] += __shfl_down_sync(m, v[a], o);
+    } else {
+      double sum = 0.0;
+      for (unsigned r = m; r; r &= r - 1) sum += __shfl_sync(m, v[a], __ffs(r) - 1);
+      v[a] = sum;
+    }
+    if (lane == __ffs(m) - 1) atomicAdd(&force[3 * body + a], v[a]);
+  }
+}
+
+// Sum of the momentum exchange t e over at most LINKS links of one body in a
+// warp.  FP32 adds in FP32; FP64 adds integers in steps of 2^(sc - 57) (a warp's
+// reduction of doubles is 15 FP64 instructions), each |t| below 2^(sc + room), so
+// that no sum reaches 2^63 steps.  Any other t (the link kernel, a link a lane: a
+// density beyond about 9 rho0; 576 links: more than about rho0/4 from rho0; a value
+// that is not a number) goes to `far`, which adds it to the body's slot.  128^3
+// pack, collisions and links in doubles: 504 us per step at 2 rho0 and 549 at
+// 40 rho0; 1214 and 4120 with an atomic per link, 578 with everything in doubles.
+template <class T, int LINKS>
 struct LinkForce {
   T F[3] = {0, 0, 0};
-  template <class Direct>
-  __device__ __forceinline__ void add(T t, const DirVal<T>& dir, const FixedK&, Direct&&) {
+  template <class Far>
+  __device__ __forceinline__ void add(T t, const DirVal<T>& dir, const FixedK&, Far&&) {
     F[0] += t * dir.ex;
     F[1] += t * dir.ey;
     F[2] += t * dir.ez;
@@ -1225,13 +1247,15 @@ struct LinkForce {
   }
   __device__ __forceinline__ double value(int a, const FixedK&) const { return (double)F[a]; }
 };
-template <>
-struct LinkForce<double> {
+template <int LINKS>
+struct LinkForce<double, LINKS> {
+  static constexpr int room = LINKS <= 32 ? 1 : (LINKS <= 128 ? -1 : (LINKS <= 256 ? -2 : -4));
+  static_assert(LINKS <= 1024, "64-bit sums");
   int64_t F[3] = {0, 0, 0};
-  template <class Direct>
-  __device__ __forceinline__ void add(double t, const DirVal<double>& dir, const FixedK& k, Direct&& direct) {
+  template <class Far>
+  __device__ __forceinline__ void add(double t, const DirVal<double>& dir, const FixedK& k, Far&& far) {
     const uint32_t hi = (uint32_t)__double2hiint(t), e = (hi >> 20) & 0x7ffu;
-    if (k.step == 0.0 || e >= (uint32_t)(1019 + k.sc)) return direct();
+    if (k.step == 0.0 || e >= (uint32_t)(1023 + room + k.sc)) return far();
     // t 2^(57 - sc) by its exponent (a t too small for that is none of a step)
     const bool tiny = (int)e < 900 + k.sc || e == 0u;
     const int64_t v = __double2ll_rn(
@@ -1283,7 +1307,7 @@ __global__ void __launch_bounds__(256, (P::shifted ? 2 : 3)) k_links(typename P:
   // terms with FP64 atomics directly
   const int b0 = (int)(__ldg(&recs[base].meta) >> 7) - 1;
   const size_t N = (size_t)S_;
-  LinkForce<T> F;
+  LinkForce<T, 32 * SEQ> F;
   int64_t k = base + threadIdx.x;
   bool live = k < nl;
   LinkRec rec{0, 0, 0, 0};
@@ -1320,11 +1344,13 @@ __global__ void __launch_bounds__(256, (P::shifted ? 2 : 3)) k_links(typename P:
       if (body >= 0) {
         const DirVal<T> dir = dir_of(tab, ip);
         const T t = exchange<P>(fpf, val, dir, p);
-        auto direct = [&] { add_force(force, body, t, dir); };
+        auto far = [&] {
+          if constexpr (!P::shifted) add_force_together(force, body, t, dir.e[0], dir.e[1], dir.e[2]);
+        };
         if (body == b0)
-          F.add(t, dir, p.kx, direct);
+          F.add(t, dir, p.kx, far);
         else
-          direct();
+          add_force(force, body, t, dir);
       }
     }
     k = kn;
@@ -1470,7 +1496,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
   }
   cp_async_commit();
   const int wb = total > 0 ? (int)(__ldg(&fl.rec[l0].meta) >> 8) - 1 : -1;
-  LinkForce<T> F;
+  LinkForce<T, 32 * (L::Q - 1)> F;
   for (int j = threadIdx.x; j < total; j += BT) {
     const int64_t li = l0 + j;
     const bool first_round = j == (int)threadIdx.x;
@@ -1494,11 +1520,13 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
       // momentum exchange as in k_links
       const DirVal<T> dir = dir_of(tab, ip);
       const T t = exchange<P>(fpf, val, dir, p);
-      auto direct = [&] { add_force(force, body, t, dir); };
+      auto far = [&] {
+        if constexpr (!P::shifted) add_force_together(force, body, t, dir.e[0], dir.e[1], dir.e[2]);
+      };
       if (body == wb)
-        F.add(t, dir, p.kx, direct);
+        F.add(t, dir, p.kx, far);
       else
-        direct();
+        add_force(force, body, t, dir);
     }
   }
   if (wb >= 0) {
@@ -1636,7 +1664,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
   T(&col)[L::Q][32] = stage[spread ? 0 : warp];
   // forces are summed for the body of the warp's first link
   const int wb = (int)(__shfl_sync(0xffffffffu, r.meta, 0) >> 8) - 1;
-  LinkForce<T> F;
+  LinkForce<T, 32 * (L::Q - 1)> F;
   for (int64_t li = first < 0 ? l1 : l0 + first; li < l1; li += step) {
     if (li != l0 + first) {
       r = fl.rec[li];
@@ -1669,11 +1697,13 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
     if (body >= 0) {
       // momentum exchange as in k_links
       const T t = exchange<P>(fpf, val, dir, p);
-      auto direct = [&] { add_force(force, body, t, dir); };
+      auto far = [&] {
+        if constexpr (!P::shifted) add_force_together(force, body, t, dir.e[0], dir.e[1], dir.e[2]);
+      };
       if (body == wb)
-        F.add(t, dir, p.kx, direct);
+        F.add(t, dir, p.kx, far);
       else
-        direct();
+        add_force(force, body, t, dir);
     }
   }
   if (!P::shifted && !spread) pull();
