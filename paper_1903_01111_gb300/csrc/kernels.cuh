@@ -492,11 +492,11 @@ __device__ __forceinline__ void collide_store(typename P::T (&f)[L::Q], const Pa
 #undef LBM_K
 #undef LBM_KI
 
-// Collision and store of one node in the step kernels.  FP64 collides on the
+// Collision and store of one node in the step kernels (SOON: see fixed64.cuh).  FP64 collides on the
 // integer grid (fixed64.cuh) and, where a kept node is outside its range,
 // takes the populations again (again(f) fills f as it was) and collides in
 // doubles.
-template <class L, class P, bool MULTI, class Again>
+template <class L, class P, bool MULTI, bool SOON, class Again>
 __device__ __forceinline__ void collide_node(typename P::T (&f)[L::Q], const Params& p, const Layout& lay, int dom,
                                              typename P::T* __restrict__ fout, size_t S, uint32_t k,
                                              Mom4<typename P::T>* __restrict__ mom, bool cache, bool keep,
@@ -507,7 +507,7 @@ __device__ __forceinline__ void collide_node(typename P::T (&f)[L::Q], const Par
     if (kx.on) {
       NodeMom m;
       // (a slot that is not kept stores zeros whatever comes out)
-      if (collide_grid(f, kx, rx.has_force != 0, m) || !keep) {
+      if (collide_grid<SOON>(f, kx, rx.has_force != 0, m) || !keep) {
         if (cache && keep) mom[k] = Mom4<double>{(double)m.r * kx.step, m.u(m.ux), m.u(m.uy), m.u(m.uz)};
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) fout[(size_t)i * S + k] = keep ? f[i] : 0.0;
@@ -709,7 +709,7 @@ constexpr int bulk_blocks_per_sm() {
 // Pull, collision and store of NPT nodes k of a thread, all their pulls issued
 // before the first collision.  MULTI: the lattice holds several domains; each
 // node's collision reads its run's domain parameters.
-template <class L, class P, bool MULTI, int NPT>
+template <class L, class P, bool MULTI, int NPT, bool SOON>
 __device__ __forceinline__ void bulk_nodes(const uint32_t (&k)[NPT], const bool (&live)[NPT],
                                            const typename P::T* fin, typename P::T* __restrict__ fout,
                                            const Layout& lay, Mom4<typename P::T>* __restrict__ mom, const Params& p) {
@@ -747,7 +747,7 @@ __device__ __forceinline__ void bulk_nodes(const uint32_t (&k)[NPT], const bool 
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) f[j][i] = P::shifted ? (T)0 : (T)L::w(i);
     }
-    collide_node<L, P, MULTI>(f[j], p, lay, dom[j], fout, S, k[j], mom, (w[j] & W_CACHE) != 0, fl, [&](T(&g)[L::Q]) {
+    collide_node<L, P, MULTI, SOON>(f[j], p, lay, dom[j], fout, S, k[j], mom, (w[j] & W_CACHE) != 0, fl, [&](T(&g)[L::Q]) {
       pull_node<L>(fin, S, k[j], lay.runs[w[j] & W_RUN], lay, p, g);
     });
     if (L::D == 2 && fl && (p.inlet | p.outlet)) open_ends<L, P>(fout, mom, S, k[j], lay.runs[w[j] & W_RUN], lay, p);
@@ -880,7 +880,7 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_b
     live[j] = t < stride && (uint64_t)k[j] < (uint64_t)lay.S;
     prefetch_ahead<L::Q>(fin, lay, (uint64_t)blockIdx.x * BT + (uint64_t)j * (stride / 32 * 32), BT, threadIdx.x, BT);
   }
-  bulk_nodes<L, P, MULTI, NPT>(k, live, fin, fout, lay, mom, p);
+  bulk_nodes<L, P, MULTI, NPT, true>(k, live, fin, fout, lay, mom, p);
   clear_force<BT>(force_next, p.nbody);
 }
 
@@ -912,7 +912,7 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, 1>())) k_bul
   prefetch_ahead<L::Q>(fin, lay, (uint64_t)k / 32 * 32 - (threadIdx.x & ~31u), BT, threadIdx.x, BT);
   T f[L::Q];
   pull_node<L>(fin, S, k, run, lay, p, f);
-  collide_node<L, P, MULTI>(f, p, lay, run.dom, fout, S, k, mom, (w & W_CACHE) != 0, true, [&](T(&g)[L::Q]) {
+  collide_node<L, P, MULTI, true>(f, p, lay, run.dom, fout, S, k, mom, (w & W_CACHE) != 0, true, [&](T(&g)[L::Q]) {
     pull_node<L>(fin, S, k, lay.runs[w & W_RUN], lay, p, g);
   });
   if (L::D == 2 && (p.inlet | p.outlet)) open_ends<L, P>(fout, mom, S, k, lay.runs[w & W_RUN], lay, p);
@@ -988,7 +988,7 @@ __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) fout[(size_t)i * S + k] = (T)0;
     } else if (fluid) {
-      collide_node<L, P, MULTI>(f, p, lay, run.dom, fout, S, k, mom, (w & W_CACHE) != 0, true, [&](T(&g)[L::Q]) {
+      collide_node<L, P, MULTI, true>(f, p, lay, run.dom, fout, S, k, mom, (w & W_CACHE) != 0, true, [&](T(&g)[L::Q]) {
         pull_node<L>(fin, S, k, lay.runs[w & W_RUN], lay, p, g);
       });
       if (p.inlet | p.outlet) open_ends<L, P>(fout, mom, S, k, lay.runs[w & W_RUN], lay, p);
@@ -1546,7 +1546,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
     T f[L::Q];
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) f[i] = col[i][lane];
-    collide_node<L, P, MULTI>(f, p, lay, dom, fout, S, k, mom_out, (w & W_CACHE) != 0, fluid, [&](T(&g)[L::Q]) {
+    collide_node<L, P, MULTI, false>(f, p, lay, dom, fout, S, k, mom_out, (w & W_CACHE) != 0, fluid, [&](T(&g)[L::Q]) {
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) g[i] = col[i][lane];
     });
@@ -1625,7 +1625,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
       live[j] = at + j < lay.ngroups && (uint64_t)k[j] < S;
     }
     prefetch_ahead<L::Q>(fin, lay, k[0] - lane, 32 * NF, lane, 32);
-    bulk_nodes<L, P, MULTI, NF>(k, live, fin, fout, lay, mom_out, p);
+    bulk_nodes<L, P, MULTI, NF, false>(k, live, fin, fout, lay, mom_out, p);
     clear_force<BT>(force_next, p.nbody);
     return;
   }
@@ -1748,7 +1748,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) f[i] = P::shifted ? (T)0 : (T)L::w(i);
     }
-    collide_node<L, P, MULTI>(f, p, lay, dom, fout, S, k, mom_out, (w & W_CACHE) != 0, fluid, [&](T(&v)[L::Q]) {
+    collide_node<L, P, MULTI, false>(f, p, lay, dom, fout, S, k, mom_out, (w & W_CACHE) != 0, fluid, [&](T(&v)[L::Q]) {
       pull_node<L>(fin, S, k, lay.runs[w & W_RUN], lay, p, v);
       take(v);
     });
