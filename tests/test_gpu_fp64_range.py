@@ -89,3 +89,145 @@ def test_forces_at_any_density(L, stencil, fused, scale):
     ref = (t[:, None] * e[lk["dir"]]).sum(0)
     n = len(lk)
     assert np.all(np.abs(F - ref) <= n * n * np.finfo(float).eps * t.max()) and np.abs(ref[0]) > 0
+
+
+# ------------------------------------------------------------- link values --
+
+QS = (1e-300, 1e-6, 1e-3, 0.1, 0.3, 0.4999999, 0.5, 0.5000001, 0.7, 0.999, 1.0)
+
+
+def _links_case(stencil, kind, seed):
+    """A lattice with solid nodes all over, VIBB links of every q, three bodies
+    (and none) in turn, walls that move; populations of `kind` (test_gpu_fixed64)
+    for rho0 = 1."""
+    from test_gpu_fixed64 import _masked, _state
+
+    rng = np.random.default_rng([seed, stencil])
+    shape = (37, 23, 1) if stencil == G.D2Q9 else (13, 9, 8)
+    N = int(np.prod(shape))
+    geo = _masked(stencil, shape, (rng.random(N) < 0.07).astype(np.uint8), bc=-1)
+    lk = geo.links
+    lk["q"] = rng.choice(QS, len(lk))
+    lk["body"] = rng.integers(-1, 3, len(lk))
+    lk["uw"] = rng.uniform(-1, 1, (len(lk), 3)) * (0.7 if kind == "fast" else 0.05)
+    if stencil == G.D2Q9:
+        lk["uw"][:, 2] = 0
+    return geo, _state(stencil, N, 1.0, kind, rng) * (geo.solid == 0)
+
+
+def _second_nodes(geo):
+    """x_ff of every link (x_f where that is solid)."""
+    n = geo.links["node"]
+    e = G.velocity_set(geo.stencil)[geo.links["dir"]].astype(int)
+    x = np.stack(np.unravel_index(n, (geo.nz, geo.ny, geo.nx)))[::-1]
+    y = (x - e.T) % np.array([[geo.nx], [geo.ny], [geo.nz]])
+    ff = y[0] + geo.nx * (y[1] + geo.ny * y[2])
+    return np.where(geo.solid[ff] != 0, n, ff)
+
+
+def _link_magnitudes(geo, f, rho0, local_rho):
+    """Per link: the sum of the magnitudes of the terms of its value, with the
+    change that one eps of each moment's terms makes in it, and the square of how
+    much the moments of its two nodes cancel."""
+    from test_gpu_fixed64 import _weights
+
+    e, w = _weights(geo.stencil)
+    lk = geo.links
+    n, d, q = lk["node"], lk["dir"], lk["q"]
+    ff = _second_nodes(geo)
+    rho, a = f.sum(0), np.abs(f).sum(0)
+    with np.errstate(all="ignore"):
+        u = np.abs(e.T @ f / rho)
+        cond = a / np.abs(rho)
+        amp = cond ** 2
+    p, m = 2 * q, np.abs(1 - 2 * q)
+
+    def K(v, c):  # 1 + 3 e.u + 4.5 (e.u)^2 - 1.5 u.u and its change with an error c eps of u
+        s = v.sum(0)
+        return 1 + 3 * s + 6 * s ** 2 + (3 + 12 * s) * c
+
+    rd = np.where(local_rho & (q > 0.5), np.abs(rho[n]), p * np.abs(rho[n]) + m * np.abs(rho[ff]))
+    with np.errstate(all="ignore"):
+        ud = u[:, n] + u[:, ff] + np.abs(lk["uw"].T)
+        M = w[d] * rd * K(ud, cond[n] + cond[ff]) + 6 * w[d] * rho0 * np.abs(lk["uw"]).sum(1)
+        for k, c in ((n, p), (ff, m)):
+            M = M + c * rd / np.abs(rho[k]) * (np.abs(f[d, k]) + w[d] * np.abs(rho[k]) * K(u[:, k], cond[k]))
+    return M, np.maximum(1.0, np.maximum(amp[n], amp[ff]))
+
+
+@pytest.mark.parametrize("kind", ["plain", "fast", "density", "odd"])
+@pytest.mark.parametrize("rho0", [1.0, 0.75, 1.4999, 3e-9, 1.7e12])
+@pytest.mark.parametrize("local_rho", [0, 1])
+@pytest.mark.parametrize("stencil", [G.D2Q9, G.D3Q19])
+def test_fp64_links_in_and_out_of_the_grid(L, stencil, local_rho, rho0, kind):
+    """One step from given populations, in both step forms, against the oracle.
+    A link value rounds about forty operations on terms of total size M, its
+    moments carry the rounding of their populations amplified by `amp`, and a
+    collision's outputs are at most 4 times its inputs' errors plus 64 eps of
+    their sum: 256 eps (sum |f| + sum M amp) of the node.  A force sums its
+    links: 64 eps M amp each and n eps of the sum of the terms."""
+    import oracle as O
+
+    geo, f0 = _links_case(stencil, kind, 11)
+    f0 = f0 * rho0
+    eps = np.finfo(float).eps
+    cfg = O.make_config(stencil=stencil, nx=geo.nx, ny=geo.ny, nz=geo.nz, tau=0.8, rho0=rho0, bc=2, vibb_density=local_rho)
+    st = O.State(f0.copy(), *O.moments(cfg, geo.solid, f0))
+    Fr = O.run(cfg, geo.solid, geo.links, st, 1, nbody=3)
+    fl = geo.solid == 0
+    M, amp = _link_magnitudes(geo, f0, rho0, local_rho)
+    from test_gpu_fixed64 import _pull, _weights
+
+    e, w = _weights(stencil)
+    lk = geo.links
+    pulled = _pull(stencil, f0, (geo.nx, geo.ny, geo.nz))  # (from solid nodes: zeros)
+    S, net = np.abs(pulled).sum(0), pulled.sum(0)
+    np.add.at(S, lk["node"], M * amp)
+    # the collision divides by the density, which the links may nearly cancel
+    rho1 = np.abs(st.rho)
+    with np.errstate(all="ignore"):
+        S = S * np.maximum(1.0, (S / rho1) ** 2)
+    t = np.abs(f0[lk["dir"], lk["node"]]) + M + 2 * w[lk["dir"]] * rho0
+    for fused in (0, 1):
+        with L.Lattice(geo, precision=L.LBM_FP64, tau=0.8, rho0=rho0, bc=2, vibb_density=local_rho) as lat:
+            lat.set_tuning(bulk_shape=1, fused=fused)
+            lat.init_equilibrium()
+            lat.set_distributions(f0)
+            lat.step(1)
+            f, F = lat.distributions(), lat.forces(3)
+        assert np.all(np.abs(f - st.fp)[:, fl] <= 256 * eps * S[fl]), (fused, np.nanmax((np.abs(f - st.fp) / S)[:, fl]))
+        for b in range(3):
+            k = lk["body"] == b
+            tol = eps * (64 * (M * amp)[k].sum() + k.sum() * t[k].sum())
+            assert np.all(np.abs(F[b] - Fr[b]) <= tol), (fused, b)
+
+
+@pytest.mark.parametrize("fused", [0, 1])
+@pytest.mark.parametrize("stencil", [G.D2Q9, G.D3Q19])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_fp64_links_keep_non_finite_values_visible(L, stencil, fused, bad):
+    """One such population reaches the node it streams to and, through the
+    moments of its node, every link that reads them, and no other node or body."""
+    geo, f0 = _links_case(stencil, "plain", 12)
+    lk = geo.links
+    ff = _second_nodes(geo)
+    n = int(lk["node"][len(lk) // 2])
+    f0[5, n] = bad
+    with L.Lattice(geo, precision=L.LBM_FP64, tau=0.8, bc=2) as lat:
+        lat.set_tuning(bulk_shape=1, fused=fused)
+        lat.init_equilibrium()
+        lat.set_distributions(f0)
+        lat.step(1)
+        f, F = lat.distributions(), lat.forces(3)
+        with pytest.raises(L.LBMError):
+            lat.check()
+    e = G.velocity_set(stencil)
+    x = np.array(np.unravel_index(n, (geo.nz, geo.ny, geo.nx)))[::-1]
+    to = (x + e[5].astype(int)) % (geo.nx, geo.ny, geo.nz)
+    reads = (lk["node"] == n) | (ff == n)
+    expect = np.zeros(geo.N, bool)
+    expect[to[0] + geo.nx * (to[1] + geo.ny * to[2])] = True
+    expect &= geo.solid == 0
+    expect[lk["node"][reads]] = True
+    assert np.array_equal(~np.isfinite(f).all(0), expect)
+    assert [not np.isfinite(F[b]).all() for b in range(3)] == [bool((reads & (lk["body"] == b)).any()) for b in range(3)]
