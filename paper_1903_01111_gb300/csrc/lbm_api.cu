@@ -133,8 +133,9 @@ struct lbm_lattice_s {
   DeviceBuf lfirst, lmask, lrec, lqd, luw;
   DeviceBuf fidx;  // FP64: storage indices of the fluid nodes (the bulk pass's thread map)
   // FP64: VIBB velocity weights [3][n_links] in the link kernel's order, and in
-  // the fused kernel's where that is another one
+  // the fused kernel's where that is another one (fused_reorders)
   DeviceBuf lqc, lqf;
+  bool fused_reorders = false;
   int64_t n_links = 0, n_fluid = 0, n_stored = 0, n_cached = 0, n_runs = 0;
   DeviceBuf force;  // [2][nbody][3]
   // sum over each body's links of 2 w_i' rho0 e_i' (FP64), the rest part of the
@@ -226,6 +227,38 @@ void release_geometry(lbm_handle h) {
                       &h->lqd,      &h->luw,       &h->dom,      &h->row_dom, &h->fidx, &h->lqc, &h->lqf};
   for (auto* b : all) release(*b);
   h->lay = Layout{};
+}
+
+// FP64: the VIBB velocity weights of n links (u*_d's and u**_d's weights of
+// Sec. 3.1 blended 1/3 : 2/3; q alone fixes them) in 2^-62, [3][n].
+template <class QOf>
+raw_vec<int64_t> vibb_weights(int64_t n, QOf&& q_of) {
+  raw_vec<int64_t> w(3 * (size_t)n);
+#pragma omp parallel for schedule(static)
+  for (int64_t j = 0; j < n; ++j) {
+    const double q = q_of(j), two_q = 2.0 * q, i1q = 1.0 / (1.0 + q);
+    const double af = q <= 0.5 ? two_q : (1.0 - q) / q, aff = q <= 0.5 ? 1.0 - two_q : 0.0;
+    const double aw = q <= 0.5 ? 0.0 : (two_q - 1.0) / q;
+    const double third = 1.0 / 3.0, unit = 0x1p62;
+    w[j] = (int64_t)std::llrint(third * af * unit);
+    w[n + j] = (int64_t)std::llrint((third * aff + 2.0 * third * (1.0 - q) * i1q) * unit);
+    w[2 * n + j] = (int64_t)std::llrint((third * aw + 2.0 * third * two_q * i1q) * unit);
+  }
+  return w;
+}
+
+// The weights in the fused kernel's link order, where that is not the link
+// kernel's: kept only while the tuning runs the fused step (24 B a link).
+lbm_status fused_weights(lbm_handle h, bool fused) {
+  if (!fused || !h->has_geometry || !h->fused_reorders) {
+    release(h->lqf);
+    return LBM_OK;
+  }
+  if (h->lqf.p) return LBM_OK;
+  raw_vec<double> q((size_t)h->n_links);
+  CUDA_TRY(cudaMemcpy(q.data(), h->lqd.p, sizeof(double) * h->n_links, cudaMemcpyDeviceToHost));
+  return upload(h->lqf, vibb_weights(h->n_links, [&](int64_t j) { return q[j]; }).data(),
+                sizeof(int64_t) * 3 * h->n_links);
 }
 
 int cx_of(const lbm_handle h, int i) { return h->Q == 9 ? D2Q9::cx(i) : D3Q19::cx(i); }
@@ -1072,23 +1105,6 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
       split_rec(j, k, (uint32_t)sidx[links[k].node], (uint32_t)sidx[lk_ff[k]]);
     }
   }
-  // FP64: the VIBB velocity weights of each link (u*_d's and u**_d's weights
-  // of Sec. 3.1 blended 1/3 : 2/3; q alone fixes them) in 2^-62, in the link
-  // kernel's order and, where it is another, in the fused kernel's
-  auto weights = [&](const int64_t* ord) {
-    raw_vec<int64_t> w(3 * (size_t)n_links);
-#pragma omp parallel for schedule(static)
-    for (int64_t j = 0; j < n_links; ++j) {
-      const double q = links[ord[j]].q, two_q = 2.0 * q, i1q = 1.0 / (1.0 + q);
-      const double af = q <= 0.5 ? two_q : (1.0 - q) / q, aff = q <= 0.5 ? 1.0 - two_q : 0.0;
-      const double aw = q <= 0.5 ? 0.0 : (two_q - 1.0) / q;
-      const double third = 1.0 / 3.0, unit = 0x1p62;
-      w[j] = (int64_t)std::llrint(third * af * unit);
-      w[n_links + j] = (int64_t)std::llrint((third * aff + 2.0 * third * (1.0 - q) * i1q) * unit);
-      w[2 * n_links + j] = (int64_t)std::llrint((third * aw + 2.0 * third * two_q * i1q) * unit);
-    }
-    return w;
-  };
   // first link of each 32-node group: storage indices of x_f are
   // non-decreasing along (node, dir) order, so ffirst[g] (the first j with
   // kf_j >= 32 g) is j for every g in (kf_{j-1} / 32, kf_j / 32], and n_links
@@ -1151,8 +1167,11 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   if (st == LBM_OK) st = upload(h->lqd, fq.data(), sizeof(double) * fq.size());
   if (st == LBM_OK && nflist > 0) st = upload(h->fidx, flist.data(), sizeof(uint32_t) * nflist);
   if (st == LBM_OK && h->rb == 8 && n_links > 0) {
-    st = upload(h->lqc, weights(order.data()).data(), sizeof(int64_t) * 3 * n_links);
-    if (st == LBM_OK && !same_order) st = upload(h->lqf, weights(ond).data(), sizeof(int64_t) * 3 * n_links);
+    st = upload(h->lqc, vibb_weights(n_links, [&](int64_t j) { return links[order[j]].q; }).data(),
+                sizeof(int64_t) * 3 * n_links);
+    if (st == LBM_OK && !same_order && h->tune.fused)
+      st = upload(h->lqf, vibb_weights(n_links, [&](int64_t j) { return links[ond[j]].q; }).data(),
+                  sizeof(int64_t) * 3 * n_links);
   }
   if (st == LBM_OK && ndom > 0) {
     std::vector<DomPar> dp(ndom);
@@ -1253,6 +1272,7 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   h->p.nbody = nbody;
   h->sidx.swap(sidx);
   h->n_links = n_links;
+  h->fused_reorders = h->rb == 8 && n_links > 0 && !same_order;
   h->n_fluid = n_fluid;
   h->n_stored = n_stored;
   h->n_cached = n_cached;
@@ -1828,6 +1848,8 @@ lbm_status lbm_set_tuning(lbm_handle h, const lbm_tuning* t) {
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     drop_graphs(h);
   }
+  const lbm_status st = fused_weights(h, v.fused != 0);
+  if (st != LBM_OK) return st;
   h->tune = v;
   h->tuned = true;
   return LBM_OK;

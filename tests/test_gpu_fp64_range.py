@@ -231,3 +231,32 @@ def test_fp64_links_keep_non_finite_values_visible(L, stencil, fused, bad):
     expect[lk["node"][reads]] = True
     assert np.array_equal(~np.isfinite(f).all(0), expect)
     assert [not np.isfinite(F[b]).all() for b in range(3)] == [bool((reads & (lk["body"] == b)).any()) for b in range(3)]
+
+
+# ----------------------------------------------------------------- memory --
+
+def test_fused_link_weights_are_held_only_for_the_fused_step(L):
+    """Bodies in turn make the fused step's link order another than the link
+    kernel's, and its velocity weights (24 B a link) a second copy: not held by
+    the split step that FP64 D3Q19 starts with, and the same step either way."""
+    geo, f0 = _links_case(G.D3Q19, "plain", 13)
+    with L.Lattice(geo, precision=L.LBM_FP64, tau=0.8, bc=2) as lat:
+        lat.init_equilibrium()
+        held = lat.info().device_bytes
+        out = []
+        for fused in (0, 1, 0, 1):
+            lat.set_tuning(bulk_shape=1, fused=fused)
+            assert lat.info().device_bytes == held + fused * 24 * len(geo.links)
+            lat.set_distributions(f0)
+            lat.step(2)
+            out.append(lat.distributions())
+    assert np.array_equal(out[0], out[2]) and np.array_equal(out[1], out[3])
+    assert np.abs(out[0] - out[1]).max() <= 1e-14
+    # chosen before the geometry
+    with L.Lattice(None, stencil=1, nx=geo.nx, ny=geo.ny, nz=geo.nz, precision=L.LBM_FP64, tau=0.8, bc=2) as lat:
+        lat.set_tuning(bulk_shape=1, fused=1)
+        lat.set_geometry(geo.solid, geo.links)
+        lat.init_equilibrium()
+        lat.set_distributions(f0)
+        lat.step(2)
+        assert np.array_equal(lat.distributions(), out[1])
