@@ -169,7 +169,7 @@ int64_t device_bytes(const lbm_handle h) {
   const DeviceBuf* all[] = {&h->f[0],     &h->f[1],     &h->mom[0],   &h->mom[1], &h->word,  &h->node_of, &h->tile, &h->row_uin, &h->groups,
                             &h->runs,     &h->row_first, &h->row_last, &h->row_in1, &h->row_out1, &h->recs,
                             &h->q,        &h->uw,       &h->lfirst, &h->lmask, &h->lrec,
-                            &h->lqd,      &h->luw,      &h->force,    &h->dom,    &h->row_dom, &h->fidx, &h->lqc, &h->lqf};
+                            &h->lqd,      &h->luw,      &h->force,    &h->dom,    &h->row_dom, &h->fidx, &h->lqc, &h->lqf, &h->force_hist};
   int64_t s = 0;
   for (auto* b : all) s += (int64_t)b->bytes;
   return s;

@@ -260,3 +260,12 @@ def test_fused_link_weights_are_held_only_for_the_fused_step(L):
         lat.set_distributions(f0)
         lat.step(2)
         assert np.array_equal(lat.distributions(), out[1])
+
+
+def test_force_slots_of_a_monitored_loop_are_counted(L):
+    geo = G.build(0, (45, 33, 1), (1, 1, 1), [G.ball((20.37, 15.61, 0), 6.3)])
+    with L.Lattice(geo, precision=L.LBM_FP64, tau=0.8, bc=2) as lat:
+        lat.init_equilibrium()
+        held = lat.info().device_bytes
+        lat.step_forces(100, 0)
+        assert lat.info().device_bytes == held + 100 * 3 * 8 * lat.info().n_bodies
