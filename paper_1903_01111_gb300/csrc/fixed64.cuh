@@ -55,6 +55,7 @@ inline void fold_fixed(FixedK& k, double omega, double fpre3, const double g[3],
   const double m = std::frexp(rho0, &e2);  // rho0 = m 2^e2, m in [1/2, 1)
   k.sc = m < 0.75 ? e2 - 1 : e2;
   bool on = e2 > -900 && e2 < 900;
+  k.grid = on ? 1 : 0;
   if (on) k.step = std::ldexp(1.0, k.sc - 62);
   for (int a = 0; a < 3; ++a) on = on && std::fabs(g[a]) <= kFixedMaxForce * rho0;
   k.on = on ? 1 : 0;

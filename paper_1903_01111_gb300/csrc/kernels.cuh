@@ -1158,7 +1158,8 @@ __device__ __forceinline__ typename P::T eval_link(const DirVal<typename P::T>& 
     fpi = f[(size_t)i * N + node];
   }
   if constexpr (!P::shifted) {
-    if (rule == 2 && p.kx.on) {
+    // (whatever the lattice's force: a domain alone and in a batch alike)
+    if (rule == 2 && p.kx.grid) {
       const int64_t c[3] = {wq[0], wq[nl], moving ? wq[2 * nl] : 0};
       const double m0[4] = {mf.r, mf.ux, mf.uy, mf.uz}, m1[4] = {mff.r, mff.ux, mff.uy, mff.uz};
       const double uw[3] = {uw0, uw1, uw2};
@@ -1255,7 +1256,7 @@ struct LinkForce<double, LINKS> {
   template <class Far>
   __device__ __forceinline__ void add(double t, const DirVal<double>& dir, const FixedK& k, Far&& far) {
     const uint32_t hi = (uint32_t)__double2hiint(t), e = (hi >> 20) & 0x7ffu;
-    if (k.step == 0.0 || e >= (uint32_t)(1023 + room + k.sc)) return far();
+    if (k.grid == 0 || e >= (uint32_t)(1023 + room + k.sc)) return far();
     // t 2^(57 - sc) by its exponent (a t too small for that is none of a step)
     const bool tiny = (int)e < 900 + k.sc || e == 0u;
     const int64_t v = __double2ll_rn(

@@ -122,7 +122,7 @@ struct FixedK {
   Halves ge[3], gp[2];
   uint32_t oh, oh2, ol;             // |1 - omega| 2^63 = oh 2^32 + ol; 2 oh
   uint64_t oc, neg;                 // centring term of its products; ~0 where 1 - omega < 0
-  int32_t sc, on;                   // grid exponent; 0: collide in doubles
+  int32_t sc, grid, on;             // grid exponent; 0: no grid for this rho0; 0: collide in doubles
 };
 
 // Run parameters handed to every kernel by value.

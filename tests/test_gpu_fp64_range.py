@@ -269,3 +269,32 @@ def test_force_slots_of_a_monitored_loop_are_counted(L):
         held = lat.info().device_bytes
         lat.step_forces(100, 0)
         assert lat.info().device_bytes == held + 100 * 3 * 8 * lat.info().n_bodies
+
+
+# ----------------------------------------------------------------- batches --
+
+def test_domains_with_strong_forces_equal_themselves_alone(L):
+    """A domain's force beyond the grid's (|g| > rho0 / 512) sends its collisions
+    to doubles, not its links: the same bits alone and in a batch whose other
+    domain has a weak force."""
+    from test_gpu_fixed64 import _masked
+
+    rng = np.random.default_rng(4)
+    nx, n, forces = 33, 20, [(0.01, 0.0, 0.0), (1e-4, 0.0, 0.0)]
+    parts = []
+    for _ in forces:
+        solid = (rng.random((n, nx)) < 0.05).astype(np.uint8)
+        solid[0] = solid[-1] = 1
+        parts.append(_masked(G.D2Q9, (nx, n, 1), solid.reshape(-1), q=0.3, bc=-1))
+    both = _masked(G.D2Q9, (nx, 2 * n, 1), np.concatenate([p.solid for p in parts]), q=0.3, bc=-1)
+    kw = dict(precision=L.LBM_FP64, bc=2, vibb_density=1)
+    with L.Lattice(both, domains=[dict(lo=n * k, n=n, nx=nx, tau=0.9, g=g) for k, g in enumerate(forces)], tau=0.9,
+                   **kw) as lat:
+        lat.init_equilibrium()
+        lat.step(7)
+        f = lat.distributions().reshape(9, 2, -1)
+    for k, g in enumerate(forces):
+        with L.Lattice(parts[k], tau=0.9, g=g, **kw) as lat:
+            lat.init_equilibrium()
+            lat.step(7)
+            assert np.array_equal(f[:, k], lat.distributions()), k
