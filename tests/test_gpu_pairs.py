@@ -153,3 +153,22 @@ def test_inlet_needs_a_second_column(L, prec):
         lat.set_geometry(np.zeros(32, np.uint8), np.zeros(0, G.LINK_DTYPE))
     assert ex.value.status == L.LBM_ERR_INVALID_ARG and "inlet" in str(ex.value)
     lat.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32s"])
+def test_states_beyond_l2_in_every_form(L, prec):
+    """More state than L2 keeps (rows end in partial groups, and the kernels
+    prefetch ahead, past the end of the storage in its last blocks): one node and
+    two per thread against the sequential walk, which does not prefetch, on a box
+    (FP32: the same bits), and both step forms with bodies."""
+    precision = L.LBM_FP64 if prec == "fp64" else L.LBM_FP32_SHIFTED
+    shape = (1501, 1003, 1)
+    box = G.build(0, shape, (1, 1, 1), [])
+    ref = _run(L, box, 3, None, dict(bulk_shape=6, fused=0), precision=precision, tau=0.7)[0]
+    for s in (1, 4, 2):
+        f = _run(L, box, 3, None, dict(bulk_shape=s, fused=0), precision=precision, tau=0.7)[0]
+        assert np.array_equal(f, ref) if prec == "fp32s" else np.abs(f - ref).max() <= 1e-14, s
+    geo = G.build(0, shape, (1, 1, 1), [G.ball((x, y, 0), 9.3) for x in (40.3, 900.7, 1480.2) for y in (30.1, 970.6)])
+    fa, fb = (_run(L, geo, 3, None, dict(bulk_shape=4, fused=k), precision=precision, tau=0.7)[0] for k in (0, 1))
+    h = np.abs(fa - np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None])[:, geo.solid == 0].max()
+    assert np.abs(fa - fb).max() <= (1e-13 if prec == "fp64" else 4 * 3 * float(np.finfo(np.float32).eps) * h)
