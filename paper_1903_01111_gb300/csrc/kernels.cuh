@@ -87,12 +87,12 @@ struct __align__(16) RunRec {
 
 // Run parameters of one domain of a batch (several independent flows
 // stacked along the last axis of one lattice, each with its own relaxation
-// time, body force and inlet profile).  A lattice of one domain reads Params.
+// time, body force and inlet profile; the profiles are in Layout's row_uin).  A
+// lattice of one domain reads Params.
 struct DomPar {
   double omega, fpre3;    // 1/tau, 3 (1 - 1/(2 tau))
   double g[3];
-  double inlet_umax, inlet_y0, inlet_y1;  // inlet rows relative to lo
-  int32_t lo, has_force;  // first row (y in 2-D, z in 3-D) of the domain
+  int32_t has_force;
   float omega_f, fpre3_f, g_f[3], hg_f[3], omega2_f;  // float copies, as in Params
   Folded kc;              // collision constants, as in Params
   FixedK kx;
@@ -133,7 +133,6 @@ struct Layout {
   const int32_t* row_in1;      // [ny*nz] storage index of the fluid node at x = 1 (open inlet rows), else -1
   const int32_t* row_out1;     // [ny*nz] ... at x = width - 2 (open outlet rows), else -1
   const DomPar* dom;           // [ndom] when ndom > 1, else null
-  const int32_t* row_dom;      // [ny*nz] domain of each row when ndom > 1
   int32_t ndom;
   const uint32_t* fluid;       // [nfluid] storage indices of the fluid nodes (FP64 lattices), else null
   int64_t nfluid;
@@ -1411,14 +1410,13 @@ __device__ __forceinline__ void cp_async_real(T* smem, const T* gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Resident blocks per SM of the fused kernel, per 256 threads: FP32 D2Q9 4
-// (64 registers: the link phase spills at the bulk kernel's 40), FP32
-// D3Q19 5 (48), FP64 2 (5 of 128 threads, 102 registers: 200^3 pack 1.10 ms per
-// step against 1.15 at 4 and 1.13 at 6).
+// Resident blocks per SM of the step kernels with links, per 256 threads: FP32
+// D2Q9 4 (64 registers: the link phase spills at the bulk kernel's 40), FP32
+// D3Q19 5 (48), FP64 2 (128; k_fused, 128^3 pack: 214 us per step, 217 and 225 with
+// room for 5 and 6 blocks of 128 threads).
 template <class L, class P, int BT>
 constexpr int fused_blocks_per_sm() {
   constexpr int base = !P::shifted ? 2 : (L::Q == 9 ? 4 : 5);
-  if (!P::shifted && BT == 128) return 4;
   return base * 256 / BT < 1 ? 1 : base * 256 / BT;
 }
 
@@ -1585,9 +1583,11 @@ constexpr int inline_free_groups() {
 // stage or barrier to read or wait for.  A warp with links evaluates them one
 // per lane (they are contiguous in the link list) while its pulls are in
 // flight, and hands the values to their nodes through its own part of shared
-// memory.  On a lattice with fewer groups with links than the chip holds
-// blocks (`spread`) a block takes one group and evaluates its links with all
-// its warps: a wall row has 96, three rounds of one warp.
+// memory.  Where there are few groups with links, up to two blocks an SM
+// (`spread`), a block takes one group and evaluates its links with all its warps: a
+// wall row has 96, three rounds of one warp.  Channels of 60 rows, us per step with
+// a block and with a warp on each group: 126 groups FP32 3.4 and 6.0, FP64 7.4 and
+// 11.5; 284 groups 5.0 and 6.3, 14.2 and 13.4; 564 groups 7.7 and 7.2, 29.9 and 27.5.
 constexpr int64_t kInlineSpread = 2 * 152;
 __host__ __device__ __forceinline__ bool inline_spread(int64_t nlinked) { return nlinked <= kInlineSpread; }
 

@@ -135,7 +135,6 @@ struct Params {
   double g[3];
   int has_force;        // g != 0
   int collision;        // 0 BGK, 1 MRT
-  double inlet_umax, inlet_y0, inlet_y1;
   int inlet, outlet;
   int vibb_local_rho;   // rho_d = rho_f when q > 1/2
   int periodic[3];

@@ -122,7 +122,7 @@ struct lbm_lattice_s {
   Layout lay{};
   // batch: domains along the last axis (empty: one domain run by cfg)
   std::vector<lbm_domain> domains;
-  DeviceBuf dom, row_dom;
+  DeviceBuf dom;
   int nbody = 1;  // force accumulators per slot
   lbm_tuning tune{-1, 256, 2, 1, 1};
   bool tuned = false;  // the caller set or tuned it
@@ -169,7 +169,7 @@ int64_t device_bytes(const lbm_handle h) {
   const DeviceBuf* all[] = {&h->f[0],     &h->f[1],     &h->mom[0],   &h->mom[1], &h->word,  &h->node_of, &h->tile, &h->row_uin, &h->groups,
                             &h->runs,     &h->row_first, &h->row_last, &h->row_in1, &h->row_out1, &h->recs,
                             &h->q,        &h->uw,       &h->lfirst, &h->lmask, &h->lrec,
-                            &h->lqd,      &h->luw,      &h->force,    &h->dom,    &h->row_dom, &h->fidx, &h->lqc, &h->lqf, &h->force_hist};
+                            &h->lqd,      &h->luw,      &h->force,    &h->dom, &h->fidx, &h->lqc, &h->lqf, &h->force_hist};
   int64_t s = 0;
   for (auto* b : all) s += (int64_t)b->bytes;
   return s;
@@ -224,7 +224,7 @@ void release_geometry(lbm_handle h) {
   DeviceBuf* all[] = {&h->f[0],     &h->f[1],      &h->mom[0],   &h->mom[1], &h->word,  &h->node_of, &h->tile, &h->row_uin, &h->groups,
                       &h->runs,     &h->row_first, &h->row_last, &h->row_in1, &h->row_out1, &h->recs,
                       &h->q,        &h->uw,        &h->lfirst, &h->lmask, &h->lrec,
-                      &h->lqd,      &h->luw,       &h->dom,      &h->row_dom, &h->fidx, &h->lqc, &h->lqf};
+                      &h->lqd,      &h->luw,       &h->dom, &h->fidx, &h->lqc, &h->lqf};
   for (auto* b : all) release(*b);
   h->lay = Layout{};
 }
@@ -471,16 +471,14 @@ lbm_status lbm_create_lattice(const lbm_config* cfg, lbm_handle* out) {
   fold_all(h);
   p.inlet = c.inlet ? 1 : 0;
   p.outlet = c.outlet ? 1 : 0;
-  p.inlet_umax = c.inlet_umax;
-  p.inlet_y0 = c.inlet_y0;
-  p.inlet_y1 = c.inlet_y1;
   p.vibb_local_rho = c.vibb_density == LBM_VIBB_RHO_LOCAL ? 1 : 0;
   for (int a = 0; a < 3; ++a) p.periodic[a] = c.periodic[a] ? 1 : 0;
   p.nbody = 1;
   h->tune.bulk_shape = h->ops.default_shape;
   if (h->rb == 8 && h->Q == 19) {
-    // the FP64 link rule's registers take the fused kernel's warps (200^3 pack
-    // 0.87 ms fused, 0.68 ms with 64-thread link blocks and the bulk pass)
+    // the FP64 link rule's registers take the fused kernel's warps, however few
+    // the links (160^3 nodes, split and fused: 0.0003 links a node 251 and 349 us
+    // per step, 0.25 277 and 404, 1.4 459 and 642)
     h->tune.fused = 0;
   }
   // small blocks spread few links over more SMs and free their registers
@@ -1195,13 +1193,8 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
         dp[k].g_f[a] = (float)dp[k].g[a];
         dp[k].hg_f[a] = (float)(0.5 * dp[k].g[a]);
       }
-      dp[k].inlet_umax = q.inlet_umax;
-      dp[k].inlet_y0 = q.inlet_y0;
-      dp[k].inlet_y1 = q.inlet_y1;
-      dp[k].lo = q.lo;
     }
     st = upload(h->dom, dp.data(), sizeof(DomPar) * ndom);
-    if (st == LBM_OK) st = upload(h->row_dom, rdom.data(), sizeof(int32_t) * rows);
   }
   if (st == LBM_OK && h->force.bytes != sizeof(double) * 6 * (size_t)nbody) {
     st = acquire(h->force, sizeof(double) * 6 * (size_t)nbody);
@@ -1244,7 +1237,6 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   h->lay.row_in1 = (const int32_t*)h->row_in1.p;
   h->lay.row_out1 = (const int32_t*)h->row_out1.p;
   h->lay.dom = ndom > 0 ? (const DomPar*)h->dom.p : nullptr;
-  h->lay.row_dom = ndom > 0 ? (const int32_t*)h->row_dom.p : nullptr;
   h->lay.ndom = std::max(ndom, 1);
   h->lay.fluid = nflist > 0 ? (const uint32_t*)h->fidx.p : nullptr;
   h->lay.nfluid = nflist;
@@ -1265,9 +1257,6 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   for (int a = 0; a < 3; ++a) p.g[a] = a < D ? d0.g[a] : 0.0;
   p.has_force = (p.g[0] != 0.0 || p.g[1] != 0.0 || p.g[2] != 0.0);
   fold_all(h);
-  p.inlet_umax = d0.inlet_umax;
-  p.inlet_y0 = d0.inlet_y0;
-  p.inlet_y1 = d0.inlet_y1;
   h->nbody = nbody;
   h->p.nbody = nbody;
   h->sidx.swap(sidx);
@@ -1283,7 +1272,9 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   // D2Q9 FP32 lattices of which more than 1 in 12 groups has links (cylinders
   // all over, 18 % of the channel batch's) run the link kernel, whose warps are
   // full, and the bulk pass: 188 against 218 us per step there, and 11.0 against
-  // 8.7 us on a 2000 x 400 channel with one cylinder (1 %).
+  // 8.7 us on a 2000 x 400 channel with one cylinder (1 %).  2048 x 1024 nodes with
+  // cylinders of radius 12, split and fused: 2.6 % of the groups 31.0 and 29.4 us,
+  // 10 % 31.1 and 31.4, 46 % 33.7 and 40.4.
   if (!h->tuned && Q == 9 && h->rb == 4) h->tune.fused = 12 * nlinked > ngroups && !inline_spread(nlinked) ? 0 : 1;
   h->has_geometry = true;
   return LBM_OK;
