@@ -1028,34 +1028,6 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
         if (!(word[k] & (W_GHOST | W_OPEN))) flist[j++] = (uint32_t)k;
     }
   }
-  // rest part of the momentum exchange per body, left out by the kernels:
-  // sum over the body's links of 2 w_i' rho0 e_i', from the exact count of
-  // its links per direction (counted in parallel, summed in a fixed order)
-  std::vector<double> rest(3 * (size_t)nbody, 0.0);
-  if (n_links > 0 && max_body >= 0) {
-    const size_t nc = (size_t)(max_body + 1) * Q;
-    std::vector<int64_t> cnt(nc, 0);
-#pragma omp parallel
-    {
-      std::vector<int64_t> mine(nc, 0);
-#pragma omp for schedule(static) nowait
-      for (int64_t k = 0; k < n_links; ++k)
-        if (links[k].body >= 0) ++mine[(size_t)links[k].body * Q + links[k].dir];
-#pragma omp critical
-      for (size_t j = 0; j < nc; ++j) cnt[j] += mine[j];
-    }
-    for (int b = 0; b <= max_body; ++b)
-      for (int d = 1; d < Q; ++d) {
-        const int64_t n = cnt[(size_t)b * Q + d];
-        if (n == 0) continue;
-        const double w = Q == 9 ? D2Q9::w(d) : D3Q19::w(d);
-        // (FP64: n times what the kernels take off a link)
-        const double t = h->rb == 8 ? (double)n * (2.0 * (w * c.rho0)) : (double)n * 2.0 * w * c.rho0;
-        rest[3 * b + 0] += t * cx_of(h, d);
-        rest[3 * b + 1] += t * cy_of(h, d);
-        rest[3 * b + 2] += t * cz_of(h, d);
-      }
-  }
   // link records: the split form's in `order`, the fused kernel's in
   // (node, dir) order (`ond`); with one body the two orders are the same and
   // one pass fills both
@@ -1080,22 +1052,46 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
     if (moving)
       for (int a = 0; a < D; ++a) uws[a * n_links + j] = L.uw[a];
   };
-#pragma omp parallel for schedule(static)
-  for (int64_t j = 0; j < n_links; ++j) {
-    const int64_t k = ond[j];
-    const lbm_link& L = links[k];
-    const uint32_t kf = (uint32_t)sidx[L.node], kff = (uint32_t)sidx[lk_ff[k]];
+  // (and the count of each body's links per direction)
+  const size_t nc = (size_t)(max_body + 1) * Q;
+  std::vector<int64_t> link_count(nc, 0);
+#pragma omp parallel
+  {
+    std::vector<int64_t> mine(nc, 0);
+#pragma omp for schedule(static) nowait
+    for (int64_t j = 0; j < n_links; ++j) {
+      const int64_t k = ond[j];
+      const lbm_link& L = links[k];
+      if (L.body >= 0) ++mine[(size_t)L.body * Q + L.dir];
+      const uint32_t kf = (uint32_t)sidx[L.node], kff = (uint32_t)sidx[lk_ff[k]];
 #pragma omp atomic update
-    fmask[kf] |= 1u << L.dir;
-    const float q32 = (float)L.q;
-    uint32_t qbits;
-    memcpy(&qbits, &q32, 4);
-    frec[j] = FusedRec{kf, kff, (uint32_t)L.dir | ((uint32_t)lk_rule[k] << 5) | ((uint32_t)(L.body + 1) << 8), qbits};
-    if (h->rb == 8) fq[j] = L.q;
-    if (moving)
-      for (int a = 0; a < D; ++a) fuw[a * n_links + j] = L.uw[a];
-    if (same_order) split_rec(j, k, kf, kff);
+      fmask[kf] |= 1u << L.dir;
+      const float q32 = (float)L.q;
+      uint32_t qbits;
+      memcpy(&qbits, &q32, 4);
+      frec[j] = FusedRec{kf, kff, (uint32_t)L.dir | ((uint32_t)lk_rule[k] << 5) | ((uint32_t)(L.body + 1) << 8), qbits};
+      if (h->rb == 8) fq[j] = L.q;
+      if (moving)
+        for (int a = 0; a < D; ++a) fuw[a * n_links + j] = L.uw[a];
+      if (same_order) split_rec(j, k, kf, kff);
+    }
+#pragma omp critical
+    for (size_t t = 0; t < nc; ++t) link_count[t] += mine[t];
   }
+  // rest part of the momentum exchange per body, left out by the kernels:
+  // sum over the body's links of 2 w_i' rho0 e_i', summed in a fixed order
+  std::vector<double> rest(3 * (size_t)nbody, 0.0);
+  for (int b = 0; b <= max_body; ++b)
+    for (int d = 1; d < Q; ++d) {
+      const int64_t n = link_count[(size_t)b * Q + d];
+      if (n == 0) continue;
+      const double w = Q == 9 ? D2Q9::w(d) : D3Q19::w(d);
+      // (FP64: n times what the kernels take off a link)
+      const double t = h->rb == 8 ? (double)n * (2.0 * (w * c.rho0)) : (double)n * 2.0 * w * c.rho0;
+      rest[3 * b + 0] += t * cx_of(h, d);
+      rest[3 * b + 1] += t * cy_of(h, d);
+      rest[3 * b + 2] += t * cz_of(h, d);
+    }
   if (!same_order) {
 #pragma omp parallel for schedule(static)
     for (int64_t j = 0; j < n_links; ++j) {
@@ -1165,10 +1161,10 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   if (st == LBM_OK) st = upload(h->lqd, fq.data(), sizeof(double) * fq.size());
   if (st == LBM_OK && nflist > 0) st = upload(h->fidx, flist.data(), sizeof(uint32_t) * nflist);
   if (st == LBM_OK && h->rb == 8 && n_links > 0) {
-    st = upload(h->lqc, vibb_weights(n_links, [&](int64_t j) { return links[order[j]].q; }).data(),
+    st = upload(h->lqc, vibb_weights(n_links, [&](int64_t j) { return qs[j]; }).data(),
                 sizeof(int64_t) * 3 * n_links);
     if (st == LBM_OK && !same_order && h->tune.fused)
-      st = upload(h->lqf, vibb_weights(n_links, [&](int64_t j) { return links[ond[j]].q; }).data(),
+      st = upload(h->lqf, vibb_weights(n_links, [&](int64_t j) { return fq[j]; }).data(),
                   sizeof(int64_t) * 3 * n_links);
   }
   if (st == LBM_OK && ndom > 0) {
