@@ -390,8 +390,9 @@ lbm_status lbm_force_noalloc(const lbm_config* cfg, const double* f_post, const 
                              const lbm_link* links, int64_t n_links, int32_t body, double* F);
 
 /* Launch shapes (lbm_tuning).  lbm_set_tuning validates and applies them
- * (from the next lbm_step); lbm_get_tuning reads the current ones.
- * Errors: INVALID_ARG. */
+ * (from the next lbm_step); lbm_get_tuning reads the current ones.  FP64
+ * lattices with several bodies hold 24 B a link more while `fused` is 1.
+ * Errors: INVALID_ARG, OOM, CUDA (the tuning stays as it was). */
 lbm_status lbm_set_tuning(lbm_handle h, const lbm_tuning* t);
 lbm_status lbm_get_tuning(lbm_handle h, lbm_tuning* t);
 

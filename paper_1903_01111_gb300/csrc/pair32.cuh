@@ -100,7 +100,8 @@ __device__ __forceinline__ void bgk_d2q9(V (&f)[9], const Bgk32<V>& c, bool forc
   r = N::add(f[0], N::add(N::add(s13, s24), N::add(s57, s68)));
   const V jx = N::add(d13, N::sub(d57, d68)), jy = N::add(d24, N::add(d57, d68));
   const V rho = N::add(c.rho0, r);
-  // 1/rho: the hardware's reciprocal and a Newton-Raphson step
+  // 1/rho: the hardware's reciprocal and a Newton-Raphson step with one rounding
+  // at its end, the correctly rounded quotient for every float from 2^-30 to 2^31
   V inv = N::rcp_seed(rho);
   inv = N::fma(inv, N::fma(N::mul(rho, N::all(-1.f)), inv, N::all(1.f)), inv);
   ux = N::mul(force ? N::add(jx, c.hx) : jx, inv);
