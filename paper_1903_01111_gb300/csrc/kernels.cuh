@@ -197,11 +197,18 @@ __device__ __forceinline__ void clear_force(double* force_next, int nbody) {
     for (int t = threadIdx.x; t < 3 * nbody; t += BT) force_next[t] = 0.0;
 }
 
-// Programmatic dependent launch: a step kernel lets its successor start as soon
-// as all its own blocks have, and the successor reads what no kernel writes
-// (node words, runs, link records) before it waits for the predecessor's
-// results.  On lattices that take microseconds a step the launch and those
-// loads are a third of it.
+// Programmatic dependent launch: a step kernel lets its successor start early,
+// and the successor reads what no kernel writes (node words, runs, link records)
+// before it waits for the predecessor's results.  On lattices that take
+// microseconds a step the launch and those loads are a third of it.
+//
+// Bulk and fused kernels let it start once they have waited themselves, so that
+// one successor at most is resident beside a kernel.  At the start of the kernel
+// instead, the next five or six steps of a lattice of some 200 blocks take up
+// their places at once, each where its predecessors left room, which piles a
+// step's blocks onto a few SMs: 32^3 nodes FP32 4.5 us per step, 2.8 so; FP64 28^3
+// 7.5 and 4.2.  k_inline and the link kernels, whose chain before the wait is
+// longer, do it first (FP32 channel 600 x 500 5.2 us per step, 5.7 the other way).
 //
 // A kernel started so is resident while its predecessor still writes the
 // populations, the moment cache and the multipliers it will read.  Such memory
@@ -707,8 +714,9 @@ constexpr int bulk_blocks_per_sm() {
 
 // Pull, collision and store of NPT nodes k of a thread, all their pulls issued
 // before the first collision.  MULTI: the lattice holds several domains; each
-// node's collision reads its run's domain parameters.
-template <class L, class P, bool MULTI, int NPT, bool SOON>
+// node's collision reads its run's domain parameters.  ALONE: in a bulk kernel,
+// not in k_inline (which has let the next start, and does without SOON).
+template <class L, class P, bool MULTI, int NPT, bool ALONE>
 __device__ __forceinline__ void bulk_nodes(const uint32_t (&k)[NPT], const bool (&live)[NPT],
                                            const typename P::T* fin, typename P::T* __restrict__ fout,
                                            const Layout& lay, Mom4<typename P::T>* __restrict__ mom, const Params& p) {
@@ -724,9 +732,11 @@ __device__ __forceinline__ void bulk_nodes(const uint32_t (&k)[NPT], const bool 
     if (live[0] && !(w[0] & (W_GHOST | W_OPEN))) run = lay.runs[w[0] & W_RUN];
     dom[0] = run.dom;
     wait_for_previous();
+    if (ALONE) let_next_start();
     if (live[0] && !(w[0] & (W_GHOST | W_OPEN))) pull_node<L>(fin, S, k[0], run, lay, p, f[0]);
   } else {
     wait_for_previous();
+    if (ALONE) let_next_start();
 #pragma unroll
     for (int j = 0; j < NPT; ++j) {
       dom[j] = 0;
@@ -746,7 +756,7 @@ __device__ __forceinline__ void bulk_nodes(const uint32_t (&k)[NPT], const bool 
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) f[j][i] = P::shifted ? (T)0 : (T)L::w(i);
     }
-    collide_node<L, P, MULTI, SOON>(f[j], p, lay, dom[j], fout, S, k[j], mom, (w[j] & W_CACHE) != 0, fl, [&](T(&g)[L::Q]) {
+    collide_node<L, P, MULTI, ALONE>(f[j], p, lay, dom[j], fout, S, k[j], mom, (w[j] & W_CACHE) != 0, fl, [&](T(&g)[L::Q]) {
       pull_node<L>(fin, S, k[j], lay.runs[w[j] & W_RUN], lay, p, g);
     });
     if (L::D == 2 && fl && (p.inlet | p.outlet)) open_ends<L, P>(fout, mom, S, k[j], lay.runs[w[j] & W_RUN], lay, p);
@@ -843,12 +853,13 @@ __device__ __forceinline__ void pair_finish(uint32_t k, bool live, const PairNod
   }
 }
 
-template <bool MULTI>
+template <bool MULTI, bool ALONE>
 __device__ __forceinline__ void bulk_pair(uint32_t k, bool live, const float* fin,
                                           float* __restrict__ fout, const Layout& lay, Mom4<float>* __restrict__ mom,
                                           const Params& p) {
   const PairNodes n = pair_nodes(k, live, lay);
   wait_for_previous();
+  if (ALONE) let_next_start();
   F2 f[9];
   pair_pull(k, n, fin, lay, p, f);
   pair_finish<MULTI>(k, live, n, f, fout, lay, mom, p);
@@ -860,12 +871,11 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, NPT>())) k_b
                                                                        typename P::T* __restrict__ fout, Layout lay,
                                                                        Mom4<typename P::T>* __restrict__ mom,
                                                                        double* force_next, Params p) {
-  let_next_start();
   const uint32_t t = blockIdx.x * BT + threadIdx.x;
   if constexpr (NPT == 2 && P::shifted && L::Q == 9) {
     if (p.collision == 0) {
       prefetch_ahead<L::Q>(fin, lay, 2ull * blockIdx.x * BT, 2 * BT, threadIdx.x, BT);
-      bulk_pair<MULTI>(2 * t, 2ull * t < (uint64_t)lay.S, fin, fout, lay, mom, p);
+      bulk_pair<MULTI, true>(2 * t, 2ull * t < (uint64_t)lay.S, fin, fout, lay, mom, p);
       clear_force<BT>(force_next, p.nbody);
       return;
     }
@@ -896,7 +906,6 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, 1>())) k_bul
     const typename P::T* fin, typename P::T* __restrict__ fout, Layout lay,
     Mom4<typename P::T>* __restrict__ mom, double* force_next, Params p) {
   using T = typename P::T;
-  let_next_start();
   const int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
   const size_t S = (size_t)lay.S;
   const bool live = t < lay.nfluid;
@@ -905,6 +914,7 @@ __global__ void __launch_bounds__(BT, (bulk_blocks_per_sm<L, P, BT, 1>())) k_bul
   RunRec run{};
   if (live) run = lay.runs[w & W_RUN];
   wait_for_previous();
+  let_next_start();
   clear_force<BT>(force_next, p.nbody);
   if (!live) return;
   // (the block's nodes lie at its share of the storage)
@@ -950,7 +960,6 @@ __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_
     const typename P::T* fin, typename P::T* __restrict__ fout, Layout lay,
     Mom4<typename P::T>* __restrict__ mom, double* force_next, Params p) {
   using T = typename P::T;
-  let_next_start();
   const size_t S = (size_t)lay.S;
   const uint32_t G = gridDim.x * BT;
   uint32_t k = blockIdx.x * BT + threadIdx.x;
@@ -959,6 +968,7 @@ __global__ void __launch_bounds__(BT, (bulk_seq_blocks_per_sm<P, BT>())) k_bulk_
   if (!(w & (W_GHOST | W_OPEN))) run = load_run_lite<L, MULTI>(lay.runs, w & W_RUN);
   uint32_t w2 = ((uint64_t)k + G < S) ? __ldg(lay.word + k + G) : W_GHOST;
   wait_for_previous();
+  let_next_start();
   clear_force<BT>(force_next, p.nbody);
 #pragma unroll 1
   for (int it = 0; it < SEQ && (uint64_t)k < S; ++it, k += G) {
@@ -1448,10 +1458,10 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_fused
   __shared__ T stage[NW][L::Q][32];
   __shared__ DirTable<T, L::Q> tab;
   __shared__ double red[3][NW];
-  let_next_start();
   fill_dir_table<L>(tab);
   // (waits before the link records: held back behind them it cost 2 %)
   wait_for_previous();
+  let_next_start();
   clear_force<BT>(force_next, p.nbody);
   __syncthreads();  // the direction table (every thread arrives here at once)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1613,7 +1623,7 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
         const bool some = mine < lay.ngroups;
         const uint32_t k = (some ? 32u * __ldg(lay.groups + mine) : 0u) + 2u * (lane & 15);
         prefetch_ahead<L::Q>(fin, lay, k & ~31u, 32, lane & 15, 16);
-        bulk_pair<MULTI>(k, some, fin, fout, lay, mom_out, p);
+        bulk_pair<MULTI, false>(k, some, fin, fout, lay, mom_out, p);
         clear_force<BT>(force_next, p.nbody);
         return;
       }
