@@ -16,9 +16,9 @@
 // fluid node; ghost slots are filled by the link kernel before the bulk
 // kernel pulls them.
 //
-// Every state of a lattice with open columns (D2Q9) holds them filled: by
-// k_open after the initialisation, by the threads of the nodes beside them in
-// every step (open_ends).
+// Every state of a lattice with open columns (D2Q9) holds them filled, by the
+// threads of the nodes beside them in the initialisation and in every step
+// (open_ends), and by k_open after the caller sets the populations.
 //
 // Step t -> t+1, on one stream, in one of two forms.  Fused: D3Q19 k_fused
 // stages each block's pulls in shared memory, evaluates the block's link rules
@@ -629,7 +629,7 @@ __device__ __forceinline__ void fill_outlet(typename P::T* f, size_t S, uint32_t
 // The open columns of a state (f, mom), one thread per row and side (D2Q9):
 // the open node is the first (inlet) or last (outlet) stored node of its row.
 // Every state of a lattice with open columns holds them filled: by this kernel
-// after the initialisation, by the step kernels themselves (open_ends).
+// after the caller sets the populations, else by open_ends.
 template <class L, class P>
 __global__ void k_open(typename P::T* __restrict__ f, const Mom4<typename P::T>* __restrict__ mom, Layout lay,
                        Params p) {
@@ -1775,8 +1775,8 @@ __global__ void __launch_bounds__(BT, (fused_blocks_per_sm<L, P, BT>())) k_inlin
 __device__ __forceinline__ bool is_fluid(uint32_t w) { return (w & (W_GHOST | W_OPEN)) == 0; }
 
 // f(x,0) = feq(rho_in, u_in) followed by the collision at t = 0 (fluid
-// nodes); zero elsewhere.  rho_in (N) and u_in (N x 3, interleaved), dense
-// indices, may be null for rho0 and rest.
+// nodes), and the open columns filled from it; zero elsewhere.  rho_in (N) and
+// u_in (N x 3, interleaved), dense indices, may be null for rho0 and rest.
 template <class L, class P>
 __global__ void k_init(typename P::T* __restrict__ f, Mom4<typename P::T>* __restrict__ mom, Layout lay,
                        const double* __restrict__ rho_in, const double* __restrict__ u_in, Params p) {
@@ -1786,6 +1786,7 @@ __global__ void k_init(typename P::T* __restrict__ f, Mom4<typename P::T>* __res
   const size_t S = (size_t)lay.S;
   const uint32_t w = lay.word[k];
   if (!is_fluid(w)) {
+    if (w & W_OPEN) return;  // (the thread of the fluid node beside it writes it)
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) f[(size_t)i * S + k] = (T)0;
     return;
@@ -1807,6 +1808,7 @@ __global__ void k_init(typename P::T* __restrict__ f, Mom4<typename P::T>* __res
   // in a batch
   const Folded* kc = lay.ndom > 1 ? &lay.dom[lay.runs[w & W_RUN].dom].kc : &p.kc;
   collide_store<L, P>(fl, p, rx, *kc, f, S, (uint32_t)k, mom, (w & W_CACHE) != 0);
+  open_ends<L, P>(f, mom, S, (uint32_t)k, lay.runs[w & W_RUN], lay, p);
 }
 
 // A float as a double by moving its bits: a hardware conversion takes the FP64

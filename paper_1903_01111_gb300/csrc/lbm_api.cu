@@ -1296,7 +1296,6 @@ lbm_status lbm_init_equilibrium(lbm_handle h, const double* rho, const double* u
   if (e == cudaSuccess && h->mom[0].bytes) e = cudaMemsetAsync(h->mom[0].p, 0, h->mom[0].bytes, h->stream);
   if (e == cudaSuccess) {
     h->ops.init(h->f[0].p, h->mom[0].p, h->lay, drho, du, h->p, h->stream);
-    if (h->p.inlet || h->p.outlet) h->ops.open(h->f[0].p, h->mom[0].p, h->lay, h->p, h->stream);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(h->force.p, 0, h->force.bytes, h->stream);
