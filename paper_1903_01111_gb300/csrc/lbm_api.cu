@@ -6,8 +6,8 @@
 // the layout tables, the link records (in the link kernel's order and in the
 // fused step kernel's (node, direction) order), the domain table of a batch
 // and two FP64 force slots.  lbm_step replays
-// captured CUDA graphs of graph_steps steps (tuned above two) and launches the
-// rest step by step; with profiling on it launches kernel
+// captured CUDA graphs of graph_steps steps (tuned above two, or a small lattice)
+// and launches the rest step by step; with profiling on it launches kernel
 // by kernel between CUDA events.  lbm_autotune picks the launch shapes.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -1310,6 +1310,16 @@ lbm_status lbm_init_equilibrium(lbm_handle h, const double* rho, const double* u
   return LBM_OK;
 }
 
+// A step of a small lattice takes the device about as long as its launch takes
+// the host (2 us), so that a program that steps several of them, each on its own
+// stream, waits for launches: runs of steps on lattices of at most kSmallNodes
+// stored nodes go in graphs of kSmallGraph, unless the caller set the tuning.
+// 32 x 24 nodes FP32, us per step of 200: three lattices in turn 1.87 one by one,
+// 0.97 in graphs (1.74 in graphs of two), one lattice 2.96 and 2.59; 300 x 200 FP64
+// 2.73 and 2.61, 6.4 and 6.1; 600 x 400 FP64 11.5 and 11.5: nothing left to gain.
+constexpr int kSmallGraph = 16;
+constexpr int64_t kSmallNodes = 1 << 17;
+
 lbm_status lbm_step(lbm_handle h, int64_t n) {
   g_msg[0] = 0;
   NvtxRange range("lbm_step");
@@ -1339,7 +1349,13 @@ lbm_status lbm_step(lbm_handle h, int64_t n) {
     ++h->step;
     --left;
   }
-  const int G = h->tune.graph_steps;
+  int G = h->tune.graph_steps;
+  if (!h->tuned && left >= 2 * kSmallGraph && h->lay.S <= kSmallNodes) {
+    // (not into a caller's capture, which takes launches only)
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    CUDA_TRY(cudaStreamIsCapturing(h->stream, &capturing));
+    if (capturing == cudaStreamCaptureStatusNone) G = kSmallGraph;
+  }
   if (G > 2 && left >= G) {
     if (!h->graphG[h->cur]) {
       lbm_status st = build_graph(h, h->cur, G, &h->graphG[h->cur]);

@@ -201,3 +201,68 @@ def test_small_lattices_do_not_crowd_themselves_out(L, prec):
         assert us(32) <= 1.1 * us(40)
     else:
         assert us(28) <= 1.45 * us(24)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32s"])
+def test_graphs_of_a_small_lattice_are_its_steps(L, prec):
+    """Runs of steps on a small lattice of untouched tuning (graphs of 16) against
+    steps launched one by one: the same bits and forces, from odd steps too, and
+    when the caller captures them."""
+    import torch
+
+    precision = L.LBM_FP64 if prec == "fp64" else L.LBM_FP32_SHIFTED
+    geo = G.cylinder_channel(nx=121, ny_fluid=30, center=(30.37, 15.61), radius=4.3)
+    kw = dict(precision=precision, tau=0.7, inlet_umax=0.05, inlet_y0=0.5, inlet_y1=30.5)
+    s = torch.cuda.Stream()
+    with L.Lattice(geo, **kw) as a, L.Lattice(geo, **kw) as b, L.Lattice(geo, stream=s.cuda_stream, **kw) as c:
+        t = b.tuning()
+        b.set_tuning(bulk_shape=t.bulk_shape, link_threads=t.link_threads, link_seq=t.link_seq, fused=t.fused, graph_steps=2)
+        for lat in (a, b, c):
+            lat.init_equilibrium(*_start(geo, 3))
+        for n in (1, 100, 33, 2, 31, 40):
+            a.step(n)
+            b.step(n)
+            c.step(n)
+            assert np.array_equal(a.distributions(), b.distributions()), n
+            scale = np.abs(b.forces()).max()
+            assert np.abs(a.forces() - b.forces()).max() <= 1e-12 * scale + (0 if prec == "fp64" else 1e-5 * scale)
+        assert a.info().step == b.info().step == 207
+        a.step(1)
+        b.step(1)
+        c.step(1)
+        c.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            c.step(40)
+        with torch.cuda.stream(s):
+            g.replay()
+        c.synchronize()
+        b.step(40)
+        assert np.array_equal(c.distributions(), b.distributions())
+
+
+def test_several_small_lattices_are_not_bound_by_launches(L):
+    """Three 32 x 24 lattices stepped in turn by one host thread: 1.9 us per step
+    when each step was a launch, 1.0 in graphs of 16; one lattice 2.6."""
+    geo = G.channel(0, 32, 24, q_lo=0.3, q_hi=0.3)
+    lats = [L.Lattice(geo, precision=L.LBM_FP32_SHIFTED, tau=0.8, bc=2, g=(1e-6, 0, 0)) for _ in range(3)]
+    for lat in lats:
+        lat.init_equilibrium()
+
+    def us(which):
+        best = np.inf
+        for _ in range(6):
+            for lat in lats:
+                lat.synchronize()
+            t = time.perf_counter()
+            for k in range(30):
+                which[k % len(which)].step(160)
+            for lat in lats:
+                lat.synchronize()
+            best = min(best, (time.perf_counter() - t) / 30 / 160 * 1e6)
+        return best
+
+    one, three = us(lats[:1]), us(lats)
+    for lat in lats:
+        lat.close()
+    assert three <= 0.55 * one
