@@ -177,8 +177,9 @@ typedef struct {
  *  graph_steps    time steps per CUDA graph replayed by lbm_step (even,
  *                 2..64); at 2 (the default) steps are launched one by one,
  *                 each letting the next start early, without a graph (until
- *                 the tuning is set, lattices of at most 131,072 stored nodes
- *                 replay graphs of 16 in calls of 32 steps and more).
+ *                 the tuning is set, lattices whose populations take at most
+ *                 24 MB replay graphs of 16, 8 and 4 in calls of 32 steps and
+ *                 more, and in shorter ones after their first 32 steps).
  *  link_seq       links per thread of the link kernel, 1 or 4 (a block
  *                 takes link_seq rounds of consecutive links, loading the
  *                 next round's record while it evaluates the current one);

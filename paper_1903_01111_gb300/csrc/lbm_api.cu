@@ -107,6 +107,23 @@ struct DeviceBuf {
   size_t bytes = 0;
 };
 
+// A step of a small lattice takes the device about as long as its launch takes
+// the host (2 us), so that a program that steps several of them, each on its own
+// stream, or a few steps at a time between read-outs, waits for launches.  Steps
+// of a lattice whose state is at most kSmallBytes (about 7 us a step; beyond it a
+// few steps take the device longer than the host with their read-out) therefore go
+// in graphs of 16, 8 and 4 (1 us of the host each), unless the caller set the
+// tuning: runs of 32 and more at once, shorter ones when a lattice has run
+// kSmallAfter steps, so that its first calls build nothing they do not use again.
+// 32 x 24 nodes FP32, us per step of 200: three lattices in turn 1.87 one by one,
+// 0.97 in graphs (1.74 in graphs of two), one lattice 2.96 and 2.59; 300 x 200 FP64
+// 2.73 and 2.61, 6.4 and 6.1; 600 x 400 FP32 one lattice 4.3 and 3.8.  Three 434 x
+// 166 FP32 boxes in turn, 8 steps and a read-out each: 57 us one by one, 35 in a
+// graph (45 in graphs of two).
+constexpr int kSmallGraphs = 3;
+constexpr int kSmallGraph[kSmallGraphs] = {16, 8, 4};
+constexpr int64_t kSmallBytes = 24 << 20, kSmallAfter = 32;
+
 struct lbm_lattice_s {
   lbm_config cfg{};
   KernelOps ops{};
@@ -154,6 +171,8 @@ struct lbm_lattice_s {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   cudaGraphExec_t graphG[2] = {nullptr, nullptr};  // tune.graph_steps steps
+  cudaGraphExec_t small_graph[2][kSmallGraphs] = {};  // kSmallGraph[.] steps (small lattices)
+  int64_t steps_run = 0;                              // since the geometry was set
   // profiling
   bool profiling = false;
   std::vector<cudaEvent_t> ev;
@@ -217,6 +236,10 @@ void drop_graphs(lbm_handle h) {
   for (int k = 0; k < 2; ++k) {
     if (h->graphG[k]) cudaGraphExecDestroy(h->graphG[k]);
     h->graphG[k] = nullptr;
+    for (cudaGraphExec_t& g : h->small_graph[k]) {
+      if (g) cudaGraphExecDestroy(g);
+      g = nullptr;
+    }
   }
 }
 
@@ -1272,6 +1295,7 @@ lbm_status lbm_set_geometry(lbm_handle h, const uint8_t* solid, const lbm_link* 
   // cylinders of radius 12, split and fused: 2.6 % of the groups 31.0 and 29.4 us,
   // 10 % 31.1 and 31.4, 46 % 33.7 and 40.4.
   if (!h->tuned && Q == 9 && h->rb == 4) h->tune.fused = 12 * nlinked > ngroups && !inline_spread(nlinked) ? 0 : 1;
+  h->steps_run = 0;
   h->has_geometry = true;
   return LBM_OK;
 }
@@ -1310,16 +1334,6 @@ lbm_status lbm_init_equilibrium(lbm_handle h, const double* rho, const double* u
   return LBM_OK;
 }
 
-// A step of a small lattice takes the device about as long as its launch takes
-// the host (2 us), so that a program that steps several of them, each on its own
-// stream, waits for launches: runs of steps on lattices of at most kSmallNodes
-// stored nodes go in graphs of kSmallGraph, unless the caller set the tuning.
-// 32 x 24 nodes FP32, us per step of 200: three lattices in turn 1.87 one by one,
-// 0.97 in graphs (1.74 in graphs of two), one lattice 2.96 and 2.59; 300 x 200 FP64
-// 2.73 and 2.61, 6.4 and 6.1; 600 x 400 FP64 11.5 and 11.5: nothing left to gain.
-constexpr int kSmallGraph = 16;
-constexpr int64_t kSmallNodes = 1 << 17;
-
 lbm_status lbm_step(lbm_handle h, int64_t n) {
   g_msg[0] = 0;
   NvtxRange range("lbm_step");
@@ -1349,13 +1363,29 @@ lbm_status lbm_step(lbm_handle h, int64_t n) {
     ++h->step;
     --left;
   }
-  int G = h->tune.graph_steps;
-  if (!h->tuned && left >= 2 * kSmallGraph && h->lay.S <= kSmallNodes) {
+  if (!h->tuned && (int64_t)h->Q * h->lay.S * (int64_t)h->rb <= kSmallBytes) {
     // (not into a caller's capture, which takes launches only)
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    CUDA_TRY(cudaStreamIsCapturing(h->stream, &capturing));
-    if (capturing == cudaStreamCaptureStatusNone) G = kSmallGraph;
+    if (left >= kSmallGraph[kSmallGraphs - 1]) CUDA_TRY(cudaStreamIsCapturing(h->stream, &capturing));
+    for (int g = 0; g < kSmallGraphs && capturing == cudaStreamCaptureStatusNone; ++g) {
+      const int m = kSmallGraph[g];
+      if (left < m || (h->steps_run < kSmallAfter && (g > 0 || left < 2 * m))) continue;
+      cudaGraphExec_t& x = h->small_graph[h->cur][g];
+      if (!x && build_graph(h, h->cur, m, &x) != LBM_OK) {
+        // (no room for it, say: the steps run one by one)
+        cudaGetLastError();
+        g_msg[0] = 0;
+        x = nullptr;
+        break;
+      }
+      for (; left >= m; left -= m) {
+        CUDA_TRY(cudaGraphLaunch(x, h->stream));
+        h->step += m;
+      }
+    }
+    h->steps_run += n;
   }
+  const int G = h->tune.graph_steps;
   if (G > 2 && left >= G) {
     if (!h->graphG[h->cur]) {
       lbm_status st = build_graph(h, h->cur, G, &h->graphG[h->cur]);

@@ -205,8 +205,8 @@ def test_small_lattices_do_not_crowd_themselves_out(L, prec):
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32s"])
 def test_graphs_of_a_small_lattice_are_its_steps(L, prec):
-    """Runs of steps on a small lattice of untouched tuning (graphs of 16) against
-    steps launched one by one: the same bits and forces, from odd steps too, and
+    """Runs of steps on a small lattice of untouched tuning (graphs of 16, 8 and 4)
+    against steps launched one by one: the same bits and forces, from odd steps too, and
     when the caller captures them."""
     import torch
 
@@ -219,7 +219,7 @@ def test_graphs_of_a_small_lattice_are_its_steps(L, prec):
         b.set_tuning(bulk_shape=t.bulk_shape, link_threads=t.link_threads, link_seq=t.link_seq, fused=t.fused, graph_steps=2)
         for lat in (a, b, c):
             lat.init_equilibrium(*_start(geo, 3))
-        for n in (1, 100, 33, 2, 31, 40):
+        for n in (1, 100, 33, 2, 31, 12, 5, 7, 16):
             a.step(n)
             b.step(n)
             c.step(n)
